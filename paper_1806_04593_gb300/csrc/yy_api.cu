@@ -62,8 +62,10 @@ static void free_all(yy_grid *g) {
     if (p) cudaFree(p);
   float *fbufs[] = {g->rot32, g->ban32, g->ysyn32, g->ysyn_t32, g->ysyn_p32, g->rho32, g->Q32,
                     g->sep_az32, g->sep_w32, g->sep_tb32};
-  double *sbufs[] = {g->sep_az, g->sep_F, g->sep_F0, g->sep_P, g->sep_dP, g->sep_Qs, g->sep_tr};
-  float *sfbufs[] = {g->sep_P32, g->sep_dP32, g->sep_Qs32, g->sep_tr32};
+  double *sbufs[] = {g->sep_az, g->sep_F, g->sep_F0, g->sep_P, g->sep_dP, g->sep_Qs, g->sep_tr, g->sep_trf,
+                     g->sep_isin};
+  float *sfbufs[] = {g->sep_P32, g->sep_dP32, g->sep_Qs32, g->sep_tr32, g->sep_T32[0],
+                     g->sep_T32[1], g->sep_T32[2], g->sep_G32};
   for (float *p : sfbufs)
     if (p) cudaFree(p);
   for (double *p : sbufs)
@@ -130,6 +132,7 @@ static yy_status create_grid(const double *r_edges, int n_r, int n_theta, int n_
   if (!g) return YY_ERR_OOM;
   memset((void *)g, 0, sizeof(yy_grid));
   cudaGetDevice(&g->device);
+  cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, g->device);
   g->n_patch = polar ? 1 : 2;
   g->n_r = n_r;
   g->n_theta = n_theta;
@@ -280,7 +283,8 @@ yy_status yy_grid_prepare(yy_grid *g, yy_precision prec) {
     case YY_FP64: return YY_OK;
     case YY_FP32: {
       if (g->ban32) return YY_OK;
-      cudaError_t e = convert_tables_f32(g);
+      cudaError_t e = synthesis_separable_prepare_f32(g);
+      if (e == cudaSuccess) e = convert_tables_f32(g);
       if (e == cudaSuccess) e = cudaDeviceSynchronize();
       return from_cuda(e);
     }

@@ -21,6 +21,7 @@ struct yy_oz_tables;
 
 struct yy_grid {
   int device;
+  int sms;              // SMs of the device
   int n_patch;          // 2: Yin-Yang; 1: full spherical polar grid (rows of every stage: n_patch n_r)
   int n_r, n_theta, n_phi, n_ang, lmax, n_lm;
   double delta_theta, delta_phi, G;
@@ -68,10 +69,11 @@ struct yy_grid {
   double *sep_P, *sep_dP, *sep_Qs;   // [n_theta][n_lm] Legendre factors at the cell colatitudes
   double *sep_tr;                    // [2 l_max + 1][n_phi] 1, cos, sin at the cell longitudes
   float *sep_P32, *sep_dP32, *sep_Qs32, *sep_tr32;   // fp32 copies
-  int sep_syn_ok;                    // the grid fits the separable synthesis's shared memory: bit 0 fp32, bit 1 float64
-  int sep_syn_rows[2];               // rows of G per chunk (fp32, float64)
-  size_t sep_syn_smem[2];            // its shared memory (fp32, float64)
-  int sep_syn_blocks[2];             // its persistent blocks (fp32, float64)
+  float *sep_T32[3];                 // sep_P32, sep_dP32, sep_Qs32 as [n_lm][n_theta]
+  float *sep_G32;                    // fp32 theta sums of the synthesis, in tiles (YY_FP32 prepared)
+  double *sep_trf;                   // [2 l_max + 1][columns] sep_tr at the folded columns (az_fold)
+  double *sep_isin;                  // [n_theta] 1 / sin(theta_j)
+  int sep_syn_ok;                    // separable synthesis available: bit 0 fp32, bit 1 float64
 
   // float32 form
   float *ban32, *ysyn32, *ysyn_t32, *ysyn_p32;   // same layouts as float64
@@ -109,6 +111,16 @@ struct yy_grid {
 
 namespace yy {
 
+// The azimuthal cells folded by their symmetries: column c < half stands for
+// cells first + c and its mirror n_phi - 1 - (first + c) about phi = 0 (phi = pi
+// on the polar grid).  Where pi is a whole number of cells, cells phi and
+// pi - phi are columns c and partner - c (partner = -1: they are not cells);
+// columns c < cols then stand for all of them.
+struct AzFold {
+  int half, cols, first, partner;
+};
+AzFold az_fold(const yy_grid *g);
+
 // Count a kernel launch of the current solve; while profiling, also record an
 // event after it on the launching stream (yy_grid_kernel_ms reads them).
 inline void note_launch(yy_grid *g, const char *name, cudaStream_t s) {
@@ -132,6 +144,18 @@ inline int grid_rows(const yy_grid *g) { return g->n_patch * g->n_r; }
 inline const double *moments_total(const yy_grid *g) { return g->n_patch == 2 ? g->Atot : g->A; }
 
 #ifdef __CUDACC__
+// exact fp32 -> float64 widening by integer operations
+__device__ __forceinline__ double widen_f32(float f) {
+  const unsigned int u = __float_as_uint(f);
+  const unsigned int ex = (u >> 23) & 0xFFu;
+  if (ex == 0u || ex == 255u) {
+    if ((u << 1) == 0u) return __hiloint2double((int)(u & 0x80000000u), 0);
+    return (double)f;
+  }
+  const unsigned int hi = (u & 0x80000000u) | ((ex + 896u) << 20) | ((u & 0x7FFFFFu) >> 3);
+  return __hiloint2double((int)hi, (int)(u << 29));
+}
+
 // The rotation M (x, y, z) -> (-x, z, y) commutes with the reflection
 // x -> -x, under which a real harmonic of order m is even or odd: cos(m phi)
 // with the sign (-1)^m, sin(m phi) with (-1)^(m + 1).  So D^l_ij vanishes
@@ -185,6 +209,9 @@ cudaError_t convert_tables_f32(yy_grid *g);
 cudaError_t separable_prepare(yy_grid *g);
 cudaError_t analysis_separable(yy_grid *g, const double *rho_yin, const double *rho_yang, bool fp64,
                                cudaStream_t s);
+// separable synthesis (yy_sep_synth.cu)
+cudaError_t synthesis_separable_prepare(yy_grid *g);
+cudaError_t synthesis_separable_prepare_f32(yy_grid *g);   // its fp32 tables and workspace
 cudaError_t synthesis_separable(yy_grid *g, double *phi_yin, double *phi_yang, double *grad_yin,
                                 double *grad_yang, bool fp64, cudaStream_t s);
 // the float64 polar stage alone: A from the azimuthal sums in sep_F

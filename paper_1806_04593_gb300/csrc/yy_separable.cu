@@ -38,18 +38,6 @@ __device__ __forceinline__ float narrow(double x) {
   return __uint_as_float((hi & 0x80000000u) | (((unsigned int)e32 << 23) + m23 + up));
 }
 
-// exact fp32 -> float64 widening by integer operations
-__device__ __forceinline__ double widen(float f) {
-  const unsigned int u = __float_as_uint(f);
-  const unsigned int ex = (u >> 23) & 0xFFu;
-  if (ex == 0u || ex == 255u) {
-    if ((u << 1) == 0u) return __hiloint2double((int)(u & 0x80000000u), 0);
-    return (double)f;
-  }
-  const unsigned int hi = (u & 0x80000000u) | ((ex + 896u) << 20) | ((u & 0x7FFFFFu) >> 3);
-  return __hiloint2double((int)hi, (int)(u << 29));
-}
-
 template <typename T>
 __device__ __forceinline__ T to_t(double x) {
   if constexpr (sizeof(T) == 4)
@@ -259,7 +247,7 @@ __device__ void theta_modes_f32(int n_theta, int n_lm, int lmax1, int nt_pad, co
         const float2 a = tb0[(size_t)j * lmax1 + l], b = f0s[j];
         pair_fma(h, lo, a.x, a.y, b.x, b.y);
       }
-      Arow[l * l] = widen(h) + widen(lo);
+      Arow[l * l] = widen_f32(h) + widen_f32(lo);
     }
   }
   for (int idx = threadIdx.x; idx < n_lm; idx += blockDim.x) {
@@ -269,7 +257,7 @@ __device__ void theta_modes_f32(int n_theta, int n_lm, int lmax1, int nt_pad, co
     float s = 0.0f;
 #pragma unroll 8
     for (int j = 0; j < n_theta; ++j) s = fmaf(tb[(size_t)j * n_lm + idx], fs[j * nt_pad + t], s);
-    Arow[idx] = widen(s);
+    Arow[idx] = widen_f32(s);
   }
 }
 
@@ -354,7 +342,7 @@ __global__ void __launch_bounds__(256) k_sep_theta_partials(SepThetaPartials a, 
       const size_t row = (size_t)(shell0 + q) * a.n_theta + j;
       const double d = a.F0[row];
       const float hi = narrow(d);
-      f0 = make_float2(hi, narrow(d - widen(hi)));
+      f0 = make_float2(hi, narrow(d - widen_f32(hi)));
       sc = a.row_scale[row];
       mn = narrow(a.mean[row]);
     }
@@ -382,7 +370,7 @@ __global__ void __launch_bounds__(256) k_sep_theta_partials(SepThetaPartials a, 
         const float2 x = a.tb0[(size_t)j * a.lmax1 + l], y = f0s[warp * a.n_theta + j];
         pair_fma(h, lo, x.x, x.y, y.x, y.y);
       }
-      a.A[(size_t)(shell0 + warp) * a.n_lm + l * l] = widen(h) + widen(lo);
+      a.A[(size_t)(shell0 + warp) * a.n_lm + l * l] = widen_f32(h) + widen_f32(lo);
     }
   }
   // the other modes: fp32 dot products over j, one table read for all S shells
@@ -401,7 +389,7 @@ __global__ void __launch_bounds__(256) k_sep_theta_partials(SepThetaPartials a, 
     }
 #pragma unroll
     for (int q = 0; q < S; ++q)
-      if (q < ns) a.A[(size_t)(shell0 + q) * a.n_lm + idx] = widen(acc[q]);
+      if (q < ns) a.A[(size_t)(shell0 + q) * a.n_lm + idx] = widen_f32(acc[q]);
   }
 }
 
@@ -432,95 +420,6 @@ cudaError_t run_separable(yy_grid *g, const double *rho_yin, const double *rho_y
                                                     (const float2 *)g->sep_F0, g->A);
   note_launch(g, "k_sep_theta", s);
   return cudaGetLastError();
-}
-
-// Separable synthesis (CUDA-core forms), persistent over shells (p, i).  Each
-// block keeps the cell-centre trig table tr[t][k] in shared memory; per field
-// (Phi, g_r, g_theta, g_phi):
-//   theta stage  G[j][t] = sum_{l >= m} q[l^2 + t] P_f[j][l^2 + t]
-//                (g_phi: the cos slot takes the sin coefficients and the sin
-//                slot minus the cos ones, from d/dphi of cos / sin (m phi))
-//   phi stage    out[j][k] = sum_t G[j][t] tr[t][k]
-// with q the combined coefficients of the field (Q, Q_r, Q_t, Q_t).  Both
-// sums run from the top down (l from l_max, t from 2 l_max): the monopole
-// (l = 0, t = 0) dominates Phi and g_r, and adding it last leaves one
-// rounding of the large value instead of one per small term (fp32: Phi
-// error about 1e-6 -> a few 1e-7).
-struct SepOut {
-  double *o[4][2];     // field, patch
-};
-
-template <typename T>
-__global__ void k_sep_synth(int n_shells, int n_r, int n_theta, int n_phi, int lmax, int n_lm, int n_fields, int jr,
-                            const double *__restrict__ Q, const T *__restrict__ P, const T *__restrict__ dP,
-                            const T *__restrict__ Qs, const T *__restrict__ tr, const SepOut out) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int nt = 2 * lmax + 1;
-  const int ntr = (n_phi + 3) & ~3;                     // padded row of the trig table
-  const int ntp = nt | 1;                               // odd row stride of G
-  T *trs = reinterpret_cast<T *>(smraw);                // [nt][ntr]
-  T *Gs = trs + (size_t)nt * ntr;                       // [jr][ntp]: G of one chunk of jr rows
-  T *qs = Gs + (size_t)jr * ntp;                        // [n_lm]
-  for (int e = threadIdx.x; e < nt * ntr; e += blockDim.x) {
-    const int t = e / ntr, k = e % ntr;
-    trs[e] = (k < n_phi) ? tr[(size_t)t * n_phi + k] : T(0);
-  }
-  const size_t n_ang = (size_t)n_theta * n_phi;
-  const size_t qsz = (size_t)n_shells * n_lm;
-  const int kg = ntr / 4;                                // groups of four longitudes
-  for (int shell = blockIdx.x; shell < n_shells; shell += gridDim.x) {
-    const int p = shell / n_r, i = shell % n_r;
-    for (int f = 0; f < n_fields; ++f) {
-      const int qb = f < 2 ? f : 2;
-      const T *tab = (f <= 1) ? P : (f == 2 ? dP : Qs);
-      __syncthreads();   // trs written / the previous field's G and q consumed
-      for (int idx = threadIdx.x; idx < n_lm; idx += blockDim.x) qs[idx] = to_t<T>(Q[qb * qsz + (size_t)shell * n_lm + idx]);
-      __syncthreads();
-      double *dst = out.o[f][p] + (size_t)i * n_ang;
-      for (int j0 = 0; j0 < n_theta; j0 += jr) {
-        const int rows = min(jr, n_theta - j0);
-        for (int e = threadIdx.x; e < rows * nt; e += blockDim.x) {
-          const int jj = e / nt, t = e % nt;
-          const int m = (t + 1) / 2;
-          const T *tj = tab + (size_t)(j0 + jj) * n_lm;
-          T g = T(0);
-          if (f < 3) {
-            for (int l = lmax; l >= m; --l) g = fma(qs[l * l + t], tj[l * l + t], g);
-          } else if (t > 0) {
-            const int src = (t & 1) ? t + 1 : t - 1;      // cos slot <- sin coefficient, sin slot <- cos
-            for (int l = lmax; l >= m; --l) g = fma(qs[l * l + src], tj[l * l + t], g);
-            if (!(t & 1)) g = -g;
-          }
-          Gs[jj * ntp + t] = g;
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < rows * kg; e += blockDim.x) {
-          const int jj = e / kg, k0 = (e % kg) * 4;
-          const int j = j0 + jj;
-          T acc[4] = {T(0), T(0), T(0), T(0)};
-          const T *gj = Gs + jj * ntp;
-          for (int t = nt - 1; t >= 0; --t) {
-            T a4[4];
-            ld4(trs + (size_t)t * ntr + k0, a4);
-            const T gv = gj[t];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) acc[u] = fma(gv, a4[u], acc[u]);
-          }
-          double *o = dst + (size_t)j * n_phi + k0;
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            if (k0 + u < n_phi) {
-              if constexpr (sizeof(T) == 4)
-                o[u] = widen(acc[u]);
-              else
-                o[u] = acc[u];
-            }
-          }
-        }
-        __syncthreads();   // G of this chunk consumed
-      }
-    }
-  }
 }
 
 }  // namespace
@@ -562,28 +461,7 @@ cudaError_t separable_prepare(yy_grid *g) {
     k_round<<<(unsigned)((n_p + 255) / 256), 256>>>(n_p, g->sep_Qs, g->sep_Qs32);
     k_round<<<(unsigned)((n_tr + 255) / 256), 256>>>(n_tr, g->sep_tr, g->sep_tr32);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // shared memory: the trig table, G of jr rows (all n_theta where they
-    // fit, else as many as fit) and one shell's coefficients
-    const int nt = 2 * g->lmax + 1, ntr = (g->n_phi + 3) & ~3;
-    const void *ks[2] = {(const void *)k_sep_synth<float>, (const void *)k_sep_synth<double>};
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device);
-    g->sep_syn_ok = 0;
-    for (int q = 0; q < 2; ++q) {
-      const size_t el = q == 0 ? sizeof(float) : sizeof(double);
-      const size_t fixed = ((size_t)nt * ntr + g->n_lm) * el, per_row = (size_t)(nt | 1) * el;
-      if (fixed + per_row > 227 * 1024) continue;
-      const int jr = (int)std::min<size_t>(g->n_theta, (227 * 1024 - fixed) / per_row);
-      g->sep_syn_rows[q] = jr;
-      g->sep_syn_smem[q] = fixed + jr * per_row;
-      if ((e = cudaFuncSetAttribute(ks[q], cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024)) != cudaSuccess)
-        return e;
-      int nb = 0;
-      if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, ks[q], 256, g->sep_syn_smem[q])) != cudaSuccess)
-        return e;
-      g->sep_syn_blocks[q] = std::max(nb, 1) * sms;
-      g->sep_syn_ok |= 1 << q;
-    }
+    if ((e = synthesis_separable_prepare(g)) != cudaSuccess) return e;
   }
   // shared memory of the azimuthal stage (the table and one chunk of rows);
   // grids too large for it leave the separable analysis unavailable
@@ -616,31 +494,6 @@ cudaError_t separable_prepare(yy_grid *g) {
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024)) != cudaSuccess)
       return e;
   return cudaSuccess;
-}
-
-cudaError_t synthesis_separable(yy_grid *g, double *phi_yin, double *phi_yang, double *grad_yin, double *grad_yang,
-                                bool fp64, cudaStream_t s) {
-  const size_t comp = (size_t)g->n_r * g->n_ang;
-  SepOut o = {};
-  o.o[0][0] = phi_yin;
-  o.o[0][1] = phi_yang;
-  for (int c = 0; c < 3 && grad_yin; ++c) {
-    o.o[1 + c][0] = grad_yin + c * comp;
-    o.o[1 + c][1] = grad_yang ? grad_yang + c * comp : nullptr;
-  }
-  const int n_fields = grad_yin ? 4 : 1;
-  const int q = fp64 ? 1 : 0;
-  const int blocks = std::min(grid_rows(g), g->sep_syn_blocks[q]);
-  if (fp64)
-    k_sep_synth<double><<<blocks, 256, g->sep_syn_smem[1], s>>>(grid_rows(g), g->n_r, g->n_theta, g->n_phi, g->lmax, g->n_lm,
-                                                                n_fields, g->sep_syn_rows[1], g->Q, g->sep_P, g->sep_dP, g->sep_Qs,
-                                                                g->sep_tr, o);
-  else
-    k_sep_synth<float><<<blocks, 256, g->sep_syn_smem[0], s>>>(grid_rows(g), g->n_r, g->n_theta, g->n_phi, g->lmax, g->n_lm,
-                                                               n_fields, g->sep_syn_rows[0], g->Q, g->sep_P32, g->sep_dP32, g->sep_Qs32,
-                                                               g->sep_tr32, o);
-  note_launch(g, "k_sep_synth", s);
-  return cudaGetLastError();
 }
 
 size_t separable_theta_partials_smem(const yy_grid *g, int nt_pad) {
