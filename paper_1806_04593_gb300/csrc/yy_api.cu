@@ -62,7 +62,7 @@ static void free_all(yy_grid *g) {
     if (p) cudaFree(p);
   float *fbufs[] = {g->rot32, g->ban32, g->ysyn32, g->ysyn_t32, g->ysyn_p32, g->rho32, g->Q32,
                     g->sep_az32, g->sep_w32, g->sep_tb32};
-  double *sbufs[] = {g->sep_az, g->sep_F, g->sep_F0, g->sep_P, g->sep_dP, g->sep_Qs, g->sep_tr, g->sep_trf,
+  double *sbufs[] = {g->sep_az, g->sep_azf, g->sep_F, g->sep_F0, g->sep_P, g->sep_dP, g->sep_Qs, g->sep_tr, g->sep_trf,
                      g->sep_isin};
   float *sfbufs[] = {g->sep_P32, g->sep_dP32, g->sep_Qs32, g->sep_tr32, g->sep_T32[0],
                      g->sep_T32[1], g->sep_T32[2], g->sep_G32};

@@ -59,9 +59,8 @@ struct yy_grid {
   int last_separable;   // the last solve used the separable analysis
   int sep_nt_pad;       // 2 l_max + 1 azimuthal functions, padded to a multiple of 4
   int sep_ok;           // the grid fits the separable kernels' shared memory: bit 0 fp32, bit 1 float64
-  int sep_jc[2];        // rows per item of the azimuthal stage (fp32, float64)
-  int sep_phi_blocks[2];  // persistent blocks of the azimuthal stage (fp32, float64)
   double *sep_az;       // [n_phi][sep_nt_pad] cell integrals of the azimuthal functions
+  double *sep_azf;      // [columns][l_max + 1][cos, sin] sep_az at the folded columns (az_fold)
   float *sep_az32, *sep_w32, *sep_tb32;   // fp32 copies of sep_az, w, tbar
   double *sep_F;        // [2 n_r][n_theta][sep_nt_pad] azimuthal stage (float64 or fp32)
   double *sep_F0;       // [2 n_r][n_theta] m = 0 row sums as fp32 pairs (fp32 form)

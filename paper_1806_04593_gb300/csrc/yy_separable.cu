@@ -26,24 +26,15 @@
 namespace yy {
 namespace {
 
-// exact float64 -> fp32 rounding by integer operations (round to nearest even)
+// exact float64 -> fp32 rounding by integer operations (round to nearest even):
+// the rounding bias added at bit 29 of the 64-bit word, bits 29..60 kept and the
+// exponent rebiased; values outside the normal fp32 range are converted
 __device__ __forceinline__ float narrow(double x) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(x);
   const unsigned int hi = (unsigned int)(u >> 32);
-  const int e32 = (int)((hi >> 20) & 0x7FFu) - 1023 + 127;
-  if (e32 <= 0 || e32 >= 255) return (u << 1) == 0ull ? __uint_as_float(hi & 0x80000000u) : (float)x;
-  const unsigned long long man = u & 0xFFFFFFFFFFFFFull;
-  const unsigned int m23 = (unsigned int)(man >> 29), rem = (unsigned int)(man & 0x1FFFFFFFull);
-  const unsigned int up = (rem > 0x10000000u || (rem == 0x10000000u && (m23 & 1u))) ? 1u : 0u;
-  return __uint_as_float((hi & 0x80000000u) | (((unsigned int)e32 << 23) + m23 + up));
-}
-
-template <typename T>
-__device__ __forceinline__ T to_t(double x) {
-  if constexpr (sizeof(T) == 4)
-    return narrow(x);
-  else
-    return x;
+  if (((hi >> 20) & 0x7FFu) - 897u >= 254u) return (float)x;
+  const unsigned int r = (unsigned int)((u + 0x0FFFFFFFull + ((u >> 29) & 1ull)) >> 29) - (896u << 23);
+  return __uint_as_float((r & 0x7FFFFFFFu) | (hi & 0x80000000u));
 }
 
 // Knuth's two-sum into an unevaluated fp32 pair (h, l)
@@ -94,11 +85,7 @@ __global__ void k_round(size_t n, const double *__restrict__ src, float *__restr
   if (e < n) dst[e] = (float)src[e];
 }
 
-constexpr int kJC = 48;    // rows j per work item (kJCSmall where the table leaves too little room)
-constexpr int kJCSmall = 16;
-constexpr int kTJ = 4;     // rows per thread
-constexpr int kTT = 4;     // azimuthal functions per thread
-__host__ __device__ constexpr int xpad(int jc) { return jc + 4; }   // padded row stride of the staged densities
+constexpr int kTT = 4;     // azimuthal functions per thread of the fp32 azimuthal stage
 
 // four consecutive values, 16-byte aligned
 __device__ __forceinline__ void ld4(const float *p, float (&o)[4]) {
@@ -108,19 +95,8 @@ __device__ __forceinline__ void ld4(const float *p, float (&o)[4]) {
   o[2] = v.z;
   o[3] = v.w;
 }
-__device__ __forceinline__ void ld4(const double *p, double (&o)[4]) {
-  const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
-  o[0] = a.x;
-  o[1] = a.y;
-  o[2] = b.x;
-  o[3] = b.y;
-}
 __device__ __forceinline__ void st4(float *p, const float (&v)[4]) {
   *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
-}
-__device__ __forceinline__ void st4(double *p, const double (&v)[4]) {
-  reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
-  reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
 }
 
 // exact product a b = p + e (fma-based) and an unevaluated-pair dot step
@@ -131,185 +107,349 @@ __device__ __forceinline__ void pair_fma(float &h, float &l, float ah, float al,
   l += e + fmaf(ah, bl, al * bh);
 }
 
-// Azimuthal stage, persistent: each block keeps the table az in shared
-// memory and takes work items (shell, chunk of JC rows j) in turn.
-//  1. all threads stage the chunk (JC n_phi consecutive densities) with 16
-//     independent loads in flight each, fold in w and store it transposed;
-//  2. (fp32) one warp per row forms the row's compensated sum (the m = 0
-//     azimuthal sum without the factor d_phi) as an unevaluated fp32 pair;
-//  3. each thread accumulates a tile of kTJ rows x kTT functions over all k
-//     with two vector shared-memory loads per 16 products.
-template <typename T, int JC>
-__global__ void k_sep_phi(int n_shells, int n_r, int n_theta, int n_phi, int nt_pad, const double *__restrict__ rho0,
-                          const double *__restrict__ rho1, const T *__restrict__ w, const T *__restrict__ az,
-                          T *__restrict__ F, float2 *__restrict__ F0) {
+// Azimuthal stage, float64.  The float64 pipe (two operations per clock per SM)
+// sets the time, so the cells are folded by their symmetries first (AzFold):
+// with E, O the sum and difference of a cell and its mirror, cos slots take E
+// and sin slots O over half the columns; where cells phi and pi - phi both
+// exist, E +- E' and O -+ O' serve the even and odd orders over a third of them
+// (on the 1-degree Yin-Yang grid 90 columns for 270 cells: 19.7 float64
+// operations per cell instead of 52; 0.97 ms there at 550 zones and l_max 25
+// against 3.02 ms without the folds, 72 against 214 us on the 2-degree grid of
+// 200 zones at l_max 15).  A block takes up to 16 consecutive rows
+// (shell, j); each thread then sums both slots of an order m for two rows.
+constexpr int kR64 = 2;
+
+struct SepPhi64 {
+  int rows, per, n_r, n_theta, n_phi, m1, nt_pad;   // per: rows of a block, even
+  AzFold fold;
+  const double *rho0, *rho1, *w;
+  const double2 *az;   // [column][m]: the cell integrals of cos and sin (m phi)
+  double *F;
+};
+
+__global__ void k_sep_phi64(const SepPhi64 a) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  T *as = reinterpret_cast<T *>(smraw);                  // [n_phi][nt_pad]
-  constexpr int XP = xpad(JC);
-  T *xs = as + (size_t)n_phi * nt_pad;                   // [n_phi][XP]
-  const int tg = nt_pad / kTT;
-  const int tt = threadIdx.x % tg, tj = threadIdx.x / tg;   // function group, row group
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-  const size_t n_ang = (size_t)n_theta * n_phi;
-  const int chunks = (n_theta + JC - 1) / JC;
-  const int items = n_shells * chunks;
-  constexpr int kU = 16;
-  const float inv_phi = 1.0f / (float)n_phi;
-
-  for (int e = threadIdx.x; e < n_phi * nt_pad; e += blockDim.x) as[e] = az[e];
-
-  for (int item = blockIdx.x; item < items; item += gridDim.x) {
-    const int shell = item / chunks, j0 = (item % chunks) * JC;
-    const int p = shell / n_r, i = shell % n_r;
-    const int rows = min(JC, n_theta - j0);
-    const int count = rows * n_phi;                      // consecutive values of the chunk
-    const double *src = (p == 0 ? rho0 : rho1) + (size_t)i * n_ang + (size_t)j0 * n_phi;
-    const T *wsrc = w + (size_t)j0 * n_phi;
-    __syncthreads();   // the previous item's tiles are done with xs (and as is written)
-    for (int e0 = threadIdx.x; e0 < JC * n_phi; e0 += kU * blockDim.x) {
-      double rv[kU];
-      T wv[kU];
-#pragma unroll
-      for (int u = 0; u < kU; ++u) {
-        const int e = e0 + u * blockDim.x;
-        rv[u] = (e < count) ? src[e] : 0.0;
-        wv[u] = (e < count) ? wsrc[e] : T(0);
-      }
-#pragma unroll
-      for (int u = 0; u < kU; ++u) {
-        const int e = e0 + u * blockDim.x;
-        if (e < JC * n_phi) {
-          // e = jj n_phi + k: quotient from the float reciprocal, then corrected
-          int jj = (int)((float)e * inv_phi);
-          int k = e - jj * n_phi;
-          if (k < 0) {
-            --jj;
-            k += n_phi;
-          } else if (k >= n_phi) {
-            ++jj;
-            k -= n_phi;
-          }
-          xs[(size_t)k * XP + jj] = to_t<T>(rv[u]) * wv[u];
+  double *xs = reinterpret_cast<double *>(smraw);   // [E even m, E odd m, O even m, O odd m][column][per]
+  const int row0 = blockIdx.x * a.per, cols = a.fold.cols, plane = cols * a.per;
+  const int patch_rows = a.n_r * a.n_theta;
+  for (int e = threadIdx.x; e < plane; e += blockDim.x) {
+    const int r = e / cols, c = e % cols, row = row0 + r;
+    double ee = 0.0, eo = 0.0, oe = 0.0, oo = 0.0;
+    if (row < a.rows) {
+      const double *x = (row >= patch_rows ? a.rho1 + (size_t)(row - patch_rows) * a.n_phi : a.rho0 + (size_t)row * a.n_phi);
+      const double *w = a.w + (size_t)(row % a.n_theta) * a.n_phi;
+      auto fold = [&](int kp, double &E, double &O) {
+        const int km = a.n_phi - 1 - kp;
+        const double u = x[kp] * w[kp];
+        if (km == kp) {
+          E = u;
+          O = 0.0;
+        } else {
+          const double v = x[km] * w[km];
+          E = u + v;
+          O = u - v;
         }
+      };
+      fold(a.fold.first + c, ee, oe);
+      eo = ee;
+      oo = oe;
+      const int pc = a.fold.partner - c;
+      if (a.fold.partner >= 0 && pc > c && pc < a.fold.half) {
+        double E, O;
+        fold(a.fold.first + pc, E, O);
+        eo = ee - E;   // cos(m (pi - phi)) = (-1)^m cos(m phi)
+        ee = ee + E;
+        oo = oe + O;   // sin(m (pi - phi)) = -(-1)^m sin(m phi)
+        oe = oe - O;
       }
     }
-    __syncthreads();
-    if constexpr (sizeof(T) == 4) {
-      for (int jj = warp; jj < rows; jj += n_warps) {
-        float h = 0.0f, l = 0.0f;
-        for (int k = lane; k < n_phi; k += 32) pair_add(h, l, xs[(size_t)k * XP + jj]);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-          const float oh = __shfl_xor_sync(0xffffffffu, h, off);
-          const float ol = __shfl_xor_sync(0xffffffffu, l, off);
-          pair_add(h, l, oh);
-          l += ol;
-        }
-        if (lane == 0) F0[(size_t)shell * n_theta + j0 + jj] = make_float2(h, l);
-      }
+    double *o = xs + c * a.per + r;
+    o[0] = ee;
+    o[plane] = eo;
+    o[2 * plane] = oe;
+    o[3 * plane] = oo;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < a.per / kR64 * a.m1; e += blockDim.x) {
+    const int r = e / a.m1 * kR64, m = e % a.m1;
+    const double *xe = xs + (m & 1 ? plane : 0) + r, *xo = xe + 2 * plane;
+    const double2 *az = a.az + m;
+    double cs[kR64] = {0.0, 0.0}, sn[kR64] = {0.0, 0.0};
+#pragma unroll 4
+    for (int c = 0; c < cols; ++c) {
+      const double2 t = az[(size_t)c * a.m1];
+      const double2 u = *reinterpret_cast<const double2 *>(xe + c * a.per), v = *reinterpret_cast<const double2 *>(xo + c * a.per);
+      cs[0] = fma(u.x, t.x, cs[0]);
+      cs[1] = fma(u.y, t.x, cs[1]);
+      sn[0] = fma(v.x, t.y, sn[0]);
+      sn[1] = fma(v.y, t.y, sn[1]);
     }
-    if (tj < JC / kTJ) {
-      T acc[kTJ][kTT];
 #pragma unroll
-      for (int a = 0; a < kTJ; ++a)
-#pragma unroll
-        for (int b = 0; b < kTT; ++b) acc[a][b] = T(0);
-#pragma unroll 2
-      for (int k = 0; k < n_phi; ++k) {
-        T x4[4], a4[4];
-        ld4(xs + (size_t)k * XP + tj * kTJ, x4);
-        ld4(as + (size_t)k * nt_pad + tt * kTT, a4);
-#pragma unroll
-        for (int a = 0; a < kTJ; ++a)
-#pragma unroll
-          for (int b = 0; b < kTT; ++b) acc[a][b] = fma(x4[a], a4[b], acc[a][b]);
-      }
-#pragma unroll
-      for (int a = 0; a < kTJ; ++a) {
-        const int j = j0 + tj * kTJ + a;
-        if (j >= n_theta) continue;
-        st4(F + ((size_t)shell * n_theta + j) * nt_pad + tt * kTT, acc[a]);
+    for (int i = 0; i < kR64; ++i) {
+      if (row0 + r + i >= a.rows) break;
+      double *F = a.F + (size_t)(row0 + r + i) * a.nt_pad;
+      if (m == 0) {
+        F[0] = cs[i];
+      } else {
+        F[2 * m - 1] = cs[i];
+        F[2 * m] = sn[i];
       }
     }
   }
 }
 
-// The fp32 polar stage on one shell: F (shared memory, [n_theta][nt_pad]) and
-// the pair row sums f0s; the m = 0 modes as an unevaluated-pair dot product,
-// the others as fp32 dot products over j.
-__device__ void theta_modes_f32(int n_theta, int n_lm, int lmax1, int nt_pad, const float *__restrict__ tb,
-                                const float2 *__restrict__ tb0, const float *fs, const float2 *f0s,
-                                double *__restrict__ Arow) {
-  if (threadIdx.x < 32) {
-    for (int l = threadIdx.x; l < lmax1; l += 32) {
-      float h = 0.0f, lo = 0.0f;
-      for (int j = 0; j < n_theta; ++j) {
-        const float2 a = tb0[(size_t)j * lmax1 + l], b = f0s[j];
-        pair_fma(h, lo, a.x, a.y, b.x, b.y);
+// az[column][m] = the cell integrals of cos and sin (m phi) at the folded columns
+__global__ void k_fold_az(int m1, int nt_pad, AzFold f, const double *__restrict__ az, double2 *__restrict__ out) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= m1 * f.cols) return;
+  const int c = e / m1, m = e % m1;
+  const double *row = az + (size_t)(f.first + c) * nt_pad;
+  out[e] = m == 0 ? make_double2(row[0], 0.0) : make_double2(row[2 * m - 1], row[2 * m]);
+}
+
+// Azimuthal stage, fp32: every F is one chain of fp32 multiply-adds over k in
+// order.  A block takes 32 consecutive rows (shell, j) of a patch and walks k in
+// pieces of 32.  Four warps copy the next piece while this one is summed (8 rows
+// each, lane = k), round and weight it and write it transposed; all threads sum
+// it, R rows x 4 functions each, the table's piece in shared memory beside it
+// (through L1 it came from L2: the staged rows leave L1 little room).  On the
+// 1-degree grid, 550 zones, l_max 25: 167 us (300 us with whole shells staged and
+// the table read per 16 products), about 70 of them instruction issue; 23 us
+// against 48 on the 2-degree grid of 200 zones at l_max 15.  The row's compensated sum (the m = 0
+// azimuthal sum without the factor d_phi) is formed by the lanes as they convert:
+// lane L adds k = L, L + 32, ... to an unevaluated fp32 pair, and shuffles add the
+// lanes' pairs.
+constexpr int kRows32 = 32, kPiece = 32, kLoadWarps = 4, kLoadRows = kRows32 / kLoadWarps;
+constexpr int kLd32 = kRows32 + 4;   // row stride of a staged k: 16-byte writes of 8 lanes on 32 banks
+
+struct SepPhi32 {
+  int n_r, n_theta, n_phi, nt_pad;
+  const double *rho[2];
+  const float *w, *az;   // az [k][nt_pad]
+  float *F;
+  float2 *F0;
+};
+
+__device__ __forceinline__ void copy_async(double *dst, const double *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async16(float *dst, const float *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async(float *dst, const float *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
+template <int kR32>
+__global__ void k_sep_phi32(const SepPhi32 a) {
+  extern __shared__ __align__(16) float azs[];            // [2][kPiece][nt_pad]
+  __shared__ __align__(16) double raw[kRows32][kPiece];
+  __shared__ __align__(16) float wts[kRows32][kPiece];
+  __shared__ __align__(16) float xs[2][kPiece * kLd32];   // [k][row]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int patch_rows = a.n_r * a.n_theta, row0 = blockIdx.x * kRows32;
+  const int rows = min(kRows32, patch_rows - row0), j0 = row0 % a.n_theta;
+  const double *src = (blockIdx.y ? a.rho[1] : a.rho[0]) + (size_t)row0 * a.n_phi;
+  const size_t out0 = (size_t)blockIdx.y * patch_rows + row0;
+  const int tg = a.nt_pad / kTT, r = threadIdx.x / tg * kR32, tt = threadIdx.x % tg;
+  const int pieces = (a.n_phi + kPiece - 1) / kPiece, q = warp * kLoadRows;
+  const bool loads = warp < kLoadWarps;
+  int wrow[kLoadRows];   // the rows' offsets in the weights
+#pragma unroll
+  for (int i = 0; i < kLoadRows; ++i) wrow[i] = (j0 + q + i) % a.n_theta * a.n_phi;
+  // the rows: a thread reads only what it copied itself; the table: after a barrier
+  auto fetch = [&](int p) {
+    const int k = p * kPiece + lane;
+    if (loads && k < a.n_phi) {
+#pragma unroll
+      for (int i = 0; i < kLoadRows; ++i) {
+        if (q + i >= rows) break;
+        copy_async(&raw[q + i][lane], src + (q + i) * a.n_phi + k);
+        copy_async(&wts[q + i][lane], a.w + wrow[i] + k);
       }
-      Arow[l * l] = widen_f32(h) + widen_f32(lo);
+    }
+    const int n = min(kPiece, a.n_phi - p * kPiece) * a.nt_pad;
+    for (int e = threadIdx.x * 4; e < n; e += blockDim.x * 4)
+      copy_async16(azs + (p & 1) * kPiece * a.nt_pad + e, a.az + (size_t)p * kPiece * a.nt_pad + e);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  fetch(0);
+  float h[kLoadRows], l[kLoadRows];
+#pragma unroll
+  for (int i = 0; i < kLoadRows; ++i) h[i] = l[i] = 0.0f;
+  float acc[kR32][kTT];
+#pragma unroll
+  for (int i = 0; i < kR32; ++i)
+#pragma unroll
+    for (int b = 0; b < kTT; ++b) acc[i][b] = 0.0f;
+  for (int p = 0; p < pieces; ++p) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (loads) {
+      const bool in = p * kPiece + lane < a.n_phi;
+      float v[kLoadRows];
+#pragma unroll
+      for (int i = 0; i < kLoadRows; ++i) {
+        v[i] = 0.0f;
+        if (in && q + i < rows) {
+          v[i] = __fmul_rn(narrow(raw[q + i][lane]), wts[q + i][lane]);   // rounded before the pair's sum
+          pair_add(h[i], l[i], v[i]);
+        }
+      }
+      float4 *to = reinterpret_cast<float4 *>(&xs[p & 1][lane * kLd32 + q]);
+      to[0] = make_float4(v[0], v[1], v[2], v[3]);
+      to[1] = make_float4(v[4], v[5], v[6], v[7]);
+    }
+    __syncthreads();   // piece p is in; the other buffers are used up
+    if (p + 1 < pieces) fetch(p + 1);
+    if (r < kRows32) {
+      const float *x = &xs[p & 1][r], *az = azs + (p & 1) * kPiece * a.nt_pad + tt * kTT;
+      const int n = min(kPiece, a.n_phi - p * kPiece);
+#pragma unroll 8
+      for (int k = 0; k < n; ++k) {
+        float t4[4], u[kR32];
+        ld4(az + k * a.nt_pad, t4);
+        if constexpr (kR32 == 4) {
+          ld4(x + k * kLd32, u);
+        } else {
+          const float2 u2 = *reinterpret_cast<const float2 *>(x + k * kLd32);
+          u[0] = u2.x;
+          u[1] = u2.y;
+        }
+#pragma unroll
+        for (int i = 0; i < kR32; ++i)
+#pragma unroll
+          for (int b = 0; b < kTT; ++b) acc[i][b] = fmaf(u[i], t4[b], acc[i][b]);
+      }
     }
   }
-  for (int idx = threadIdx.x; idx < n_lm; idx += blockDim.x) {
+  if (r < kRows32)
+#pragma unroll
+    for (int i = 0; i < kR32; ++i)
+      if (r + i < rows) st4(a.F + (out0 + r + i) * a.nt_pad + tt * kTT, acc[i]);
+  if (!loads) return;
+#pragma unroll
+  for (int i = 0; i < kLoadRows; ++i) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const float oh = __shfl_xor_sync(0xffffffffu, h[i], off);
+      const float ol = __shfl_xor_sync(0xffffffffu, l[i], off);
+      pair_add(h[i], l[i], oh);
+      l[i] += ol;
+    }
+    if (lane == 0 && q + i < rows) a.F0[out0 + q + i] = make_float2(h[i], l[i]);
+  }
+}
+
+// The polar stages' dot products over j wait for table loads from L2, so a
+// thread keeps eight of them in flight and a block has a thread per mode, up to
+// 1024.
+constexpr int kBatch = 8;
+int theta_threads(int n_lm, int extra) { return std::min(1024, (n_lm + 31) / 32 * 32 + extra); }
+
+// Polar stage, fp32: a block takes S shells, their F in shared memory, so that a
+// table value serves all of them; per mode and shell an fp32 dot product over j
+// in order.  The last warp takes the m = 0 modes: an unevaluated-pair dot product
+// of the pair-split table (with d_phi folded in) and the pair row sums, then one
+// float64 addition.  1-degree grid, 550 zones: 43 us with four shells a block,
+// 70 with one; 200 zones of 2-degree cells: 14 with two, 12 with one.
+template <int S>
+__global__ void k_sep_theta32(int n_shells, int n_theta, int n_lm, int lmax1, int nt_pad, const float *__restrict__ tb,
+                              const float2 *__restrict__ tb0, const float *__restrict__ F, const float2 *__restrict__ F0,
+                              double *__restrict__ A) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int shell0 = blockIdx.x * S, ns = min(S, n_shells - shell0), rows = S * n_theta;
+  float2 *f0s = reinterpret_cast<float2 *>(smraw);                 // [S][n_theta]
+  float *fs = reinterpret_cast<float *>(f0s + rows + (rows & 1));     // [S][n_theta][nt_pad]
+  const size_t row0 = (size_t)shell0 * n_theta;
+  for (int e = threadIdx.x; e < ns * n_theta * nt_pad / 4; e += blockDim.x)
+    reinterpret_cast<float4 *>(fs)[e] = reinterpret_cast<const float4 *>(F + row0 * nt_pad)[e];
+  for (int e = threadIdx.x; e < ns * n_theta; e += blockDim.x) f0s[e] = F0[row0 + e];
+  __syncthreads();
+  const int modes = blockDim.x - 32;   // threads of the m > 0 modes
+  if ((int)threadIdx.x >= modes) {
+    for (int e = threadIdx.x - modes; e < ns * lmax1; e += 32) {
+      const int q = e / lmax1, l = e % lmax1;
+      const float2 *y = f0s + q * n_theta;
+      float h = 0.0f, lo = 0.0f;
+      for (int j0 = 0; j0 < n_theta; j0 += kBatch) {
+        float2 x[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) x[u] = tb0[(size_t)min(j0 + u, n_theta - 1) * lmax1 + l];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u)
+          if (j0 + u < n_theta) pair_fma(h, lo, x[u].x, x[u].y, y[j0 + u].x, y[j0 + u].y);
+      }
+      A[(size_t)(shell0 + q) * n_lm + l * l] = widen_f32(h) + widen_f32(lo);
+    }
+    return;
+  }
+  for (int idx = threadIdx.x; idx < n_lm; idx += modes) {
     const int l = degree_of(idx);
     const int t = idx - l * l;
     if (t == 0) continue;
-    float s = 0.0f;
-#pragma unroll 8
-    for (int j = 0; j < n_theta; ++j) s = fmaf(tb[(size_t)j * n_lm + idx], fs[j * nt_pad + t], s);
-    Arow[idx] = widen_f32(s);
+    const float *tab = tb + idx, *f = fs + t;
+    float s[S];
+#pragma unroll
+    for (int q = 0; q < S; ++q) s[q] = 0.0f;
+    for (int j0 = 0; j0 < n_theta; j0 += kBatch) {
+      float v[kBatch];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) v[u] = tab[(size_t)min(j0 + u, n_theta - 1) * n_lm];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u)
+        if (j0 + u < n_theta) {
+#pragma unroll
+          for (int q = 0; q < S; ++q) s[q] = fmaf(v[u], f[(q * n_theta + j0 + u) * nt_pad], s[q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < S; ++q)
+      if (q < ns) A[(size_t)(shell0 + q) * n_lm + idx] = widen_f32(s[q]);
   }
 }
 
-// Polar stage: one block per shell, the shell's F staged in shared memory, one
-// thread per mode.  The m = 0 modes (fp32 form): an unevaluated-pair dot
-// product of the pair-split table (with d_phi folded in) and the pair row
-// sums, then one float64 addition; float64 for the float64 form.
-template <typename T>
-__global__ void __launch_bounds__(256) k_sep_theta(int n_theta, int n_lm, int lmax1, int nt_pad,
-                                                   const T *__restrict__ tb, const float2 *__restrict__ tb0,
-                                                   const T *__restrict__ F, const float2 *__restrict__ F0,
-                                                   double *__restrict__ A) {
+// Polar stage, float64: one block per shell, the shell's F staged in shared
+// memory, one thread per mode.
+__global__ void k_sep_theta64(int n_theta, int n_lm, int nt_pad, const double *__restrict__ tb,
+                                                     const double *__restrict__ F, double *__restrict__ A) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int shell = blockIdx.x;
-  const T *Fs = F + (size_t)shell * n_theta * nt_pad;
-  if constexpr (sizeof(T) == 4) {
-    float2 *f0s = reinterpret_cast<float2 *>(smraw);       // [n_theta]
-    T *fs = reinterpret_cast<T *>(f0s + n_theta + (n_theta & 1));   // [n_theta][nt_pad]
-    for (int e = threadIdx.x; e < n_theta * nt_pad; e += blockDim.x) fs[e] = Fs[e];
-    for (int j = threadIdx.x; j < n_theta; j += blockDim.x) f0s[j] = F0[(size_t)shell * n_theta + j];
-    __syncthreads();
-    theta_modes_f32(n_theta, n_lm, lmax1, nt_pad, tb, tb0, fs, f0s, A + (size_t)shell * n_lm);
-  } else {
-    // The polar cells are symmetric about the equator (cell n_theta - 1 - j is
-    // cell j reflected), so the cell integrals of P_l^m(cos theta) sin theta
-    // have its parity: T_j' = (-1)^(l + m) T_j.  With S_j = F_j + F_j' and
-    // D_j = F_j - F_j', a mode is the sum over j < ceil(n_theta / 2) of T_j S_j
-    // (even l + m) or T_j D_j (odd): half the products.  A middle row (odd
-    // n_theta) is its own mirror and enters once, as both S and D.
-    const int half = (n_theta + 1) >> 1;
-    T *cs = reinterpret_cast<T *>(smraw);                  // [2][half][nt_pad]: S, then D
-    for (int e = threadIdx.x; e < half * nt_pad; e += blockDim.x) {
-      const int j = e / nt_pad, jm = n_theta - 1 - j;
-      const T a = Fs[e], b = Fs[(size_t)(jm - j) * nt_pad + e];
-      cs[e] = jm == j ? a : a + b;
-      cs[(size_t)half * nt_pad + e] = jm == j ? a : a - b;
+  const double *Fs = F + (size_t)shell * n_theta * nt_pad;
+  // The polar cells are symmetric about the equator (cell n_theta - 1 - j is
+  // cell j reflected), so the cell integrals of P_l^m(cos theta) sin theta
+  // have its parity: T_j' = (-1)^(l + m) T_j.  With S_j = F_j + F_j' and
+  // D_j = F_j - F_j', a mode is the sum over j < ceil(n_theta / 2) of T_j S_j
+  // (even l + m) or T_j D_j (odd): half the products.  A middle row (odd
+  // n_theta) is its own mirror and enters once, as both S and D.
+  const int half = (n_theta + 1) >> 1;
+  double *cs = reinterpret_cast<double *>(smraw);                  // [2][half][nt_pad]: S, then D
+  for (int e = threadIdx.x; e < half * nt_pad; e += blockDim.x) {
+    const int j = e / nt_pad, jm = n_theta - 1 - j;
+    const double a = Fs[e], b = Fs[(size_t)(jm - j) * nt_pad + e];
+    cs[e] = jm == j ? a : a + b;
+    cs[(size_t)half * nt_pad + e] = jm == j ? a : a - b;
+  }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < n_lm; idx += blockDim.x) {
+    const int l = degree_of(idx);
+    const int t = idx - l * l;
+    const double *c = cs + ((((l + ((t + 1) >> 1)) & 1) != 0) ? (size_t)half * nt_pad : 0) + t;
+    const double *tab = tb + idx;
+    double s = 0.0;
+    for (int j0 = 0; j0 < half; j0 += kBatch) {
+      double v[kBatch];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) v[u] = tab[(size_t)min(j0 + u, half - 1) * n_lm];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u)
+        if (j0 + u < half) s = fma(v[u], c[(j0 + u) * nt_pad], s);
     }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < n_lm; idx += blockDim.x) {
-      const int l = degree_of(idx);
-      const int t = idx - l * l;
-      const T *c = cs + ((((l + ((t + 1) >> 1)) & 1) != 0) ? (size_t)half * nt_pad : 0) + t;
-      T s = T(0);
-#pragma unroll 8
-      for (int j = 0; j < half; ++j) s = fma(tb[(size_t)j * n_lm + idx], c[j * nt_pad], s);
-      A[(size_t)shell * n_lm + idx] = s;
-    }
+    A[(size_t)shell * n_lm + idx] = s;
   }
 }
 
-// Dynamic shared memory of k_sep_theta: the fp32 form stages F and the m = 0
-// pair sums, the float64 form the mirrored sums S and D of ceil(n_theta / 2)
+// Dynamic shared memory of the polar stages: the fp32 form stages a shell's F and
+// m = 0 pair sums, the float64 form the mirrored sums S and D of ceil(n_theta / 2)
 // rows each.
 static size_t theta_smem(int n_theta, int nt_pad, size_t el) {
   if (el == sizeof(double)) return (size_t)(n_theta + 1) * nt_pad * sizeof(double);
@@ -393,33 +533,16 @@ __global__ void __launch_bounds__(256) k_sep_theta_partials(SepThetaPartials a, 
   }
 }
 
-// launch shape of the azimuthal stage with JC rows per item
-int phi_threads(int nt_pad, int jc) { return ((nt_pad / kTT) * (jc / kTJ) + 31) / 32 * 32; }   // whole warps
-size_t phi_smem(const yy_grid *g, int nt_pad, int jc, size_t el) {
-  return (size_t)g->n_phi * (nt_pad + xpad(jc)) * el;
-}
-
-template <typename T>
-cudaError_t run_separable(yy_grid *g, const double *rho_yin, const double *rho_yang, const T *w, const T *az,
-                          const T *tb, T *F, int blocks, cudaStream_t s) {
-  const int nt_pad = g->sep_nt_pad;
-  const int jc = g->sep_jc[sizeof(T) == 8];
-  const int threads = phi_threads(nt_pad, jc);
-  const size_t smem_phi = phi_smem(g, nt_pad, jc, sizeof(T));
-  const int shells = grid_rows(g);
-  const int grid = std::min(shells * ((g->n_theta + jc - 1) / jc), blocks);
-  if (jc == kJC)
-    k_sep_phi<T, kJC><<<grid, threads, smem_phi, s>>>(shells, g->n_r, g->n_theta, g->n_phi, nt_pad, rho_yin, rho_yang,
-                                                      w, az, F, (float2 *)g->sep_F0);
-  else
-    k_sep_phi<T, kJCSmall><<<grid, threads, smem_phi, s>>>(shells, g->n_r, g->n_theta, g->n_phi, nt_pad, rho_yin,
-                                                           rho_yang, w, az, F, (float2 *)g->sep_F0);
-  note_launch(g, "k_sep_phi", s);
-  const size_t smem_theta = theta_smem(g->n_theta, nt_pad, sizeof(T));
-  k_sep_theta<T><<<shells, 256, smem_theta, s>>>(g->n_theta, g->n_lm, g->lmax + 1, nt_pad, tb, g->sep_tb0, F,
-                                                    (const float2 *)g->sep_F0, g->A);
-  note_launch(g, "k_sep_theta", s);
-  return cudaGetLastError();
+// Rows per block of the float64 azimuthal stage: 16 (two blocks or more per SM
+// at the folded columns of one-degree cells), halved while the SMs are short of
+// blocks or the staged rows do not fit; 0: not even two rows fit.
+size_t phi64_smem(const AzFold &f, int rows) { return 4 * (size_t)f.cols * rows * sizeof(double); }
+int phi64_rows(const yy_grid *g) {
+  const AzFold f = az_fold(g);
+  const long long rows = (long long)grid_rows(g) * g->n_theta;
+  int per = 16;
+  while (per > 2 && (phi64_smem(f, per) > 113 * 1024 || (rows + per - 1) / per < 2 * g->sms)) per /= 2;
+  return phi64_smem(f, per) <= 227 * 1024 ? per : 0;
 }
 
 }  // namespace
@@ -463,35 +586,28 @@ cudaError_t separable_prepare(yy_grid *g) {
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = synthesis_separable_prepare(g)) != cudaSuccess) return e;
   }
-  // shared memory of the azimuthal stage (the table and one chunk of rows);
-  // grids too large for it leave the separable analysis unavailable
-  // (the float64 table at l_max 40 on 1-degree cells needs the short chunk)
-  const size_t tail_t = (size_t)(g->n_theta + 1) * sizeof(float2);
+  const AzFold fold = az_fold(g);
+  const int m1 = g->lmax + 1;
+  A((void **)&g->sep_azf, (size_t)m1 * fold.cols * sizeof(double2));
+  if (e != cudaSuccess) return e;
+  k_fold_az<<<(m1 * fold.cols + 255) / 256, 256>>>(m1, nt_pad, fold, g->sep_az, (double2 *)g->sep_azf);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  // float64: the polar stage's sums and the folded rows in shared memory.
+  // fp32: grids whose table and 16 padded rows of a shell fit 227 KB; the others
+  // keep the dense contraction, whose fp32 sums round differently.  (Rows
+  // (shell, j) are counted in 32 bits.)
   g->sep_ok = 0;
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device);
-  for (int q = 0; q < 2; ++q) {
-    const size_t el = q ? sizeof(double) : sizeof(float);
-    if ((size_t)g->n_theta * nt_pad * el + tail_t > 227 * 1024 || theta_smem(g->n_theta, nt_pad, el) > 227 * 1024)
-      continue;
-    const int jc = phi_smem(g, nt_pad, kJC, el) <= 227 * 1024 ? kJC : kJCSmall;
-    const size_t sm = phi_smem(g, nt_pad, jc, el);
-    if (sm > 227 * 1024) continue;
-    const void *kp = q ? (jc == kJC ? (const void *)k_sep_phi<double, kJC> : (const void *)k_sep_phi<double, kJCSmall>)
-                       : (jc == kJC ? (const void *)k_sep_phi<float, kJC> : (const void *)k_sep_phi<float, kJCSmall>);
-    // the attribute belongs to the kernel, not to this grid: always the maximum
-    if ((e = cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024)) != cudaSuccess)
-      return e;
-    int nb = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kp, phi_threads(nt_pad, jc), sm)) != cudaSuccess)
-      return e;
-    g->sep_jc[q] = jc;
-    g->sep_phi_blocks[q] = std::max(nb, 1) * sms;
-    g->sep_ok |= 1 << q;
-  }
+  const bool counted = (long long)grid_rows(g) * g->n_theta <= 1 << 30;
+  const size_t tail_t = (size_t)(g->n_theta + 1) * sizeof(float2), limit = 227 * 1024;
+  if (counted && theta_smem(g->n_theta, nt_pad, sizeof(double)) <= limit && phi64_rows(g) > 0) g->sep_ok |= 2;
+  if (counted && (size_t)g->n_theta * nt_pad * sizeof(float) + tail_t <= limit &&
+      theta_smem(g->n_theta, nt_pad, sizeof(float)) <= limit && (size_t)g->n_phi * (nt_pad + 20) * sizeof(float) <= limit)
+    g->sep_ok |= 1;
   // the attribute belongs to the kernel, not to this grid: always the maximum
-  for (auto f : {(const void *)k_sep_theta<float>, (const void *)k_sep_theta<double>, (const void *)k_sep_theta_partials})
-    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024)) != cudaSuccess)
+  for (auto f : {(const void *)k_sep_phi64, (const void *)k_sep_phi32<2>, (const void *)k_sep_phi32<4>, (const void *)k_sep_theta32<1>, (const void *)k_sep_theta32<2>,
+                 (const void *)k_sep_theta32<4>, (const void *)k_sep_theta64, (const void *)k_sep_theta_partials})
+    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  f == (const void *)k_sep_phi32<2> || f == (const void *)k_sep_phi32<4> ? 64 * 1024 : 227 * 1024)) != cudaSuccess)
       return e;
   return cudaSuccess;
 }
@@ -517,18 +633,50 @@ cudaError_t separable_theta_partials(yy_grid *g, SepThetaPartials a, cudaStream_
 
 cudaError_t separable_theta_f64(yy_grid *g, cudaStream_t s) {
   const int nt_pad = g->sep_nt_pad;
-  const size_t smem_theta = theta_smem(g->n_theta, nt_pad, sizeof(double));
-  k_sep_theta<double><<<grid_rows(g), 256, smem_theta, s>>>(g->n_theta, g->n_lm, g->lmax + 1, nt_pad, g->tbar,
-                                                            g->sep_tb0, g->sep_F, (const float2 *)g->sep_F0, g->A);
-  note_launch(g, "k_sep_theta<double>", s);
+  k_sep_theta64<<<grid_rows(g), theta_threads(g->n_lm, 0), theta_smem(g->n_theta, nt_pad, sizeof(double)), s>>>(g->n_theta, g->n_lm, nt_pad, g->tbar,
+                                                                                          g->sep_F, g->A);
+  note_launch(g, "k_sep_theta64", s);
   return cudaGetLastError();
 }
 
 cudaError_t analysis_separable(yy_grid *g, const double *rho_yin, const double *rho_yang, bool fp64, cudaStream_t s) {
-  if (fp64)
-    return run_separable<double>(g, rho_yin, rho_yang, g->w, g->sep_az, g->tbar, g->sep_F, g->sep_phi_blocks[1], s);
-  return run_separable<float>(g, rho_yin, rho_yang, g->sep_w32, g->sep_az32, g->sep_tb32, (float *)g->sep_F,
-                              g->sep_phi_blocks[0], s);
+  const int nt_pad = g->sep_nt_pad, rows = grid_rows(g) * g->n_theta;
+  if (fp64) {
+    const int per = phi64_rows(g), m1 = g->lmax + 1;
+    const SepPhi64 a = {rows, per, g->n_r, g->n_theta, g->n_phi, m1, nt_pad, az_fold(g), rho_yin, rho_yang, g->w,
+                        (const double2 *)g->sep_azf, g->sep_F};
+    const int threads = std::max(64, (per / kR64 * m1 + 31) / 32 * 32);   // one item per thread (672 at l_max 80)
+    k_sep_phi64<<<(rows + per - 1) / per, threads, phi64_smem(a.fold, per), s>>>(a);
+    note_launch(g, "k_sep_phi64", s);
+    return separable_theta_f64(g, s);
+  }
+  const SepPhi32 a = {g->n_r, g->n_theta, g->n_phi, nt_pad, {rho_yin, rho_yang}, g->sep_w32, g->sep_az32, (float *)g->sep_F,
+                      (float2 *)g->sep_F0};
+  // rows per thread: four, or two where that leaves half of the loading warps without sums
+  const int tg = nt_pad / kTT, R = kRows32 / 2 * tg <= 32 * kLoadWarps ? 2 : 4;
+  const int threads = std::max(32 * kLoadWarps, (kRows32 / R * tg + 31) / 32 * 32);   // one item per thread (352 at l_max 80)
+  const dim3 blocks((unsigned)((g->n_r * g->n_theta + kRows32 - 1) / kRows32), (unsigned)g->n_patch);
+  const size_t table = 2 * (size_t)kPiece * nt_pad * sizeof(float);
+  if (R == 2)
+    k_sep_phi32<2><<<blocks, threads, table, s>>>(a);
+  else
+    k_sep_phi32<4><<<blocks, threads, table, s>>>(a);
+  note_launch(g, "k_sep_phi32", s);
+  // shells per block: as many as leave every SM a block (and fit two blocks per SM)
+  const size_t shell = theta_smem(g->n_theta, nt_pad, sizeof(float));
+  const int shells = grid_rows(g), mode_threads = theta_threads(g->n_lm, 32);
+  auto polar = [&](auto k, int S) {
+    k<<<(shells + S - 1) / S, mode_threads, S * shell, s>>>(shells, g->n_theta, g->n_lm, g->lmax + 1, nt_pad, g->sep_tb32, g->sep_tb0,
+                                                       (const float *)g->sep_F, (const float2 *)g->sep_F0, g->A);
+  };
+  if (shells >= 4 * g->sms && 4 * shell <= 113 * 1024)
+    polar(k_sep_theta32<4>, 4);
+  else if (shells >= 3 * g->sms && 2 * shell <= 113 * 1024)
+    polar(k_sep_theta32<2>, 2);
+  else
+    polar(k_sep_theta32<1>, 1);
+  note_launch(g, "k_sep_theta32", s);
+  return cudaGetLastError();
 }
 
 }  // namespace yy
