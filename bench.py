@@ -372,7 +372,7 @@ def kernel_work(name, spec, n_lm, gradient, prec):
     elif name.startswith("k_sep_theta"):
         w = {"flop": 2.0 * n_r2 * n_lm * half, "flop_kind": "fp64" if "double" in name or prec == "fp64" else "fp32",
              "bytes": rows * (-(-nt // 4) * 4) * f64 + n_r2 * n_lm * f64}
-    elif name == "k_scan_warp":
+    elif name == "k_scan_tile":
         w = {"bytes": n_r2 * n_lm * f64 * 4}
     elif name == "k_rotate_moments":
         s = sum((2 * l + 1) ** 2 for l in range(L + 1))

@@ -55,7 +55,7 @@ static yy_status from_cuda(cudaError_t e) {
 static void free_all(yy_grid *g) {
   if (!g) return;
   double *dbufs[] = {g->r_edges, g->w,      g->tbar,      g->ban,       g->ysyn,  g->ysyn_t,
-                     g->ysyn_p,  g->rot,    g->scan,      g->scan_maps, g->gl_nodes, g->A,
+                     g->ysyn_p,  g->rot,    g->scan,      g->scan_prod, g->scan_maps, g->gl_nodes, g->A,
                      g->Atot,    g->part,   g->cin,       g->Q,         g->stage_rho, g->stage_phi,
                      g->stage_grad};
   for (double *p : dbufs)
@@ -176,6 +176,7 @@ static yy_status create_grid(const double *r_edges, int n_r, int n_theta, int n_
   A((void **)&g->sep_tr, (size_t)(2 * l_max + 1) * n_phi * sizeof(double));
   if (!polar) A((void **)&g->rot32, rotation_table_size(l_max) * sizeof(float));
   A((void **)&g->scan, (size_t)n_r * (l_max + 1) * 8 * sizeof(double));
+  A((void **)&g->scan_prod, (size_t)(l_max + 1) * 32 * 2 * sizeof(double));
   {
     int nc = 1, ch = 1;
     scan_geometry(g, &nc, &ch);
@@ -198,6 +199,7 @@ static yy_status create_grid(const double *r_edges, int n_r, int n_theta, int n_
     gauss_legendre01(n_mu, tg + 2 * n_gl, tg + 2 * n_gl + n_mu);
     e = build_tables(g, gl.data(), n_gl);
   }
+  if (e == cudaSuccess) e = build_scan_products(g);
   if (e == cudaSuccess) e = separable_prepare(g);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
@@ -366,7 +368,7 @@ yy_status yy_potential(yy_grid *g, const double *rho_yin, const double *rho_yang
   g->last_sep_synthesis = sep_synth ? 1 : 0;
   if (e == cudaSuccess && !g->atot_done) e = ozaki ? ozaki_rotate(g, s) : rotate_moments(g, prec == YY_FP64, s);
   // the separable tensor-core synthesis reads the coefficients in fp32 (the scan's copy)
-  if (e == cudaSuccess) e = radial_scan(g, f32 || (sep_synth && !simt && !ozaki), true, s);
+  if (e == cudaSuccess) e = radial_scan(g, f32 || (sep_synth && !simt && !ozaki), s);
   if (e == cudaSuccess && !simt)
     e = sep_synth ? tc_theta(g, prec, grad_yin != nullptr, s) : tc_pack_coefficients(g, prec, s);
   mark(2);

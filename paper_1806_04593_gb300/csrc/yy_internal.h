@@ -38,6 +38,7 @@ struct yy_grid {
   double *rot;         // [sum_l (2l+1)^2]        D^l, other-frame harmonics in own-frame ones
   float *rot32;        // same, rounded to float32
   double *scan;        // [n_r][lmax+1][8]        a_in, b_in, e_out, f_out, output factors
+  double *scan_prod;   // [lmax+1][32][2]         products of a_in and e_out over the scan's chunks
   double *scan_maps;   // [2][chunks][n_lm] x 4   per-chunk affine maps of the scans
   double *gl_nodes;    // GL nodes / weights on [0, 1] for the weight integrals
 
@@ -218,10 +219,10 @@ cudaError_t separable_theta_f64(yy_grid *g, cudaStream_t s);
 
 // Atot = A + D^T A(other patch), float32 products unless fp64 (yy_scan.cu)
 cudaError_t rotate_moments(yy_grid *g, bool fp64, cudaStream_t s);
-// radial scans (yy_scan.cu): Atot -> Q (and Q32 if want_f32); f64_out: output
-// factors applied in float64 (else in fp32, for the reduced-precision forms)
+// radial scans (yy_scan.cu): Atot -> Q (and Q32 if want_f32)
 void scan_geometry(const yy_grid *g, int *nc, int *ch);
-cudaError_t radial_scan(yy_grid *g, bool want_f32, bool f64_out, cudaStream_t s);
+cudaError_t build_scan_products(yy_grid *g);
+cudaError_t radial_scan(yy_grid *g, bool want_f32, cudaStream_t s);
 
 // Grouped solves (yy_tc.cu): every field solved densely in a tensor-core form,
 // one launch per stage over all of them; NOT_SUPPORTED when a field does not
@@ -235,19 +236,19 @@ int tc_group_launches(const TcGroup *grp);
 void tc_group_destroy(TcGroup *grp);
 
 // Grouped radial scans (one launch for many fields, yy_scan.cu): a field's
-// arguments when its scan takes the one-pass warp form (n_r <= 768), the
+// arguments when its scan takes the one-pass form (n_r <= 768), the
 // 128-thread blocks it takes, and the launch over a device table of fields
 // with a block map (per block: field << 24 | the field's own block).
 struct ScanGroupField {
-  int n_patch, n_r, lmax, n_lm, ch;   // ch: radii per lane, 8, 12, 18 or 24
+  int n_patch, n_r, lmax, n_lm, ch;   // ch: radii per thread
   const double *A, *coef;
+  const double2 *prod;
   double *Q;
   float *Q32;
 };
 bool scan_group_field(yy_grid *g, bool want_f32, ScanGroupField *f);
 int scan_group_blocks(const ScanGroupField &f);
-cudaError_t scan_group_launch(const ScanGroupField *fields, const uint32_t *block_map, int blocks, bool f64_out,
-                              cudaStream_t s);
+cudaError_t scan_group_launch(const ScanGroupField *fields, const uint32_t *block_map, int blocks, cudaStream_t s);
 
 // tensor-core path (yy_tc.cu)
 yy_status tc_prepare(yy_grid *g, yy_precision prec);

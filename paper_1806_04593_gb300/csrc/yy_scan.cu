@@ -201,30 +201,43 @@ k_rotate_moments(int n_r, int n_lm, const T *__restrict__ rot, const double *__r
   }
 }
 
-// Radial scans with one warp per (patch, mode): lane L owns the radii
-// [L ch, L ch + ch), ch = ceil(n_r / 32) <= CH, and keeps its moments and inner
-// sums in registers.  Each recurrence is folded into one affine map per lane,
-// the maps are composed across the warp by shuffles (prefix for the inner
-// sums, suffix for the outer ones), and each lane then replays its radii from
-// the composed start value.  Steps past n_r use the identity map, and every
-// load is unconditional (clamped index) so that no load waits behind the
-// float64 chain.  F64OUT: output factors applied in float64; otherwise (the
-// reduced-precision paths, whose packing rounds Q to fp32 anyway) in fp32
-// from fp32 roundings of c_n and d_n, widened back exactly.
-template <int CH, bool F64OUT>
-__device__ __forceinline__ void scan_warp_body(int w, int n_patch, int n_r, int lmax, int n_lm,
+// Radial scans with one thread per (patch, mode, chunk of radii): 32 chunks of
+// ch = ceil(n_r / 32) <= CH radii, held in registers.  Each recurrence is folded
+// into one affine map per chunk, the maps are composed across the chunks in
+// shared memory (prefix for the inner sums, suffix for the outer ones, both in
+// the same five steps), and each thread then replays its radii from the composed
+// start value.  Steps past n_r use the identity map, and every load is
+// unconditional (clamped index) so that no load waits behind the float64 chain.
+//
+// A block takes four neighbouring modes: their values of a radius are one 32-byte
+// sector of A and of each output.  (With a warp per mode, lanes on the radii,
+// every 8-byte access took a sector of its own: 39 us on the 1-degree grid at
+// l_max 25, against 31.)  The float64 pipe is the next bound: 11 operations
+// per point; the products of a_n and e_n over a chunk come from a table, and the
+// terms b_n A_n and f_n A_(n+1) stay in registers between the fold and the replay.
+constexpr int kScanModes = 4, kScanThreads = 32 * kScanModes;
+struct ScanShared {
+  double2 m[2][2][kScanThreads];   // [buffer][inner, outer]: (product, offset) of each thread's map
+};
+
+template <int CH>
+__device__ __forceinline__ void scan_tile_body(ScanShared &sm, int block, int n_patch, int n_r, int lmax, int n_lm,
                                                const double *__restrict__ A, const double *__restrict__ coef,
-                                               double *__restrict__ Q, float *__restrict__ Q32) {
-  const int lane = threadIdx.x & 31;
-  if (w >= n_patch * n_lm) return;
-  const int p = w / n_lm, j = w % n_lm;
+                                               const double2 *__restrict__ prod, double *__restrict__ Q,
+                                               float *__restrict__ Q32) {
+  const int tid = threadIdx.x, groups = (n_lm + kScanModes - 1) / kScanModes;
+  const int p = block / groups, j0 = block % groups * kScanModes + (tid & (kScanModes - 1));
+  const int chunk = tid / kScanModes;
+  const bool mode_ok = j0 < n_lm;
+  const int j = mode_ok ? j0 : n_lm - 1;
   const int l = mode_degree(j);
   const int L1 = lmax + 1;
   const int ch = (n_r + 31) / 32;
-  const int n0 = lane * ch;
+  const int n0 = chunk * ch;
   const double *Ap = A + (size_t)p * n_r * n_lm + j;
   const double *cl = coef + (size_t)l * 8;          // + n L1 8
   const size_t cstride = (size_t)L1 * 8;
+  // av: A_n, then f_n A_(n+1); cv: b_n A_n, then c_n
   double av[CH], cv[CH];
 #pragma unroll
   for (int i = 0; i < CH; ++i) {
@@ -232,149 +245,164 @@ __device__ __forceinline__ void scan_warp_body(int w, int n_patch, int n_r, int 
     const double v = Ap[(size_t)n * n_lm];
     av[i] = (i < ch && n0 + i < n_r) ? v : 0.0;
   }
-  // A_{n0 + ch}: first moment of the next lane's radii
-  double a_next = __shfl_down_sync(0xffffffffu, av[0], 1);
-  if (lane == 31) a_next = 0.0;
+  double a_next = Ap[(size_t)min(n0 + ch, n_r - 1) * n_lm];   // first moment of the next chunk
+  if (n0 + ch >= n_r) a_next = 0.0;
+  const double2 pr = prod[l * 32 + chunk];
 
-  // inner sums c_n = a_n c_{n-1} + b_n A_n
-  double al = 1.0, be = 0.0;
+  // folds: c_n = a_n c_{n-1} + b_n A_n upwards, d_n = e_n d_{n+1} + f_n A_{n+1} downwards (d_{n_r - 1} = 0)
+  double bi = 0.0, bo = 0.0;
 #pragma unroll
   for (int i = 0; i < CH; ++i) {
     const bool ok = i < ch && n0 + i < n_r;
     const double2 k01 = *(const double2 *)(cl + (size_t)min(n0 + i, n_r - 1) * cstride);
     const double a = ok ? k01.x : 1.0, b = ok ? k01.y : 0.0;
-    be = fma(a, be, b * av[i]);
-    al *= a;
+    cv[i] = b * av[i];
+    bi = fma(a, bi, cv[i]);
   }
 #pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const double ao = __shfl_up_sync(0xffffffffu, al, off);
-    const double bo = __shfl_up_sync(0xffffffffu, be, off);
-    if (lane >= off) {
-      be = fma(al, bo, be);
-      al *= ao;
-    }
-  }
-  double x = __shfl_up_sync(0xffffffffu, be, 1);
-  if (lane == 0) x = 0.0;
-#pragma unroll
-  for (int i = 0; i < CH; ++i) {
+  for (int i = 0; i < CH; ++i) {   // av[i] <- f_n A_(n+1): upwards, so that av[i + 1] is still A
     const bool ok = i < ch && n0 + i < n_r;
-    const double2 k01 = *(const double2 *)(cl + (size_t)min(n0 + i, n_r - 1) * cstride);
-    const double a = ok ? k01.x : 1.0, b = ok ? k01.y : 0.0;
-    x = fma(a, x, b * av[i]);
-    cv[i] = x;
+    const double an = (i + 1 < ch) ? av[i + 1 < CH ? i + 1 : i] : a_next;   // 0 past n_r
+    const double f = ok ? cl[(size_t)min(n0 + i, n_r - 1) * cstride + 3] : 0.0;
+    av[i] = f * an;
   }
-
-  // outer sums d_n = e_n d_{n+1} + f_n A_{n+1}, d_{n_r - 1} = 0
-  al = 1.0;
-  be = 0.0;
 #pragma unroll
   for (int i = CH - 1; i >= 0; --i) {
     const bool ok = i < ch && n0 + i < n_r;
-    const double an = (i + 1 < ch) ? av[i + 1 < CH ? i + 1 : i] : a_next;   // 0 past n_r
-    const double2 k23 = *(const double2 *)(cl + (size_t)min(n0 + i, n_r - 1) * cstride + 2);
-    const double e = ok ? k23.x : 1.0, f = ok ? k23.y : 0.0;
-    be = fma(e, be, f * an);
-    al *= e;
+    const double e = ok ? cl[(size_t)min(n0 + i, n_r - 1) * cstride + 2] : 1.0;
+    bo = fma(e, bo, av[i]);
   }
+  // compose: after the steps bi / bo map 0 across this chunk and all before / after it
+  double ai = pr.x, ao = pr.y;
 #pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const double ao = __shfl_down_sync(0xffffffffu, al, off);
-    const double bo = __shfl_down_sync(0xffffffffu, be, off);
-    if (lane + off < 32) {
-      be = fma(al, bo, be);
-      al *= ao;
+  for (int step = 0; step < 5; ++step) {
+    const int off = 1 << step, at = off * kScanModes;
+    double2 (*m)[kScanThreads] = sm.m[step & 1];
+    m[0][tid] = make_double2(ai, bi);
+    m[1][tid] = make_double2(ao, bo);
+    __syncthreads();
+    if (chunk >= off) {
+      const double2 q = m[0][tid - at];
+      bi = fma(ai, q.y, bi);
+      ai *= q.x;
+    }
+    if (chunk + off < 32) {
+      const double2 q = m[1][tid + at];
+      bo = fma(ao, q.y, bo);
+      ao *= q.x;
     }
   }
-  double y = __shfl_down_sync(0xffffffffu, be, 1);
-  if (lane == 31) y = 0.0;
+  sm.m[1][0][tid].y = bi;
+  sm.m[1][1][tid].y = bo;
+  __syncthreads();
+  double x = chunk > 0 ? sm.m[1][0][tid - kScanModes].y : 0.0;
+  double y = chunk < 31 ? sm.m[1][1][tid + kScanModes].y : 0.0;
+#pragma unroll
+  for (int i = 0; i < CH; ++i) {
+    const bool ok = i < ch && n0 + i < n_r;
+    const double a = ok ? cl[(size_t)min(n0 + i, n_r - 1) * cstride] : 1.0;
+    x = fma(a, x, cv[i]);
+    cv[i] = x;
+  }
   const size_t qsz = (size_t)n_patch * n_r * n_lm;
 #pragma unroll
   for (int i = CH - 1; i >= 0; --i) {
     const bool ok = i < ch && n0 + i < n_r;
-    const double an = (i + 1 < ch) ? av[i + 1 < CH ? i + 1 : i] : a_next;
     const double *k = cl + (size_t)min(n0 + i, n_r - 1) * cstride;
-    const double2 k23 = *(const double2 *)(k + 2);
-    const double e = ok ? k23.x : 1.0, f = ok ? k23.y : 0.0;
-    y = fma(e, y, f * an);
-    if (!ok) continue;
+    const double e = ok ? k[2] : 1.0;
+    y = fma(e, y, av[i]);
+    if (!ok || !mode_ok) continue;
     const size_t o = ((size_t)p * n_r + n0 + i) * n_lm + j;
     const double cn = cv[i];
-    if constexpr (F64OUT) {
-      const double2 k45 = *(const double2 *)(k + 4);
-      const double2 k67 = *(const double2 *)(k + 6);
-      const double sum = cn + y;
-      const double q = k45.x * sum, qr = fma(k45.y, cn, k67.x * y), qt = k67.y * sum;
-      Q[o] = q;
-      Q[qsz + o] = qr;
-      Q[2 * qsz + o] = qt;
-      if (Q32 != nullptr) {
-        Q32[o] = to_f32(q);
-        Q32[qsz + o] = to_f32(qr);
-        Q32[2 * qsz + o] = to_f32(qt);
-      }
-    } else {
-      const double2 k45 = *(const double2 *)(k + 4);
-      const double2 k67 = *(const double2 *)(k + 6);
-      const float cf = to_f32(cn), yf = to_f32(y);
-      const float sum = cf + yf;
-      Q[o] = to_f64(to_f32(k45.x) * sum);
-      Q[qsz + o] = to_f64(fmaf(to_f32(k45.y), cf, to_f32(k67.x) * yf));
-      Q[2 * qsz + o] = to_f64(to_f32(k67.y) * sum);
+    const double2 k45 = *(const double2 *)(k + 4);
+    const double2 k67 = *(const double2 *)(k + 6);
+    const double sum = cn + y;
+    const double q = k45.x * sum, qr = fma(k45.y, cn, k67.x * y), qt = k67.y * sum;
+    Q[o] = q;
+    Q[qsz + o] = qr;
+    Q[2 * qsz + o] = qt;
+    if (Q32 != nullptr) {
+      Q32[o] = to_f32(q);
+      Q32[qsz + o] = to_f32(qr);
+      Q32[2 * qsz + o] = to_f32(qt);
     }
   }
 }
 
-template <int CH, bool F64OUT>
-__global__ void __launch_bounds__(128, 3)
-k_scan_warp(int n_patch, int n_r, int lmax, int n_lm, const double *__restrict__ A, const double *__restrict__ coef,
-            double *__restrict__ Q, float *__restrict__ Q32) {
-  scan_warp_body<CH, F64OUT>((int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), n_patch, n_r, lmax, n_lm, A, coef,
-                             Q, Q32);
+// the register forms: radii per thread
+#define YY_SCAN_FORMS(X) X(2) X(4) X(8) X(12) X(18) X(24)
+int scan_form(int n_r) {
+#define YY_SCAN_PICK(CH) \
+  if (n_r <= 32 * CH) return CH;
+  YY_SCAN_FORMS(YY_SCAN_PICK)
+#undef YY_SCAN_PICK
+  return 0;
+}
+
+template <int CH>
+__global__ void __launch_bounds__(kScanThreads, 3)
+k_scan_tile(int n_patch, int n_r, int lmax, int n_lm, const double *__restrict__ A, const double *__restrict__ coef,
+            const double2 *__restrict__ prod, double *__restrict__ Q, float *__restrict__ Q32) {
+  __shared__ ScanShared sm;
+  scan_tile_body<CH>(sm, (int)blockIdx.x, n_patch, n_r, lmax, n_lm, A, coef, prod, Q, Q32);
+}
+
+// products of a_n and of e_n over each of the 32 chunks, in the order of the folds
+__global__ void k_scan_products(int n_r, int lmax, const double *__restrict__ coef, double2 *__restrict__ prod) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= (lmax + 1) * 32) return;
+  const int l = e / 32, ch = (n_r + 31) / 32, n0 = e % 32 * ch;
+  double a = 1.0, b = 1.0;
+  for (int i = 0; i < ch; ++i)
+    if (n0 + i < n_r) a *= coef[((size_t)(n0 + i) * (lmax + 1) + l) * 8];
+  for (int i = ch - 1; i >= 0; --i)
+    if (n0 + i < n_r) b *= coef[((size_t)(n0 + i) * (lmax + 1) + l) * 8 + 2];
+  prod[e] = make_double2(a, b);
 }
 
 // Many fields' scans in one launch: block b scans for field block_map[b] >> 24
-// (its block block_map[b] & 0xFFFFFF, four (patch, mode) warps each), in the
-// register form the field's radial grid needs (ch = 8, 12, 18 or 24 radii per lane).
-template <bool F64OUT>
-__global__ void __launch_bounds__(128, 3)
+// (its block block_map[b] & 0xFFFFFF), in the register form the field's radial
+// grid needs.
+__global__ void __launch_bounds__(kScanThreads, 3)
 k_scan_group(const ScanGroupField *__restrict__ fields, const uint32_t *__restrict__ block_map) {
+  __shared__ ScanShared sm;
   const uint32_t m = block_map[blockIdx.x];
   const ScanGroupField f = fields[m >> 24];
-  const int w = (int)(m & 0xFFFFFFu) * 4 + (int)(threadIdx.x >> 5);
+  const int b = (int)(m & 0xFFFFFFu);
   switch (f.ch) {
-    case 8: scan_warp_body<8, F64OUT>(w, f.n_patch, f.n_r, f.lmax, f.n_lm, f.A, f.coef, f.Q, f.Q32); break;
-    case 12: scan_warp_body<12, F64OUT>(w, f.n_patch, f.n_r, f.lmax, f.n_lm, f.A, f.coef, f.Q, f.Q32); break;
-    case 18: scan_warp_body<18, F64OUT>(w, f.n_patch, f.n_r, f.lmax, f.n_lm, f.A, f.coef, f.Q, f.Q32); break;
-    default: scan_warp_body<24, F64OUT>(w, f.n_patch, f.n_r, f.lmax, f.n_lm, f.A, f.coef, f.Q, f.Q32); break;
+#define YY_SCAN_CASE(CH) \
+  case CH: scan_tile_body<CH>(sm, b, f.n_patch, f.n_r, f.lmax, f.n_lm, f.A, f.coef, f.prod, f.Q, f.Q32); break;
+    YY_SCAN_FORMS(YY_SCAN_CASE)
+#undef YY_SCAN_CASE
   }
 }
 
 }  // namespace
 
 bool scan_group_field(yy_grid *g, bool want_f32, ScanGroupField *f) {
-  if (g->n_r > 32 * 24) return false;
+  f->ch = scan_form(g->n_r);
+  if (f->ch == 0) return false;
   f->n_patch = g->n_patch;
   f->n_r = g->n_r;
   f->lmax = g->lmax;
   f->n_lm = g->n_lm;
-  f->ch = g->n_r <= 32 * 8 ? 8 : g->n_r <= 32 * 12 ? 12 : g->n_r <= 32 * 18 ? 18 : 24;
   f->A = moments_total(g);
   f->coef = g->scan;
+  f->prod = (const double2 *)g->scan_prod;
   f->Q = g->Q;
   f->Q32 = want_f32 ? g->Q32 : nullptr;
   return true;
 }
 
-int scan_group_blocks(const ScanGroupField &f) { return (f.n_patch * f.n_lm + 3) / 4; }
+int scan_group_blocks(const ScanGroupField &f) { return f.n_patch * ((f.n_lm + kScanModes - 1) / kScanModes); }
 
-cudaError_t scan_group_launch(const ScanGroupField *fields, const uint32_t *block_map, int blocks, bool f64_out,
-                              cudaStream_t st) {
-  if (f64_out)
-    k_scan_group<true><<<blocks, 128, 0, st>>>(fields, block_map);
-  else
-    k_scan_group<false><<<blocks, 128, 0, st>>>(fields, block_map);
+cudaError_t scan_group_launch(const ScanGroupField *fields, const uint32_t *block_map, int blocks, cudaStream_t st) {
+  k_scan_group<<<blocks, kScanThreads, 0, st>>>(fields, block_map);
+  return cudaGetLastError();
+}
+
+cudaError_t build_scan_products(yy_grid *g) {
+  k_scan_products<<<g->lmax + 1, 32>>>(g->n_r, g->lmax, g->scan, (double2 *)g->scan_prod);
   return cudaGetLastError();
 }
 
@@ -406,27 +434,19 @@ void scan_geometry(const yy_grid *g, int *nc, int *ch) {
   *nc = (g->n_r + *ch - 1) / *ch;
 }
 
-cudaError_t radial_scan(yy_grid *g, bool want_f32, bool f64_out, cudaStream_t st) {
+cudaError_t radial_scan(yy_grid *g, bool want_f32, cudaStream_t st) {
   float *q32 = want_f32 ? g->Q32 : nullptr;
-  // one warp per block: the SMs get the warps in equal numbers (with four per
-  // block, 1352 warps left some SMs three blocks and most two, and the
-  // three-block SMs set the time)
-  const unsigned wblocks = (unsigned)(g->n_patch * g->n_lm);
   const double *At = moments_total(g);
-  if (g->n_r <= 32 * 24) {
-#define YY_SCAN_WARP(CH)                                                                               \
-  (f64_out ? (k_scan_warp<CH, true><<<wblocks, 32, 0, st>>>(g->n_patch, g->n_r, g->lmax, g->n_lm, At, g->scan, g->Q, q32), 0) \
-           : (k_scan_warp<CH, false><<<wblocks, 32, 0, st>>>(g->n_patch, g->n_r, g->lmax, g->n_lm, At, g->scan, g->Q, q32), 0))
-    if (g->n_r <= 32 * 8)
-      YY_SCAN_WARP(8);
-    else if (g->n_r <= 32 * 12)
-      YY_SCAN_WARP(12);
-    else if (g->n_r <= 32 * 18)
-      YY_SCAN_WARP(18);
-    else
-      YY_SCAN_WARP(24);
-#undef YY_SCAN_WARP
-    note_launch(g, "k_scan_warp", st);
+  const int form = scan_form(g->n_r);
+  if (form > 0) {
+    const unsigned blocks = (unsigned)(g->n_patch * ((g->n_lm + kScanModes - 1) / kScanModes));
+    switch (form) {
+#define YY_SCAN_CASE(CH) \
+  case CH: k_scan_tile<CH><<<blocks, kScanThreads, 0, st>>>(g->n_patch, g->n_r, g->lmax, g->n_lm, At, g->scan, (const double2 *)g->scan_prod, g->Q, q32); break;
+      YY_SCAN_FORMS(YY_SCAN_CASE)
+#undef YY_SCAN_CASE
+    }
+    note_launch(g, "k_scan_tile", st);
     return cudaGetLastError();
   }
   // long radial grids: chunks spread over warps, two passes

@@ -3785,7 +3785,7 @@ static cudaError_t group_run(const TcGroup *G, cudaStream_t s) {
   if ((e = cudaLaunchKernelEx(&cfg, k_tc_pair<F, 0, true>, none, G->an_top)) != cudaSuccess) return e;
   k_reduce_rotate_group<<<G->rr_nblocks, 256, 0, s>>>(G->rr, G->rr_map);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = scan_group_launch(G->sc, G->sc_map, G->sc_nblocks, true, s)) != cudaSuccess) return e;
+  if ((e = scan_group_launch(G->sc, G->sc_map, G->sc_nblocks, s)) != cudaSuccess) return e;
   k_pack_group<F, 32><<<G->cf_nblocks, 256, 0, s>>>(G->cf_jobs, G->cf_map, G->cf_class);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   cfg = pair_config(G->sy_pairs, G->sy_smem, s, attr);
