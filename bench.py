@@ -57,7 +57,7 @@ FORMS = ("fp64_ozaki", "fp16x2", "bf16x3", "tf32", "fp32", "fp64")
 DTYPE = {"fp64": "f64", "fp32": "f32", "fp16x2": "fp16x2 (fp32 accumulate, f64 scans)",
          "bf16x3": "bf16x3 (fp32 accumulate, f64 scans)", "tf32": "tf32 (fp32 accumulate, f64 scans)",
          "fp64_ozaki": "f64"}
-PRODUCTS = {"fp16x2": 3, "bf16x3": 6, "tf32": 1}
+PRODUCTS = {"fp16x2": 3, "bf16x3": 6, "tf32": 1, "ozaki_synth": 15}
 
 # DRAM bytes (read + write) per launch of a kernel, from one ncu capture of
 # this workload (profiles/), valid only while the kernel sources are the ones
@@ -345,10 +345,10 @@ def kernel_work(name, spec, n_lm, gradient, prec):
     f64 = 8
     out_bytes = J * n_r2 * spec.n_ang * f64
     w = {}
-    if name.startswith("k_tc_pair<FormOzaki,3>/synthesis") or name == "k_oz_synth":
-        k_pad = -(-nt // 32) * 32
-        w = {"flop": 2.0 * rows * spec.n_phi * nt * J, "flop_kind": "tensor", "products": "ozaki",
-             "bytes": out_bytes + J * rows * k_pad * 6 * 2}
+    if name == "k_oz_synth":   # half of the longitudes with half of the slots twice: the folded sums
+        gk = 64 if L <= 31 else 128
+        w = {"flop": rows * spec.n_phi * nt * J, "flop_kind": "tensor", "products": "ozaki_synth",
+             "bytes": out_bytes + J * rows * gk * 5 * 2}
     elif name.startswith("k_tc_pair<FormOzaki,3>/analysis") or name == "k_oz_analysis":
         k_pad = -(-spec.n_phi // 64) * 64
         w = {"flop": 2.0 * rows * spec.n_phi * nt, "flop_kind": "tensor", "products": "ozaki",
@@ -357,9 +357,9 @@ def kernel_work(name, spec, n_lm, gradient, prec):
         # float-float multiply-adds of Phi, g_r and g_theta (g_phi is formed
         # from Phi's sums), one per term and mirrored row pair
         ffma = sum(L + 1 - (t + 1) // 2 for t in range(nt)) * min(J, 3)
-        gk = 64 if nt <= 64 else 128
+        gk = 64 if L <= 31 else 128
         w = {"flop": 2.0 * n_r2 * half * ffma, "flop_kind": "ff",
-             "bytes": J * rows * gk * 6 * 2 + min(J, 3) * n_r2 * n_lm * f64}
+             "bytes": J * rows * gk * 5 * 2 + min(J, 3) * n_r2 * n_lm * f64}
     elif name == "k_q_ff":
         w = {"bytes": 2 * min(J, 3) * n_r2 * n_lm * f64}
     elif name == "k_rhow_ozaki":
@@ -369,8 +369,9 @@ def kernel_work(name, spec, n_lm, gradient, prec):
         nt_pad = -(-nt // 4) * 4
         w = {"flop": 2.0 * n_r2 * n_lm * half, "flop_kind": "ff",
              "bytes": rows * nt_pad * f64 + n_r2 * n_lm * f64}
-    elif name.startswith("k_sep_theta"):
-        w = {"flop": 2.0 * n_r2 * n_lm * half, "flop_kind": "fp64" if "double" in name or prec == "fp64" else "fp32",
+    elif name in ("k_sep_theta64", "k_sep_theta32"):
+        w = {"flop": 2.0 * n_r2 * n_lm * (half if name == "k_sep_theta64" else spec.n_theta),
+             "flop_kind": "fp64" if name == "k_sep_theta64" else "fp32",
              "bytes": rows * (-(-nt // 4) * 4) * f64 + n_r2 * n_lm * f64}
     elif name == "k_scan_tile":
         w = {"bytes": n_r2 * n_lm * f64 * 4}
@@ -384,12 +385,22 @@ def kernel_work(name, spec, n_lm, gradient, prec):
         w = {"flop": 2.0 * n_r2 * n_lm * spec.n_ang, "flop_kind": "tensor", "products": prec}
     elif name == "k_pack_stream":
         w = {"bytes": n_r2 * spec.n_ang * f64 + n_r2 * spec.n_ang * {"fp16x2": 4, "bf16x3": 6, "tf32": 4}.get(prec, 4)}
-    elif name == "k_sep_synth":
-        w = {"flop": J * (2.0 * rows * n_lm + 2.0 * rows * spec.n_phi * nt),
-             "flop_kind": "fp64" if prec == "fp64" else "fp32", "bytes": out_bytes}
-    elif name == "k_sep_phi":
-        w = {"flop": 2.0 * rows * spec.n_phi * nt, "flop_kind": "fp64" if prec == "fp64" else "fp32",
-             "bytes": n_r2 * spec.n_ang * f64}
+    elif name in ("k_synth_f64", "k_phi32", "k_theta32", "k_sep_phi64", "k_sep_phi32"):
+        # separable sums; the float64 kernels run them over the cells folded by
+        # their symmetries: the operations of the folded sums
+        kind = "fp64" if name.endswith("64") else "fp32"
+        cols = spec.n_phi
+        if kind == "fp64":
+            whole = math.pi / ((1.5 * math.pi + 2 * spec.delta_phi) / spec.n_phi)
+            cols = spec.n_phi / 3 if abs(whole - round(whole)) < 1e-9 else spec.n_phi / 2
+        if name.startswith("k_sep_phi"):
+            w = {"flop": 2.0 * rows * cols * nt, "bytes": n_r2 * spec.n_ang * f64}
+        elif name == "k_theta32":
+            w = {"flop": J * 2.0 * rows * n_lm, "bytes": J * rows * nt * 4}
+        else:
+            theta = 0.0 if name == "k_phi32" else min(J, 3) * 2.0 * n_r2 * half * n_lm
+            w = {"flop": theta + J * 2.0 * rows * cols * nt, "bytes": out_bytes}
+        w["flop_kind"] = kind
     return w
 
 
@@ -403,7 +414,7 @@ def roofline_of(name, ms, spec, n_lm, gradient, prec, peaks, ozaki_products):
         kind = w["flop_kind"]
         if kind == "tensor":
             prods = ozaki_products if w.get("products") == "ozaki" else PRODUCTS.get(w.get("products"), 1)
-            ratio = 0.5 if prec == "tf32" and w.get("products") != "ozaki" else 1.0
+            ratio = 0.5 if prec == "tf32" and not w.get("products", "").startswith("ozaki") else 1.0
             hw = w["flop"] * prods
             cands.append({"bound": "tensor", "achieved": hw / s / 1e12, "peak": peaks["bf16_tflops"] * ratio,
                           "unit": "TFLOP/s",
@@ -639,8 +650,8 @@ def run_ours(args, dist):
                    "n_r": spec.n_r, "n_theta": spec.n_theta, "n_phi": spec.n_phi, "l_max": spec.lmax,
                    "gradient": gradient, "precision": prec, "parallelism": f"replicas x{dist.world}",
                    "l2": "L2 flushed (252 MB write) before every timed step"},
-        "precision_note": ("float64 results: the azimuthal stages of analysis and synthesis as bf16 digit "
-                           "products on tcgen05 (48-bit operands, exact per level, rounded once to float64), "
+        "precision_note": ("float64 results: the azimuthal stages of analysis (bf16) and synthesis (fp16) as "
+                           "digit products on tcgen05 (48- and 50-bit operands, rounded once to float64), "
                            "the polar stages in float-float arithmetic on the fp32 pipe (about 48 bits), "
                            "combination and radial scans in float64") if prec == "fp64_ozaki" else None,
         "gemm_tflops": grid.flops(gradient) / (dev_s_max / args.steps) / 1e12,

@@ -2104,13 +2104,11 @@ cudaError_t tc_synthesis(yy_grid *g, yy_precision prec, double *py, double *pg, 
 // ---------------------------------------------------------------------------
 //
 // The separable synthesis with its azimuthal stage on the tensor cores at
-// float64 accuracy: a float64 polar stage forms G[t] per output row (shell,
-// j) and field and cuts each row into FormOzaki's six fixed-point slices
-// under the row's power-of-two scale; k_tc_pair (out_mode 3) contracts them
-// with the slices of the trig table (scaled by 1/2: cos 0 = 1 must lie inside
-// (-1, 1)) over K = 2 l_max + 1 <= 127 (rows of 64 or 128 slots, one fill),
-// exact per level, and rounds each value once.  The monopole slot t = 0 is
-// part of the contraction: it is exact too.
+// float64 accuracy: a float-float polar stage forms G[t] per output row (shell,
+// j) and field and cuts each row into FormOzSynth's five digits under the row's
+// power-of-two scale; k_oz_synth contracts them with the digits of the trig
+// table, the cos and the sin slots apart over half of the longitudes, and rounds
+// each value once.  The monopole slot is part of the contraction: it is exact too.
 
 // Balanced base-256 digits of X < 2^48 (most significant first): each
 // digit taken in [-127, 128] with a carry into the next; the top one is at
@@ -2373,20 +2371,9 @@ __device__ __forceinline__ void ff_fma_x2(ulonglong2 q, ffx2 qn_hi, ulonglong2 p
 // 127 (each in [-127, 128], the carries done by the addition) and the top
 // one is Y >> 40.  Each digit comes out as the fp32 bit pattern of its
 // value, whose upper half is the bf16 pattern (an integer below 2^8 in
-// magnitude has sixteen zero low bits), most significant digit first:
-// x_digit_pre gives the patterns of 2^23 + digit + 127 (the top one's of
-// 2^23 + digit), from which one fp32 subtraction each leaves the digit.
-__device__ __forceinline__ void x_digit_pre(unsigned long long X, uint32_t (&pre)[6]) {
-  const unsigned long long Y = X + 0x7F7F7F7F7Full;
-  const uint32_t ylo = (uint32_t)Y, yhi = (uint32_t)(Y >> 32);
-  pre[0] = 0x4B000000u | (yhi >> 8);
-  pre[1] = __byte_perm(yhi, 0x4B000000u, 0x7540);
-  pre[2] = __byte_perm(ylo, 0x4B000000u, 0x7543);
-  pre[3] = __byte_perm(ylo, 0x4B000000u, 0x7542);
-  pre[4] = __byte_perm(ylo, 0x4B000000u, 0x7541);
-  pre[5] = __byte_perm(ylo, 0x4B000000u, 0x7540);
-}
-
+// magnitude has sixteen zero low bits), most significant digit first: the
+// patterns of 2^23 + digit + 127 (the top one's of 2^23 + digit), from which
+// one fp32 subtraction each leaves the digit.
 __device__ __forceinline__ void x_digit_bits(unsigned long long X, uint32_t (&bits)[6]) {
   const unsigned long long Y = X + 0x7F7F7F7F7Full;
   const uint32_t ylo = (uint32_t)Y, yhi = (uint32_t)(Y >> 32);
@@ -2400,12 +2387,23 @@ __device__ __forceinline__ void x_digit_bits(unsigned long long X, uint32_t (&bi
 
 __device__ __forceinline__ ffx2 x2_pack(uint32_t lo, uint32_t hi) { return ((ffx2)hi << 32) | lo; }
 
-// The digit patterns (x_digit_pre) of two float-float values (hi, lo) at
-// once, both halves of each packed register: X = round(|value| 2^K), 2^K =
-// p1 p2 the row's scale, as described below for ff_row.  The scalings by
-// 2^-32 and 2^-16 are exact (or leave a sum of 1.5 2^23 that rounds to it
-// either way), so each multiply-and-add is one fused operation.
-__device__ __forceinline__ void ff_digit_pre_x2(ffx2 hi, ffx2 lo, ffx2 p1, ffx2 p2, uint32_t (&pre)[2][6]) {
+// The balanced base-1024 digits (FormOzSynth) of two float-float values (hi, lo)
+// at once, both halves of each packed register: X = round(|value| 2^K) <= 2^49,
+// 2^K = p1 p2 the row's scale, on the fp32 pipe, 16 bits at a time: A =
+// |hi| 2^K and B = +-lo 2^K (exact power-of-two scalings), T2 = rint(A 2^-32), T1 =
+// rint((A - T2 2^32) 2^-16), T1' = rint(B 2^-16) (|B| <= 2^24; the remainders
+// exact by fused multiply-add), T0 = rint(A's remainder + B's), each rint by adding
+// and removing 1.5 2^23 (whose bit pattern then holds the integer), X = T2 2^32 +
+// (T1 + T1') 2^16 + T0.  The last sum rounds only where the remainders span more
+// than 24 bits, so X is the nearest integer except near a tie.  The scalings by 2^-32 and 2^-16 are
+// exact (or leave a sum of 1.5 2^23 that rounds to it either way), so each
+// multiply-and-add is one fused operation.  Then the digits in one step: with
+// Y = X + 511 (1 + 2^10 + 2^20 + 2^30), the low four digits are Y's 10-bit
+// fields less 511 (each in [-511, 512], the carries done by the addition) and
+// the top one is Y >> 40.  A field f is the fp16 pattern 0x6400 | f of 1024 + f, from
+// which one exact fp16 subtraction leaves the digit: w[s] = digit s of both values
+// as fp16 patterns, most significant first, both with the sign bits `sm`.
+__device__ __forceinline__ void ff_digits_x2(ffx2 hi, ffx2 lo, ffx2 p1, ffx2 p2, uint32_t (&w)[5]) {
   constexpr ffx2 kSign = 0x8000000080000000ull;
   constexpr ffx2 kM = 0x4B4000004B400000ull;             // 1.5 2^23 in both halves
   constexpr uint32_t kMBits = 0x4B400000u;
@@ -2416,56 +2414,47 @@ __device__ __forceinline__ void ff_digit_pre_x2(ffx2 hi, ffx2 lo, ffx2 p1, ffx2 
   const ffx2 R1 = fma_x2(sub_x2(s2, kM), 0xCF800000CF800000ull, A);                  // A - T2 2^32
   const ffx2 s1 = fma_x2(R1, 0x3780000037800000ull, kM);                             // R1 2^-16 + M
   const ffx2 R2 = fma_x2(sub_x2(s1, kM), 0xC7800000C7800000ull, R1);                 // R1 - T1 2^16
-  const ffx2 s0 = add_x2(add_x2(R2, B), kM);
+  const ffx2 sb = fma_x2(B, 0x3780000037800000ull, kM);                              // B 2^-16 + M
+  const ffx2 B0 = fma_x2(sub_x2(sb, kM), 0xC7800000C7800000ull, B);                  // B - T1' 2^16
+  const ffx2 s0 = add_x2(add_x2(R2, B0), kM);
+  uint32_t yl[2], yh[2];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const long long X = ((long long)(int)((uint32_t)(s2 >> (32 * h)) - kMBits) << 32) +
-                        ((long long)(int)((uint32_t)(s1 >> (32 * h)) - kMBits) << 16) +
+                        ((long long)(int)((uint32_t)(s1 >> (32 * h)) + (uint32_t)(sb >> (32 * h)) - 2u * kMBits) << 16) +
                         (long long)(int)((uint32_t)(s0 >> (32 * h)) - kMBits);
-    x_digit_pre((unsigned long long)X, pre[h]);
+    const unsigned long long Y = (unsigned long long)X + 511ull * (1ull + (1ull << 10) + (1ull << 20) + (1ull << 30));
+    yl[h] = (uint32_t)Y;
+    yh[h] = (uint32_t)(Y >> 32);
+  }
+  const uint32_t sm = ((uint32_t)hi >> 31 << 15) | ((uint32_t)(hi >> 32) & 0x80000000u);
+  const uint32_t f[5] = {__byte_perm(yh[0] >> 8, yh[1] >> 8, 0x5410),
+                         __byte_perm(__funnelshift_r(yl[0], yh[0], 30), __funnelshift_r(yl[1], yh[1], 30), 0x5410),
+                         __byte_perm(yl[0] >> 20, yl[1] >> 20, 0x5410), __byte_perm(yl[0] >> 10, yl[1] >> 10, 0x5410),
+                         __byte_perm(yl[0], yl[1], 0x5410)};
+#pragma unroll
+  for (int s = 0; s < 5; ++s) {
+    const uint32_t x = (f[s] & 0x03FF03FFu) | 0x64006400u;
+    const __half2 d = __hsub2(*reinterpret_cast<const __half2 *>(&x), __float2half2_rn(s == 0 ? 1024.f : 1535.f));
+    w[s] = *reinterpret_cast<const uint32_t *>(&d) ^ sm;
   }
 }
 
-// the row scale of ff_row: 2^K with K = 48 - e as two normal fp32 factors
+// the row scale of ff_row: 2^K with K = 50 - e as two normal fp32 factors
 __device__ __forceinline__ void ff_row_scale(int e, float &p1, float &p2) {
-  const int K = 48 - e, K1 = K >> 1, K2 = K - K1;
+  const int K = 50 - e, K1 = K >> 1, K2 = K - K1;
   p1 = __uint_as_float((uint32_t)(K1 + 127) << 23);
   p2 = __uint_as_float((uint32_t)(K2 + 127) << 23);
-}
-
-// The bias digits of output mode 4 in a lane's two slots of each 64-slot
-// group (slots nt and nt + 1 hold G = 0): the top digit slice gets bf16 6144
-// (kOzBiasG) at slot nt, the next one at slot nt + 1; zero without a bias.
-template <int NG>
-__device__ __forceinline__ void ff_bias_masks(int lane, int nt, int bias, uint32_t (&bmask)[NG][2]) {
-  constexpr uint32_t kBiasBits = 0x45C0u;               // bf16 of kOzBiasG (6144)
-#pragma unroll
-  for (int g = 0; g < NG; ++g)
-#pragma unroll
-    for (int sl = 0; sl < 2; ++sl) {
-      const int t = 64 * g + 2 * lane, tb = nt + sl;
-      bmask[g][sl] = !bias ? 0u : (t == tb ? kBiasBits : 0u) | (t + 1 == tb ? kBiasBits << 16 : 0u);
-    }
 }
 
 // One row of float-float values cut into digits: lane L holds slots
 // 64 g + 2 L and 64 g + 2 L + 1.  The row's scale 2^e: the largest |hi|
 // stepped up by one ulp bounds every |hi + lo| (|lo| is at most half an ulp),
-// so every value is below 2^(e - 1).  X = round(|value| 2^(48 - e)) <= 2^47
-// on the fp32 pipe, 16 bits at a time: A = |hi| 2^(48 - e) and B = +-lo
-// 2^(48 - e) (exact power-of-two scalings), T2 = rint(A 2^-32), T1 =
-// rint((A - T2 2^32) 2^-16) (the remainders exact by fused multiply-add), T0
-// = rint(remainder + B), each rint by adding and removing 1.5 2^23 (whose
-// bit pattern then holds the integer), X = T2 2^32 + T1 2^16 + T0.  The last
-// addition rounds only where the remainder and B span more than 24 bits, so
-// X is the nearest integer except within 2^-9 of a tie.  Then the balanced
-// base-256 digits in one step: with Y = X + 127 (1 + 2^8 + ... + 2^32), the
-// low five digits are Y's bytes less 127 (each in [-127, 128], the carries
-// done by the addition) and the top one is Y >> 40.  qe: the power of two
-// the values carry.
+// so every value is below 2^(e - 1) and X = round(|value| 2^(50 - e)) <= 2^49.
+// qe: the power of two the values carry; qt: that of the trig table.
 template <int NG>
-__device__ __forceinline__ void ff_row(const float2 (&v)[NG][2], int lane, __nv_bfloat16 *dst, size_t stride,
-                                       int *gexp, const uint32_t (&bmask)[NG][2], int qe) {
+__device__ __forceinline__ void ff_row(const float2 (&v)[NG][2], int lane, __half *dst, size_t stride, int *gexp, int qe,
+                                       int qt) {
   uint32_t mb = 0u;
 #pragma unroll
   for (int g = 0; g < NG; ++g)
@@ -2484,33 +2473,38 @@ __device__ __forceinline__ void ff_row(const float2 (&v)[NG][2], int lane, __nv_
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
     // the lane's two values, one in each half
-    const uint32_t h0 = __float_as_uint(v[g][0].x), h1 = __float_as_uint(v[g][1].x);
-    uint32_t pre[2][6];
-    ff_digit_pre_x2(x2_pack(h0, h1), x2_pack(__float_as_uint(v[g][0].y), __float_as_uint(v[g][1].y)), p1x, p2x,
-                    pre);
-    const int t = 64 * g + 2 * lane;
-    const uint32_t sm = ((h0 >> 31) << 15) | (h1 & 0x80000000u);
-    uint32_t *d32 = reinterpret_cast<uint32_t *>(dst + t);
+    uint32_t w[5];
+    ff_digits_x2(x2_pack(__float_as_uint(v[g][0].x), __float_as_uint(v[g][1].x)),
+                 x2_pack(__float_as_uint(v[g][0].y), __float_as_uint(v[g][1].y)), p1x, p2x, w);
+    uint32_t *d32 = reinterpret_cast<uint32_t *>(dst + 64 * g + 2 * lane);
 #pragma unroll
-    for (int sl = 0; sl < 6; ++sl) {
-      // 2^23 + 127 (the top digit: 2^23) off both halves: the digits' fp32 patterns
-      const ffx2 d = sub_x2(x2_pack(pre[0][sl], pre[1][sl]), sl == 0 ? 0x4B0000004B000000ull : 0x4B00007F4B00007Full);
-      uint32_t w = __byte_perm((uint32_t)d, (uint32_t)(d >> 32), 0x7632) ^ sm;
-      if (sl < 2) w |= bmask[g][sl];                    // the bias digits (ff_bias_masks)
-      d32[sl * (stride / 2)] = w;
-    }
+    for (int sl = 0; sl < 5; ++sl) d32[sl * (stride / 2)] = w[sl];
   }
-  // value = 2^(e + qe + 1 - 64) (digit sums): trig scale 2^1, digit weights 2^-64
-  if (lane == 0) *gexp = exm == 0 ? 0 : e + qe + 1 - 64;
+  // value = 2^(e + qe + qt - 50) V: V in units of 2^-50 of the two scales
+  if (lane == 0) *gexp = exm == 0 ? 0 : e + qe + qt - 50;
 }
 
+// Slots of a G row (and of a trig digit row): classes of 32, the cos slots
+// then the sin slots of orders m = 0 .. 31; above l_max 31 (NG = 2) cos of even m,
+// cos of odd m, sin of even m, sin of odd m, each by m / 2.
+template <int NG>
+__host__ __device__ __forceinline__ int oz_slot(int m, int sine) {
+  return NG == 1 ? 32 * sine + m : 64 * sine + 32 * (m & 1) + (m >> 1);
+}
+template <int NG>
+__host__ __device__ __forceinline__ int oz_slot_order(int slot) {
+  return NG == 1 ? (slot & 31) : 2 * (slot & 31) + ((slot >> 5) & 1);
+}
+template <int NG>
+__host__ __device__ __forceinline__ int oz_slot_sine(int slot) { return (slot >> (NG == 1 ? 5 : 6)) & 1; }
+
 struct OzThetaFFArgs {
-  int n_shells, shells_pad, n_theta, half, lmax, n_lm, n_pm, nt, gphi, rows_pad, gk, n_r, bias;
+  int n_shells, shells_pad, n_theta, half, lmax, n_lm, n_pm, gphi, rows_pad, gk, n_r, qt;
   const float4 *Qf;             // [3][n_pm][shells_pad] (k_q_ff)
   const int *qexp;              // [3][n_shells]
   const float2 *Pf[2];          // [n_theta][n_lm]: P and dP/dtheta as (hi, lo)
   const double *inv_sin, *inv_r;
-  __nv_bfloat16 *G[4];
+  __half *G[4];
   int *gexp[4];
 };
 
@@ -2587,7 +2581,6 @@ __global__ void __launch_bounds__(512, 2) k_theta_ff(OzThetaFFArgs a) {
       } else {
         m = k == 0 ? gi : L + 1 - gi;
       }
-      const int t0 = m == 0 ? 0 : 2 * m - 1;
       const bool two_slots = m > 0;
       // both slots of m at once (m = 0: the second is zero); aH[i][0], aL[i][0]:
       // terms l = l_max, l_max - 2, ...; [1]: l = l_max - 1, ...
@@ -2634,9 +2627,9 @@ __global__ void __launch_bounds__(512, 2) k_theta_ff(OzThetaFFArgs a) {
         for (int i = 0; i < TP; ++i) {
           const float2 a0 = make_float2(x2_half(aH[i][0], s), x2_half(aL[i][0], s));
           const float2 a1 = make_float2(x2_half(aH[i][1], s), x2_half(aL[i][1], s));
-          srow[(2 * i) * a.gk + t0 + s] = ff_sum(a0, a1, 1.f);
+          srow[(2 * i) * a.gk + oz_slot<NG>(m, s)] = ff_sum(a0, a1, 1.f);
           const float2 d = ff_sum(a0, a1, -1.f);
-          srow[(2 * i + 1) * a.gk + t0 + s] = make_float2(sg * d.x, sg * d.y);
+          srow[(2 * i + 1) * a.gk + oz_slot<NG>(m, s)] = make_float2(sg * d.x, sg * d.y);
         }
       }
     }
@@ -2646,12 +2639,10 @@ __global__ void __launch_bounds__(512, 2) k_theta_ff(OzThetaFFArgs a) {
   // values: its coefficients are the angular set, -Q / r (r the shell's
   // outer edge), and its table m P / sin theta is m / sin theta times Phi's
   // P in the other slot of the same m, so
-  //   G_phi[t] = (+1 for t even, -1 for t odd) (m / (r sin theta)) G_Phi[swap t]
-  // (sin theta_j' = sin theta_j); slot 0 and the slots past nt are zero.
+  //   G_phi[t] = (+1 in the sin slot, -1 in the cos slot) (m / (r sin theta)) G_Phi[swap t]
+  // (sin theta_j' = sin theta_j); m = 0 and the slots without an order are zero.
   const size_t stride = (size_t)a.rows_pad * a.gk;
-  uint32_t bmask[NG][2];
-  ff_bias_masks<NG>(lane, a.nt, a.bias, bmask);
-  __nv_bfloat16 *const Gf = f == 0 ? a.G[0] : f == 1 ? a.G[1] : a.G[2];
+  __half *const Gf = f == 0 ? a.G[0] : f == 1 ? a.G[1] : a.G[2];
   int *const gexp = f == 0 ? a.gexp[0] : f == 1 ? a.gexp[1] : a.gexp[2];
   for (int rr = warp; rr < 32 * R; rr += W) {
     const int sl = rr / R, ri = rr - sl * R;
@@ -2665,34 +2656,34 @@ __global__ void __launch_bounds__(512, 2) k_theta_ff(OzThetaFFArgs a) {
     for (int g = 0; g < NG; ++g)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int t = 64 * g + 2 * lane + h;
-        v[g][h] = t < a.nt ? src[t] : make_float2(0.f, 0.f);
+        const int t = 64 * g + 2 * lane + h, m = oz_slot_order<NG>(t);
+        v[g][h] = m <= L && !(m == 0 && oz_slot_sine<NG>(t)) ? src[t] : make_float2(0.f, 0.f);
       }
     const size_t row = (size_t)shell * a.n_theta + j;
     const int qe = qe_s[sl];
-    ff_row<NG>(v, lane, Gf + row * a.gk, stride, gexp + row, bmask, qe);
+    ff_row<NG>(v, lane, Gf + row * a.gk, stride, gexp + row, qe, a.qt);
     if (f != 0 || !a.gphi) continue;
     const float ch = cphi[sl][ri].x, cl = cphi[sl][ri].y;
 #pragma unroll
     for (int g = 0; g < NG; ++g)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int t = 64 * g + 2 * lane + h;
+        const int t = 64 * g + 2 * lane + h, m = oz_slot_order<NG>(t);
         float2 w = make_float2(0.f, 0.f);
-        if (t >= 1 && t < a.nt) {
-          const float2 x = src[(t & 1) ? t + 1 : t - 1];
-          const float mf = (float)((t + 1) >> 1);
+        if (m >= 1 && m <= L) {
+          const float2 x = src[t ^ (NG == 1 ? 32 : 64)];
+          const float mf = (float)m;
           const float c0 = __fmul_rn(ch, mf);
           const float c1 = __fmaf_rn(cl, mf, __fmaf_rn(ch, mf, -c0));   // c m = c0 + c1
           const float y = __fmul_rn(x.x, c0);
           const float ye = __fmaf_rn(x.x, c1, __fmaf_rn(x.y, c0, __fmaf_rn(x.x, c0, -y)));
           const float hs = __fadd_rn(y, ye);
           w = make_float2(hs, __fsub_rn(ye, __fsub_rn(hs, y)));
-          if (t & 1) w = make_float2(-w.x, -w.y);
+          if (!oz_slot_sine<NG>(t)) w = make_float2(-w.x, -w.y);
         }
         v[g][h] = w;
       }
-    ff_row<NG>(v, lane, a.G[3] + row * a.gk, stride, a.gexp[3] + row, bmask, qe);
+    ff_row<NG>(v, lane, a.G[3] + row * a.gk, stride, a.gexp[3] + row, qe, a.qt);
   }
 }
 
@@ -3020,12 +3011,14 @@ __global__ void __launch_bounds__(256) k_rhow_ozaki(OzRhoArgs a) {
 }  // namespace yy
 
 struct yy_oz_tables {
-  int rows, rows_pad, bn, row_tiles, b_rows_pad, stages, pair_slots;
+  int rows, rows_pad, b_rows_pad;
   int gk;                       // slots of a G row and of a trig digit row: 64 (l_max <= 31) or 128
-  int bias;                     // synthesis with biased level sums (one fill): k_oz_synth
-  int synth_slots;              // resident clusters of k_oz_synth (0: use k_tc_pair output mode 4)
-  yy::OzSynthMaps synth_maps;   // its G maps (those of `maps`) and the trig map with 48-row boxes
-  void *G[4];                   // per field: slices [6][rows_pad][64]
+  int qt;                       // the trig digits are those of trig 2^-qt
+  yy::AzFold fold;              // the columns of the synthesis (half of the longitudes)
+  int shift;                    // columns before the first folded one (OzSynthArgs)
+  int synth_slots;              // resident clusters of k_oz_synth
+  yy::OzSynthMaps synth_maps;
+  void *G[4];                   // per field: digit slices [5][rows_pad][gk]
   int *gexp[4];                 // per field: [rows_pad]
   double *inv_sin, *inv_r;      // 1 / sin theta_j at the polar cell centres, 1 / r_(n+1) per shell
   int shells_pad;               // shells rounded up to 32 (k_theta_ff's tiles)
@@ -3034,8 +3027,7 @@ struct yy_oz_tables {
   float2 *Pf[2];                // [n_theta][n_lm]: P and dP/dtheta as fp32 pairs
   float2 *tbf;                  // [ceil(n_theta / 2)][n_lm]: the analysis table T as fp32 pairs
   float2 *Df;                   // [sum_l (2l+1)^2]: the rotation D^l as fp32 pairs (two patches)
-  void *trig;                   // slices of trig / 2: [6][b_rows_pad][64]
-  yy::PairMaps maps;
+  void *trig;                   // digit slices of trig 2^-qt: [9][b_rows_pad][gk]
   // analysis (FormOzaki in fills of kFillK): rho w digit rows as operand A, the azimuthal table as operand B
   int an_ok, an_kpad, an_bn, an_row_tiles, an_b_rows_pad, an_stages, an_slots, an_eb;
   void *an_x;                   // [6][rows_pad][an_kpad]
@@ -3265,45 +3257,82 @@ cudaError_t ozaki_rotate(yy_grid *g, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// balanced base-1024 digits of X <= 2^49 (most significant first): each in
+// [-511, 512] with a carry into the next
+static void oz_digits1024(unsigned long long X, int (&d)[5]) {
+  for (int s = 4; s > 0; --s) {
+    int v = (int)(X & 1023u);
+    X >>= 10;
+    if (v > 512) {
+      v -= 1024;
+      X += 1;
+    }
+    d[s] = v;
+  }
+  d[0] = (int)X;
+}
+
+// fp16 bits of a value that fp16 holds exactly
+static uint16_t half_bits(float v) {
+  const __half h = __float2half_rn(v);
+  uint16_t u;
+  memcpy(&u, &h, 2);
+  return u;
+}
+
+// Trig digit slices (FormOzSynth): digits 0..3 of y = trig 2^-qt, then digits
+// 0..4 scaled by 2^-10, rows = columns of the fold, slots by class.  False: a
+// level sum of levels 0..2 could reach 2^24 at some column (|G digit| <= 512).
+template <int NG>
+static bool oz_trig_digits(const yy_grid *g, const yy_oz_tables *o, const std::vector<double> &tr, int qt,
+                           std::vector<uint16_t> &sl) {
+  typedef FormOzSynth F;
+  std::fill(sl.begin(), sl.end(), (uint16_t)0);
+  bool exact = true;
+  for (int c = 0; c < o->fold.half + o->shift; ++c) {
+    // a column before the first repeats that one's mirror cell
+    const bool mirror = c < o->shift;
+    const int k = o->fold.first + (mirror ? 0 : c - o->shift);
+    long long asum[4][3] = {};   // per class, of the three top digits
+    for (int m = 0; m <= g->lmax; ++m)
+      for (int sine = 0; sine < (m > 0 ? 2 : 1); ++sine) {
+        const int t = oz_slot<NG>(m, sine);
+        const double x = tr[(size_t)(m == 0 ? 0 : 2 * m - 1 + sine) * g->n_phi + k];
+        const double y = ldexp(mirror && sine ? -x : x, -qt);
+        int d[5];
+        oz_digits1024((unsigned long long)floor(ldexp(fabs(y), 50) + 0.5), d);
+        for (int s = 0; s < 5; ++s) {
+          const float v = (float)(y < 0 ? -d[s] : d[s]);
+          if (s < F::kTrigScaled) sl[((size_t)s * o->b_rows_pad + c) * o->gk + t] = half_bits(v);
+          sl[((size_t)(F::kTrigScaled + s) * o->b_rows_pad + c) * o->gk + t] = half_bits(ldexpf(v, -10));
+          if (s < 3) asum[t / F::kClassSlots][s] += abs(d[s]);
+        }
+      }
+    for (auto &u : asum) exact = exact && 512 * (u[0] + u[1] + u[2]) < (1ll << 24);
+  }
+  return exact;
+}
+
 yy_status ozaki_prepare(yy_grid *g) {
-  typedef FormOzaki F;
+  typedef FormOzSynth F;
   if (g->oz) return YY_OK;
   const int nt = 2 * g->lmax + 1;
-  if (nt > 2 * F::kMaxK || !g->sep_tr || !g->sep_P || !g->sep_dP || !g->sep_Qs) return YY_ERR_NOT_SUPPORTED;
+  if (nt > 127 || !g->sep_tr || !g->sep_P || !g->sep_dP || !g->sep_Qs) return YY_ERR_NOT_SUPPORTED;
   yy_oz_tables *o = new (std::nothrow) yy_oz_tables();
   if (!o) return YY_ERR_OOM;
-  o->gk = nt <= F::kMaxK ? F::kMaxK : 2 * F::kMaxK;   // K of the synthesis contraction: one fill either way
+  o->gk = g->lmax <= 31 ? 64 : 128;
   o->rows = grid_rows(g) * g->n_theta;
   o->rows_pad = round_up(o->rows, 2 * kPairRows);
-  o->bn = 32;   // eight accumulators of bn columns fill one 256-column TMEM buffer
-  o->row_tiles = (g->n_phi + o->bn - 1) / o->bn;
-  // trig rows padded for both synthesis kernels: tiles of bn (k_tc_pair) and
-  // of kOzSynthBN (k_oz_synth)
-  o->b_rows_pad = round_up(g->n_phi, kOzSynthBN);
-  o->stages = pair_stages<F>(o->bn, kEpiStageBytes);
+  o->fold = az_fold(g);
+  o->shift = g->n_phi % 2 == 0 ? o->fold.first & 1 : 0;   // runs of columns from even cells
+  o->b_rows_pad = round_up(o->fold.half + o->shift, kOzBN);
   yy_status st = YY_OK;
-  if (o->stages < 2 ||
-      cudaFuncSetAttribute(k_tc_pair<F, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess ||
-      cudaFuncSetAttribute(k_tc_pair<F, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess)
-    st = YY_ERR_NOT_SUPPORTED;
-  if (st == YY_OK) {
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg =
-        pair_config(64, o->stages * pair_stage_bytes<F>(o->bn) + kSmemFixed + kEpiStageBytes, 0, attr);
-    int n = 0, n4 = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, (void *)k_tc_pair<F, 3>, &cfg) != cudaSuccess || n < 1 ||
-        cudaOccupancyMaxActiveClusters(&n4, (void *)k_tc_pair<F, 4>, &cfg) != cudaSuccess || n4 < 1) {
-      cudaGetLastError();
-      st = YY_ERR_NOT_SUPPORTED;
-    }
-    o->pair_slots = n < n4 ? n : n4;
-  }
   cudaError_t e = cudaSuccess;
   auto A = [&](void **ptr, size_t bytes) {
     if (e == cudaSuccess) e = dmalloc(ptr, bytes);
   };
-  const size_t g_bytes = (size_t)F::kPA * o->rows_pad * o->gk * F::kElem;
-  const size_t t_elems = (size_t)F::kPB * o->b_rows_pad * o->gk;
+  const size_t g_bytes = (size_t)F::kSlices * o->rows_pad * o->gk * F::kElem;
+  const size_t t_elems = (size_t)F::kTrig * o->b_rows_pad * o->gk;
   if (st == YY_OK) {
     for (int f = 0; f < 4; ++f) {
       A(&o->G[f], g_bytes);
@@ -3365,64 +3394,36 @@ yy_status ozaki_prepare(yy_grid *g) {
     if (e != cudaSuccess) st = e == cudaErrorMemoryAllocation ? YY_ERR_OOM : YY_ERR_CUDA;
   }
   if (st == YY_OK) {
-    // trig digits on the host: y = trig / 2, |y| <= 1/2, X = round(|y| 2^48)
-    // (exact: |y| 2^48 < 2^52), balanced digits with the sign of y
+    // trig digits on the host, of trig / 4; a smaller scale has other digits,
+    // should a column's sums come out too large
     std::vector<double> tr((size_t)nt * g->n_phi);
-    std::vector<uint16_t> sl(t_elems, 0);
+    std::vector<uint16_t> sl(t_elems);
     if (cudaMemcpy(tr.data(), g->sep_tr, tr.size() * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
       st = YY_ERR_CUDA;
-    // output mode 4 needs two spare K columns and |S_L| < 2^22 for every
-    // level and longitude: |S_L| <= 128 sum over the level's products (s, u)
-    // of sum_t |trig digit u at t| (G digits are at most 128 in magnitude)
-    bool bias = nt + 2 <= o->gk;
-    for (int k = 0; k < g->n_phi && st == YY_OK; ++k) {
-      long long asum[6] = {0, 0, 0, 0, 0, 0};
-      for (int t = 0; t < nt; ++t) {
-        const double y = tr[(size_t)t * g->n_phi + k] * 0.5;
-        int d[6];
-        oz_digits((unsigned long long)floor(ldexp(fabs(y), 48) + 0.5), d);
-        for (int s2 = 0; s2 < F::kPB; ++s2) {
-          sl[((size_t)s2 * o->b_rows_pad + k) * o->gk + t] = bf16_int(y < 0 ? -d[s2] : d[s2]);
-          asum[s2] += d[s2] < 0 ? -d[s2] : d[s2];
-        }
-      }
-      for (int L = 0; L < F::kAccs; ++L) {
-        long long b = 0;
-        for (int s2 = F::s_lo(L); s2 <= (L < 5 ? L : 5); ++s2) b += asum[L - s2];
-        if (128 * b >= (1ll << 22)) bias = false;
-      }
-    }
-    if (bias) {
-      // the trig side of the bias columns: 2^11 in every slice at nt, in slice 5 at nt + 1
-      const uint16_t two11 = bf16_int(2048);   // a power of two: exact in bf16
-      for (int k = 0; k < o->b_rows_pad; ++k) {
-        for (int s2 = 0; s2 < F::kPB; ++s2) sl[((size_t)s2 * o->b_rows_pad + k) * o->gk + nt] = two11;
-        sl[((size_t)5 * o->b_rows_pad + k) * o->gk + nt + 1] = two11;
-      }
-    }
-    o->bias = bias ? 1 : 0;
+    const int q0 = 2;
+    auto digits = [&](int q) { return o->gk == 64 ? oz_trig_digits<1>(g, o, tr, q, sl) : oz_trig_digits<2>(g, o, tr, q, sl); };
+    for (o->qt = q0; st == YY_OK && !digits(o->qt) && o->qt < q0 + 2;) ++o->qt;
     if (st == YY_OK && cudaMemcpy(o->trig, sl.data(), t_elems * F::kElem, cudaMemcpyHostToDevice) != cudaSuccess)
       st = YY_ERR_CUDA;
   }
   if (st == YY_OK) {
-    bool ok = make_map<F>(&o->maps.b[0], o->trig, o->gk, F::kPB * o->b_rows_pad, o->bn / 2);
+    bool ok = make_map<F>(&o->synth_maps.b, o->trig, o->gk, F::kTrig * o->b_rows_pad, kOzBN / 2);
     for (int f = 0; f < 4 && ok; ++f)
-      ok = make_map<F>(&o->maps.a[f], o->G[f], o->gk, F::kPA * o->rows_pad, kPairRows);
-    if (!ok) st = YY_ERR_NOT_SUPPORTED;
-  }
-  if (st == YY_OK && o->bias && o->gk == kOzSynthKB * 32) {
-    // the synthesis kernel with the G tile resident (falls back to the pair
-    // kernel's output mode 4 where it cannot run)
+      ok = make_map<F>(&o->synth_maps.a[f], o->G[f], o->gk, F::kSlices * o->rows_pad, kPairRows);
+    const void *k = o->gk == 64 ? (const void *)k_oz_synth<2> : (const void *)k_oz_synth<4>;
+    const int smem = o->gk == 64 ? oz_synth_smem<2>() : oz_synth_smem<4>();
     int n = 0;
-    for (int f = 0; f < 4; ++f) o->synth_maps.a[f] = o->maps.a[f];
-    if (make_map<F>(&o->synth_maps.b, o->trig, o->gk, F::kPB * o->b_rows_pad, kOzSynthBN / 2) &&
-        cudaFuncSetAttribute(k_oz_synth, cudaFuncAttributeMaxDynamicSharedMemorySize, kOzSynthSmem) == cudaSuccess) {
+    if (ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess) {
       cudaLaunchAttribute attr[1];
-      cudaLaunchConfig_t cfg = pair_config(64, kOzSynthSmem, 0, attr);
-      if (cudaOccupancyMaxActiveClusters(&n, (void *)k_oz_synth, &cfg) != cudaSuccess) n = 0;
+      cudaLaunchConfig_t cfg = pair_config(64, smem, 0, attr);
+      cfg.blockDim = dim3(kOzThreads);
+      if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) n = 0;
     }
-    cudaGetLastError();
-    o->synth_slots = n > 0 ? n : 0;
+    o->synth_slots = n;
+    if (n < 1) {
+      cudaGetLastError();
+      st = YY_ERR_NOT_SUPPORTED;
+    }
   }
   if (st == YY_OK) st = ozaki_prepare_analysis(g, o);
   if (st != YY_OK) {
@@ -3435,7 +3436,6 @@ yy_status ozaki_prepare(yy_grid *g) {
 }
 
 cudaError_t ozaki_synthesis(yy_grid *g, double *py, double *pg, double *gy, double *gg, cudaStream_t s) {
-  typedef FormOzaki F;
   yy_oz_tables *o = g->oz;
   const int n_jobs = gy ? 4 : 1;
   const int n_shells = grid_rows(g);
@@ -3464,12 +3464,11 @@ cudaError_t ozaki_synthesis(yy_grid *g, double *py, double *pg, double *gy, doub
   fa.lmax = g->lmax;
   fa.n_lm = g->n_lm;
   fa.n_pm = n_pm_of(g->lmax);
-  fa.nt = 2 * g->lmax + 1;
   fa.gphi = n_jobs == 4 ? 1 : 0;
   fa.rows_pad = o->rows_pad;
   fa.gk = o->gk;
   fa.n_r = g->n_r;
-  fa.bias = o->bias;
+  fa.qt = o->qt;
   fa.Qf = o->Qf;
   fa.qexp = o->qexp;
   fa.Pf[0] = o->Pf[0];
@@ -3477,7 +3476,7 @@ cudaError_t ozaki_synthesis(yy_grid *g, double *py, double *pg, double *gy, doub
   fa.inv_sin = o->inv_sin;
   fa.inv_r = o->inv_r;
   for (int f = 0; f < 4; ++f) {
-    fa.G[f] = (__nv_bfloat16 *)o->G[f];
+    fa.G[f] = (__half *)o->G[f];
     fa.gexp[f] = o->gexp[f];
   }
   const int n_groups = g->lmax / 2 + 1, tp = theta_ff_tp(o->gk);
@@ -3494,63 +3493,33 @@ cudaError_t ozaki_synthesis(yy_grid *g, double *py, double *pg, double *gy, doub
   const size_t comp = (size_t)g->n_r * g->n_ang;
   double *o0[4] = {py, gy, gy ? gy + comp : nullptr, gy ? gy + 2 * comp : nullptr};
   double *o1[4] = {pg, gg, gg ? gg + comp : nullptr, gg ? gg + 2 * comp : nullptr};
-  if (o->bias && o->synth_slots > 0) {
-    OzSynthArgs z = {};
-    z.cells = o->rows;
-    z.cell_tiles = o->rows_pad / (2 * kPairRows);
-    z.cols = g->n_phi;
-    z.col_tiles = o->b_rows_pad / kOzSynthBN;
-    z.a_rows = o->rows_pad;
-    z.b_rows = o->b_rows_pad;
-    z.out_split = g->n_r * g->n_theta;
-    z.ldo = g->n_phi;
-    z.n_jobs = n_jobs;
-    z.prefetch = 1;
-    z.err = g->err;
-    for (int f = 0; f < n_jobs; ++f) {
-      z.job[f].out0 = o0[f];
-      z.job[f].out1 = o1[f];
-      z.job[f].cell_exp = o->gexp[f];
-    }
-    const int tiles = z.cell_tiles * n_jobs;
-    const int pairs = tiles < o->synth_slots ? tiles : o->synth_slots;
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = pair_config(pairs, kOzSynthSmem, s, attr);
-    e = cudaLaunchKernelEx(&cfg, k_oz_synth, o->synth_maps, z);
-    note_launch(g, "k_oz_synth", s);
-    return e;
-  }
-  PairArgs a = {};
-  a.stages = o->stages;
-  a.cells = o->rows;
-  a.cell_tiles = o->rows_pad / (2 * kPairRows);
-  a.rows = g->n_phi;
-  a.row_tiles = o->row_tiles;
-  a.bn = o->bn;
-  a.kb_total = o->gk * F::kElem / kRowBytes;   // one fill (level sums below 2^24 up to K = 160)
-  a.k_splits = 1;
-  a.kb_per_split = a.kb_total;
-  a.a_rows = o->rows_pad;
-  a.b_rows = o->b_rows_pad;
-  a.out_mode = o->bias ? 4 : 3;
-  a.out_split = g->n_r * g->n_theta;
-  a.ldo = g->n_phi;
-  a.n_jobs = n_jobs;
-  a.err = g->err;
+  OzSynthArgs z = {};
+  z.cells = o->rows;
+  z.cell_tiles = o->rows_pad / (2 * kPairRows);
+  z.col_tiles = o->b_rows_pad / kOzBN;
+  z.n_phi = g->n_phi;
+  z.first = o->fold.first;
+  z.shift = o->shift;
+  z.half = o->fold.half;
+  z.a_rows = o->rows_pad;
+  z.b_rows = o->b_rows_pad;
+  z.out_split = g->n_r * g->n_theta;
+  z.ldo = g->n_phi;
+  z.n_jobs = n_jobs;
+  z.err = g->err;
   for (int f = 0; f < n_jobs; ++f) {
-    PairJob &J = a.job[f];
-    J.out0 = o0[f];
-    J.out1 = o1[f];
-    J.cell_exp = o->gexp[f];
-    J.ta = f;
-    J.tb = 0;
+    z.job[f].out0 = o0[f];
+    z.job[f].out1 = o1[f];
+    z.job[f].cell_exp = o->gexp[f];
   }
-  const int tiles = a.cell_tiles * a.row_tiles * n_jobs;
-  const int pairs = tiles < o->pair_slots ? tiles : o->pair_slots;
+  const int tiles = z.cell_tiles * n_jobs;
+  const int pairs = tiles < o->synth_slots ? tiles : o->synth_slots;
   cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = pair_config(pairs, o->stages * pair_stage_bytes<F>(o->bn) + kSmemFixed + kEpiStageBytes, s, attr);
-  e = o->bias ? cudaLaunchKernelEx(&cfg, k_tc_pair<F, 4>, o->maps, a) : cudaLaunchKernelEx(&cfg, k_tc_pair<F, 3>, o->maps, a);
-  note_launch(g, "k_tc_pair<FormOzaki,3>/synthesis", s);
+  cudaLaunchConfig_t cfg = pair_config(pairs, o->gk == 64 ? oz_synth_smem<2>() : oz_synth_smem<4>(), s, attr);
+  cfg.blockDim = dim3(kOzThreads);
+  e = o->gk == 64 ? cudaLaunchKernelEx(&cfg, k_oz_synth<2>, o->synth_maps, z)
+                  : cudaLaunchKernelEx(&cfg, k_oz_synth<4>, o->synth_maps, z);
+  note_launch(g, "k_oz_synth", s);
   return e;
 }
 
