@@ -9,7 +9,7 @@
 // contractions run over half of the longitudes with half of the slots each.
 //
 // Digits (FormOzSynth): x = sum_s a_s 2^(-10 (s + 1)), five balanced base-1024
-// digits |a_s| <= 512, exact in fp16; rows of G scaled to |x| <= 1/2, the trig
+// digits |a_s| <= 512 (528 for one of G's), exact in fp16; rows of G scaled to |x| <= 1/2, the trig
 // table to |y| <= 1/4 (1/8 above l_max 31).  The products of digit levels L = s + t
 // <= 4 are kept, the dropped ones add up to below 2^-50 of the scales.  A class
 // (the cos or sin slots; above l_max 31 those of even and of odd m apart) has at

@@ -2387,62 +2387,48 @@ __device__ __forceinline__ void x_digit_bits(unsigned long long X, uint32_t (&bi
 
 __device__ __forceinline__ ffx2 x2_pack(uint32_t lo, uint32_t hi) { return ((ffx2)hi << 32) | lo; }
 
-// The balanced base-1024 digits (FormOzSynth) of two float-float values (hi, lo)
-// at once, both halves of each packed register: X = round(|value| 2^K) <= 2^49,
-// 2^K = p1 p2 the row's scale, on the fp32 pipe, 16 bits at a time: A =
-// |hi| 2^K and B = +-lo 2^K (exact power-of-two scalings), T2 = rint(A 2^-32), T1 =
-// rint((A - T2 2^32) 2^-16), T1' = rint(B 2^-16) (|B| <= 2^24; the remainders
-// exact by fused multiply-add), T0 = rint(A's remainder + B's), each rint by adding
-// and removing 1.5 2^23 (whose bit pattern then holds the integer), X = T2 2^32 +
-// (T1 + T1') 2^16 + T0.  The last sum rounds only where the remainders span more
-// than 24 bits, so X is the nearest integer except near a tie.  The scalings by 2^-32 and 2^-16 are
-// exact (or leave a sum of 1.5 2^23 that rounds to it either way), so each
-// multiply-and-add is one fused operation.  Then the digits in one step: with
-// Y = X + 511 (1 + 2^10 + 2^20 + 2^30), the low four digits are Y's 10-bit
-// fields less 511 (each in [-511, 512], the carries done by the addition) and
-// the top one is Y >> 40.  A field f is the fp16 pattern 0x6400 | f of 1024 + f, from
-// which one exact fp16 subtraction leaves the digit: w[s] = digit s of both values
-// as fp16 patterns, most significant first, both with the sign bits `sm`.
+// Base-1024 digits (FormOzSynth) of two float-float values (hi, lo) at once, both
+// halves of each packed register, in fp32 arithmetic: with H = hi 2^K, 2^K = p1 p2
+// the row's scale, |H| <= 512, each digit is the remainder rounded to an integer
+// by adding and removing M = 1.5 2^23, and the next remainder is 1024 times what
+// is left (exact by fused multiply-add): the first two digits come from hi, whose
+// 24 bits end in the third, where L = lo 2^(K + 20) (|L| <= 16) joins; the sum of the
+// remainder and L there rounds off less than 2^-25 of that digit's unit.  So
+// sum_s d_s 1024^(4 - s) is (hi + lo) 2^(K + 40) to within one half in the last digit, with
+// |d_s| <= 512 (|d_2| <= 528).  w[s] = digit s of both values as fp16 (exact), most
+// significant first.  (Through a 50-bit integer, its fields and signs: 195 us for
+// k_theta_ff on the 1-degree grid against 172.)
+__device__ __forceinline__ uint32_t x2_half2(ffx2 v) {
+  uint32_t d;
+  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(x2_half(v, 1)), "f"(x2_half(v, 0)));
+  return d;
+}
 __device__ __forceinline__ void ff_digits_x2(ffx2 hi, ffx2 lo, ffx2 p1, ffx2 p2, uint32_t (&w)[5]) {
-  constexpr ffx2 kSign = 0x8000000080000000ull;
   constexpr ffx2 kM = 0x4B4000004B400000ull;             // 1.5 2^23 in both halves
-  constexpr uint32_t kMBits = 0x4B400000u;
-  const ffx2 sg = hi & kSign;
-  const ffx2 A = mul_x2(mul_x2(hi ^ sg, p1), p2);        // |hi| 2^K
-  const ffx2 B = mul_x2(mul_x2(lo ^ sg, p1), p2);        // +-lo 2^K, the sign of |value|
-  const ffx2 s2 = fma_x2(A, 0x2F8000002F800000ull, kM);                              // A 2^-32 + M
-  const ffx2 R1 = fma_x2(sub_x2(s2, kM), 0xCF800000CF800000ull, A);                  // A - T2 2^32
-  const ffx2 s1 = fma_x2(R1, 0x3780000037800000ull, kM);                             // R1 2^-16 + M
-  const ffx2 R2 = fma_x2(sub_x2(s1, kM), 0xC7800000C7800000ull, R1);                 // R1 - T1 2^16
-  const ffx2 sb = fma_x2(B, 0x3780000037800000ull, kM);                              // B 2^-16 + M
-  const ffx2 B0 = fma_x2(sub_x2(sb, kM), 0xC7800000C7800000ull, B);                  // B - T1' 2^16
-  const ffx2 s0 = add_x2(add_x2(R2, B0), kM);
-  uint32_t yl[2], yh[2];
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const long long X = ((long long)(int)((uint32_t)(s2 >> (32 * h)) - kMBits) << 32) +
-                        ((long long)(int)((uint32_t)(s1 >> (32 * h)) + (uint32_t)(sb >> (32 * h)) - 2u * kMBits) << 16) +
-                        (long long)(int)((uint32_t)(s0 >> (32 * h)) - kMBits);
-    const unsigned long long Y = (unsigned long long)X + 511ull * (1ull + (1ull << 10) + (1ull << 20) + (1ull << 30));
-    yl[h] = (uint32_t)Y;
-    yh[h] = (uint32_t)(Y >> 32);
-  }
-  const uint32_t sm = ((uint32_t)hi >> 31 << 15) | ((uint32_t)(hi >> 32) & 0x80000000u);
-  const uint32_t f[5] = {__byte_perm(yh[0] >> 8, yh[1] >> 8, 0x5410),
-                         __byte_perm(__funnelshift_r(yl[0], yh[0], 30), __funnelshift_r(yl[1], yh[1], 30), 0x5410),
-                         __byte_perm(yl[0] >> 20, yl[1] >> 20, 0x5410), __byte_perm(yl[0] >> 10, yl[1] >> 10, 0x5410),
-                         __byte_perm(yl[0], yl[1], 0x5410)};
-#pragma unroll
-  for (int s = 0; s < 5; ++s) {
-    const uint32_t x = (f[s] & 0x03FF03FFu) | 0x64006400u;
-    const __half2 d = __hsub2(*reinterpret_cast<const __half2 *>(&x), __float2half2_rn(s == 0 ? 1024.f : 1535.f));
-    w[s] = *reinterpret_cast<const uint32_t *>(&d) ^ sm;
-  }
+  constexpr ffx2 k1024 = 0x4480000044800000ull;
+  constexpr ffx2 kNeg = 0xBF800000BF800000ull;            // -1
+  constexpr ffx2 k2p20 = 0x4980000049800000ull;
+  const ffx2 H = mul_x2(mul_x2(hi, p1), p2);
+  const ffx2 L = mul_x2(mul_x2(mul_x2(lo, p1), p2), k2p20);
+  const ffx2 d0 = sub_x2(add_x2(H, kM), kM);
+  const ffx2 r0 = sub_x2(H, d0);
+  const ffx2 d1 = sub_x2(fma_x2(r0, k1024, kM), kM);
+  const ffx2 r1 = fma_x2(r0, k1024, mul_x2(d1, kNeg));
+  const ffx2 d2 = sub_x2(add_x2(fma_x2(r1, k1024, kM), L), kM);
+  const ffx2 r2 = add_x2(fma_x2(r1, k1024, mul_x2(d2, kNeg)), L);
+  const ffx2 d3 = sub_x2(fma_x2(r2, k1024, kM), kM);
+  const ffx2 r3 = fma_x2(r2, k1024, mul_x2(d3, kNeg));
+  const ffx2 d4 = sub_x2(fma_x2(r3, k1024, kM), kM);
+  w[0] = x2_half2(d0);
+  w[1] = x2_half2(d1);
+  w[2] = x2_half2(d2);
+  w[3] = x2_half2(d3);
+  w[4] = x2_half2(d4);
 }
 
-// the row scale of ff_row: 2^K with K = 50 - e as two normal fp32 factors
+// the row scale of ff_row: 2^K with K = 10 - e as two normal fp32 factors
 __device__ __forceinline__ void ff_row_scale(int e, float &p1, float &p2) {
-  const int K = 50 - e, K1 = K >> 1, K2 = K - K1;
+  const int K = 10 - e, K1 = K >> 1, K2 = K - K1;
   p1 = __uint_as_float((uint32_t)(K1 + 127) << 23);
   p2 = __uint_as_float((uint32_t)(K2 + 127) << 23);
 }
@@ -2450,7 +2436,7 @@ __device__ __forceinline__ void ff_row_scale(int e, float &p1, float &p2) {
 // One row of float-float values cut into digits: lane L holds slots
 // 64 g + 2 L and 64 g + 2 L + 1.  The row's scale 2^e: the largest |hi|
 // stepped up by one ulp bounds every |hi + lo| (|lo| is at most half an ulp),
-// so every value is below 2^(e - 1) and X = round(|value| 2^(50 - e)) <= 2^49.
+// so every value is below 2^(e - 1).
 // qe: the power of two the values carry; qt: that of the trig table.
 template <int NG>
 __device__ __forceinline__ void ff_row(const float2 (&v)[NG][2], int lane, __half *dst, size_t stride, int *gexp, int qe,
@@ -3282,7 +3268,7 @@ static uint16_t half_bits(float v) {
 
 // Trig digit slices (FormOzSynth): digits 0..3 of y = trig 2^-qt, then digits
 // 0..4 scaled by 2^-10, rows = columns of the fold, slots by class.  False: a
-// level sum of levels 0..2 could reach 2^24 at some column (|G digit| <= 512).
+// level sum of levels 0..2 could reach 2^24 at some column (|G digit| <= 528).
 template <int NG>
 static bool oz_trig_digits(const yy_grid *g, const yy_oz_tables *o, const std::vector<double> &tr, int qt,
                            std::vector<uint16_t> &sl) {
@@ -3308,7 +3294,7 @@ static bool oz_trig_digits(const yy_grid *g, const yy_oz_tables *o, const std::v
           if (s < 3) asum[t / F::kClassSlots][s] += abs(d[s]);
         }
       }
-    for (auto &u : asum) exact = exact && 512 * (u[0] + u[1] + u[2]) < (1ll << 24);
+    for (auto &u : asum) exact = exact && 528 * (u[0] + u[1] + u[2]) < (1ll << 24);
   }
   return exact;
 }
