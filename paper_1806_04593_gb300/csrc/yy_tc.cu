@@ -2414,7 +2414,7 @@ __device__ __forceinline__ void ff_digits_x2(ffx2 hi, ffx2 lo, ffx2 p1, ffx2 p2,
   const ffx2 r0 = sub_x2(H, d0);
   const ffx2 d1 = sub_x2(fma_x2(r0, k1024, kM), kM);
   const ffx2 r1 = fma_x2(r0, k1024, mul_x2(d1, kNeg));
-  const ffx2 d2 = sub_x2(add_x2(fma_x2(r1, k1024, kM), L), kM);
+  const ffx2 d2 = sub_x2(add_x2(fma_x2(r1, k1024, L), kM), kM);   // of the rounded sum: within 2^-15 of the nearest
   const ffx2 r2 = add_x2(fma_x2(r1, k1024, mul_x2(d2, kNeg)), L);
   const ffx2 d3 = sub_x2(fma_x2(r2, k1024, kM), kM);
   const ffx2 r3 = fma_x2(r2, k1024, mul_x2(d3, kNeg));

@@ -34,7 +34,7 @@ def digits(hi, lo, K):
     r0 = f32(H - d0)
     d1 = f32(fma(r0, k, M) - M)
     r1 = fma(r0, k, f32(-d1))
-    d2 = f32(f32(fma(r1, k, M) + L) - M)
+    d2 = f32(f32(fma(r1, k, L) + M) - M)
     r2 = f32(fma(r1, k, f32(-d2)) + L)
     d3 = f32(fma(r2, k, M) - M)
     r3 = fma(r2, k, f32(-d3))
