@@ -342,6 +342,12 @@ yy_status yy_potential(yy_grid *g, const double *rho_yin, const double *rho_yang
   const bool f32 = (prec == YY_FP32);
   g->launches = 0;
   g->atot_done = 0;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {   // another thread's capture keeps the legacy stream out
+    cudaGetLastError();
+    capture = cudaStreamCaptureStatusActive;
+  }
+  g->overlap = !prof && capture == cudaStreamCaptureStatusNone;
   mark(0);
   if (e == cudaSuccess) {
     const bool separable = g->analysis_method == YY_ANALYSIS_SEPARABLE ||
@@ -383,6 +389,7 @@ yy_status yy_potential(yy_grid *g, const double *rho_yin, const double *rho_yang
                     : tc_synthesis(g, prec, phi_yin, phi_yang, grad_yin, grad_yang, s);
   }
   mark(3);
+  g->overlap = 0;
   return from_cuda(e);
 }
 

@@ -80,6 +80,7 @@ struct OzAnalysisMaps {
 
 __global__ void __launch_bounds__(kThreads, 1)
 k_oz_analysis(const __grid_constant__ OzAnalysisMaps maps, const __grid_constant__ OzAnalysisArgs a) {
+  pdl_wait();
   typedef FormOzaki F;
   constexpr int KSTEPS = kRowBytes / 32;
   constexpr int S = kOzAnStages;

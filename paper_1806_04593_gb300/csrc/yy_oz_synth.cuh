@@ -153,6 +153,7 @@ __device__ __forceinline__ void oz_store_runs1(const double *ebuf, double *const
 template <int NCLS>
 __global__ void __launch_bounds__(kOzThreads, 1)
 k_oz_synth(const __grid_constant__ OzSynthMaps maps, const __grid_constant__ OzSynthArgs a) {
+  pdl_wait();
   typedef FormOzSynth F;
   constexpr int KSTEPS = kRowBytes / 32;        // MMAs of K = 16 per class
   constexpr int BH = kOzBN / 2;                 // trig rows per CTA and tile

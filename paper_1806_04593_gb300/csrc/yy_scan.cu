@@ -166,6 +166,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 k_rotate_moments(int n_r, int n_lm, const T *__restrict__ rot, const double *__restrict__ A,
                  double *__restrict__ Atot) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char smraw[];
   T *a = reinterpret_cast<T *>(smraw);   // [2][n_lm]
   const int n = blockIdx.x;
@@ -343,6 +344,7 @@ template <int CH>
 __global__ void __launch_bounds__(kScanThreads, 3)
 k_scan_tile(int n_patch, int n_r, int lmax, int n_lm, const double *__restrict__ A, const double *__restrict__ coef,
             const double2 *__restrict__ prod, double *__restrict__ Q, float *__restrict__ Q32) {
+  pdl_begin();
   __shared__ ScanShared sm;
   scan_tile_body<CH>(sm, (int)blockIdx.x, n_patch, n_r, lmax, n_lm, A, coef, prod, Q, Q32);
 }
@@ -418,12 +420,9 @@ cudaError_t rotate_moments(yy_grid *g, bool fp64, cudaStream_t st) {
     if (e != cudaSuccess) return e;
   }
   const dim3 grid((unsigned)g->n_r, (unsigned)((g->n_lm + 255) / 256));
-  if (fp64)
-    k_rotate_moments<double><<<grid, 256, smem, st>>>(g->n_r, g->n_lm, g->rot, g->A, g->Atot);
-  else
-    k_rotate_moments<float><<<grid, 256, smem, st>>>(g->n_r, g->n_lm, g->rot32, g->A, g->Atot);
-  note_launch(g, "k_rotate_moments", st);
-  return cudaGetLastError();
+  return fp64 ? launch_kernel(g, "k_rotate_moments", k_rotate_moments<double>, grid, 256, smem, st, g->n_r, g->n_lm, g->rot, g->A, g->Atot)
+              : launch_kernel(g, "k_rotate_moments", k_rotate_moments<float>, grid, 256, smem, st, g->n_r, g->n_lm, g->rot32, g->A,
+                              g->Atot);
 }
 
 void scan_geometry(const yy_grid *g, int *nc, int *ch) {
@@ -442,12 +441,10 @@ cudaError_t radial_scan(yy_grid *g, bool want_f32, cudaStream_t st) {
     const unsigned blocks = (unsigned)(g->n_patch * ((g->n_lm + kScanModes - 1) / kScanModes));
     switch (form) {
 #define YY_SCAN_CASE(CH) \
-  case CH: k_scan_tile<CH><<<blocks, kScanThreads, 0, st>>>(g->n_patch, g->n_r, g->lmax, g->n_lm, At, g->scan, (const double2 *)g->scan_prod, g->Q, q32); break;
+  case CH: return launch_kernel(g, "k_scan_tile", k_scan_tile<CH>, blocks, kScanThreads, 0, st, g->n_patch, g->n_r, g->lmax, g->n_lm, At, g->scan, (const double2 *)g->scan_prod, g->Q, q32);
       YY_SCAN_FORMS(YY_SCAN_CASE)
 #undef YY_SCAN_CASE
     }
-    note_launch(g, "k_scan_tile", st);
-    return cudaGetLastError();
   }
   // long radial grids: chunks spread over warps, two passes
   ScanGeom s;

@@ -63,6 +63,7 @@ __host__ __device__ constexpr int stride_g(int rows) { return rows + 2; }
 
 template <int NF>
 __global__ void __launch_bounds__(256, 3) k_synth_f64(const Synth64 a, int jp) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char smraw[];
   const int rp = rows64(NF, jp), ld = stride_g(rp), nt = 2 * a.lmax + 1;
   double *Gs = reinterpret_cast<double *>(smraw);                  // [nt][ld]
@@ -200,6 +201,7 @@ __host__ __device__ constexpr int theta_groups(int n_theta, int items) { return 
 
 template <int NF>
 __global__ void __launch_bounds__(kThetaThreads) k_theta32(const Synth32 a) {
+  pdl_begin();
   constexpr int S = kS32, NQ = NF == 4 ? 3 : 1;   // g_phi uses the coefficients of g_theta
   extern __shared__ __align__(16) unsigned char smraw[];
   float *qs = reinterpret_cast<float *>(smraw);   // [group][l - m][NQ][cos, sin][S]
@@ -302,6 +304,7 @@ constexpr int kPhiThreads = 256;
 // TRS: the trig table in shared memory (else read through L1); PAIR: rows of even length
 template <bool PAIR, bool TRS>
 __global__ void __launch_bounds__(kPhiThreads, 2) k_phi32(const Synth32 a, int n_fields) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char smraw[];
   const int nt = 2 * a.lmax + 1, cols = cols32(a.n_phi), ldk = TRS ? cols * kC32 : a.n_phi;
   const int size = nt * a.tile;   // a multiple of 8 values
@@ -454,9 +457,7 @@ cudaError_t run64(yy_grid *g, const Synth64 &a0, cudaStream_t s) {
   Synth64 a = a0;
   a.chunks = (pairs + jp - 1) / jp;
   jp = (pairs + a.chunks - 1) / a.chunks;   // even chunks
-  k_synth_f64<NF><<<(unsigned)(grid_rows(g) * a.chunks), 256, smem64<NF>(g->lmax, jp), s>>>(a, jp);
-  note_launch(g, "k_synth_f64", s);
-  return cudaGetLastError();
+  return launch_kernel(g, "k_synth_f64", k_synth_f64<NF>, (unsigned)(grid_rows(g) * a.chunks), 256, smem64<NF>(g->lmax, jp), s, a, jp);
 }
 
 // Rows per tile of the fp32 form: multiples of eight whose items (eight rows x
@@ -492,12 +493,9 @@ Phi32 phi32_shape(const yy_grid *g, int n_fields) {
 }
 
 template <bool PAIR>
-void launch_phi32(const yy_grid *g, const Synth32 &a, const Phi32 &f, int nf, cudaStream_t s) {
-  const int blocks = std::min(nf * a.tiles, 2 * g->sms);
-  if (f.trig_smem)
-    k_phi32<PAIR, true><<<blocks, kPhiThreads, f.tiles_smem + f.trig_smem, s>>>(a, nf);
-  else
-    k_phi32<PAIR, false><<<blocks, kPhiThreads, f.tiles_smem, s>>>(a, nf);
+cudaError_t launch_phi32(yy_grid *g, const Synth32 &a, const Phi32 &f, int nf, cudaStream_t s) {
+  return launch_kernel(g, "k_phi32", f.trig_smem ? k_phi32<PAIR, true> : k_phi32<PAIR, false>, std::min(nf * a.tiles, 2 * g->sms),
+                       kPhiThreads, f.tiles_smem + f.trig_smem, s, a, nf);
 }
 
 cudaError_t run32(yy_grid *g, Synth32 a, bool grad, cudaStream_t s) {
@@ -510,17 +508,9 @@ cudaError_t run32(yy_grid *g, Synth32 a, bool grad, cudaStream_t s) {
   while (a.items > 1 && qsm_of(a.items) > 100 * 1024) a.items /= 2;
   const size_t qsm = qsm_of(a.items);
   const dim3 theta((unsigned)(((a.n_shells + kS32 - 1) / kS32 * a.n_theta + a.items - 1) / a.items), (unsigned)(a.lmax / 2 + 1));
-  if (grad)
-    k_theta32<4><<<theta, kThetaThreads, qsm, s>>>(a);
-  else
-    k_theta32<1><<<theta, kThetaThreads, qsm, s>>>(a);
-  note_launch(g, "k_theta32", s);
-  if (g->n_phi % 2 == 0)
-    launch_phi32<true>(g, a, f, nf, s);
-  else
-    launch_phi32<false>(g, a, f, nf, s);
-  note_launch(g, "k_phi32", s);
-  return cudaGetLastError();
+  const cudaError_t e = launch_kernel(g, "k_theta32", grad ? k_theta32<4> : k_theta32<1>, theta, kThetaThreads, qsm, s, a);
+  if (e != cudaSuccess) return e;
+  return g->n_phi % 2 == 0 ? launch_phi32<true>(g, a, f, nf, s) : launch_phi32<false>(g, a, f, nf, s);
 }
 
 }  // namespace

@@ -128,6 +128,7 @@ struct SepPhi64 {
 };
 
 __global__ void k_sep_phi64(const SepPhi64 a) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char smraw[];
   double *xs = reinterpret_cast<double *>(smraw);   // [E even m, E odd m, O even m, O odd m][column][per]
   const int row0 = blockIdx.x * a.per, cols = a.fold.cols, plane = cols * a.per;
@@ -242,6 +243,7 @@ __device__ __forceinline__ void copy_async(float *dst, const float *src) {
 
 template <int kR32>
 __global__ void k_sep_phi32(const SepPhi32 a) {
+  pdl_begin();
   extern __shared__ __align__(16) float azs[];            // [2][kPiece][nt_pad]
   __shared__ __align__(16) double raw[kRows32][kPiece];
   __shared__ __align__(16) float wts[kRows32][kPiece];
@@ -356,6 +358,7 @@ template <int S>
 __global__ void k_sep_theta32(int n_shells, int n_theta, int n_lm, int lmax1, int nt_pad, const float *__restrict__ tb,
                               const float2 *__restrict__ tb0, const float *__restrict__ F, const float2 *__restrict__ F0,
                               double *__restrict__ A) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char smraw[];
   const int shell0 = blockIdx.x * S, ns = min(S, n_shells - shell0), rows = S * n_theta;
   float2 *f0s = reinterpret_cast<float2 *>(smraw);                 // [S][n_theta]
@@ -412,6 +415,7 @@ __global__ void k_sep_theta32(int n_shells, int n_theta, int n_lm, int lmax1, in
 // memory, one thread per mode.
 __global__ void k_sep_theta64(int n_theta, int n_lm, int nt_pad, const double *__restrict__ tb,
                                                      const double *__restrict__ F, double *__restrict__ A) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char smraw[];
   const int shell = blockIdx.x;
   const double *Fs = F + (size_t)shell * n_theta * nt_pad;
@@ -633,10 +637,8 @@ cudaError_t separable_theta_partials(yy_grid *g, SepThetaPartials a, cudaStream_
 
 cudaError_t separable_theta_f64(yy_grid *g, cudaStream_t s) {
   const int nt_pad = g->sep_nt_pad;
-  k_sep_theta64<<<grid_rows(g), theta_threads(g->n_lm, 0), theta_smem(g->n_theta, nt_pad, sizeof(double)), s>>>(g->n_theta, g->n_lm, nt_pad, g->tbar,
-                                                                                          g->sep_F, g->A);
-  note_launch(g, "k_sep_theta64", s);
-  return cudaGetLastError();
+  return launch_kernel(g, "k_sep_theta64", k_sep_theta64, grid_rows(g), theta_threads(g->n_lm, 0),
+                       theta_smem(g->n_theta, nt_pad, sizeof(double)), s, g->n_theta, g->n_lm, nt_pad, g->tbar, g->sep_F, g->A);
 }
 
 cudaError_t analysis_separable(yy_grid *g, const double *rho_yin, const double *rho_yang, bool fp64, cudaStream_t s) {
@@ -646,9 +648,8 @@ cudaError_t analysis_separable(yy_grid *g, const double *rho_yin, const double *
     const SepPhi64 a = {rows, per, g->n_r, g->n_theta, g->n_phi, m1, nt_pad, az_fold(g), rho_yin, rho_yang, g->w,
                         (const double2 *)g->sep_azf, g->sep_F};
     const int threads = std::max(64, (per / kR64 * m1 + 31) / 32 * 32);   // one item per thread (672 at l_max 80)
-    k_sep_phi64<<<(rows + per - 1) / per, threads, phi64_smem(a.fold, per), s>>>(a);
-    note_launch(g, "k_sep_phi64", s);
-    return separable_theta_f64(g, s);
+    const cudaError_t e = launch_kernel(g, "k_sep_phi64", k_sep_phi64, (rows + per - 1) / per, threads, phi64_smem(a.fold, per), s, a);
+    return e == cudaSuccess ? separable_theta_f64(g, s) : e;
   }
   const SepPhi32 a = {g->n_r, g->n_theta, g->n_phi, nt_pad, {rho_yin, rho_yang}, g->sep_w32, g->sep_az32, (float *)g->sep_F,
                       (float2 *)g->sep_F0};
@@ -657,26 +658,18 @@ cudaError_t analysis_separable(yy_grid *g, const double *rho_yin, const double *
   const int threads = std::max(32 * kLoadWarps, (kRows32 / R * tg + 31) / 32 * 32);   // one item per thread (352 at l_max 80)
   const dim3 blocks((unsigned)((g->n_r * g->n_theta + kRows32 - 1) / kRows32), (unsigned)g->n_patch);
   const size_t table = 2 * (size_t)kPiece * nt_pad * sizeof(float);
-  if (R == 2)
-    k_sep_phi32<2><<<blocks, threads, table, s>>>(a);
-  else
-    k_sep_phi32<4><<<blocks, threads, table, s>>>(a);
-  note_launch(g, "k_sep_phi32", s);
+  const cudaError_t e = launch_kernel(g, "k_sep_phi32", R == 2 ? k_sep_phi32<2> : k_sep_phi32<4>, blocks, threads, table, s, a);
+  if (e != cudaSuccess) return e;
   // shells per block: as many as leave every SM a block (and fit two blocks per SM)
   const size_t shell = theta_smem(g->n_theta, nt_pad, sizeof(float));
   const int shells = grid_rows(g), mode_threads = theta_threads(g->n_lm, 32);
   auto polar = [&](auto k, int S) {
-    k<<<(shells + S - 1) / S, mode_threads, S * shell, s>>>(shells, g->n_theta, g->n_lm, g->lmax + 1, nt_pad, g->sep_tb32, g->sep_tb0,
-                                                       (const float *)g->sep_F, (const float2 *)g->sep_F0, g->A);
+    return launch_kernel(g, "k_sep_theta32", k, (shells + S - 1) / S, mode_threads, S * shell, s, shells, g->n_theta, g->n_lm,
+                         g->lmax + 1, nt_pad, g->sep_tb32, g->sep_tb0, (const float *)g->sep_F, (const float2 *)g->sep_F0, g->A);
   };
-  if (shells >= 4 * g->sms && 4 * shell <= 113 * 1024)
-    polar(k_sep_theta32<4>, 4);
-  else if (shells >= 3 * g->sms && 2 * shell <= 113 * 1024)
-    polar(k_sep_theta32<2>, 2);
-  else
-    polar(k_sep_theta32<1>, 1);
-  note_launch(g, "k_sep_theta32", s);
-  return cudaGetLastError();
+  if (shells >= 4 * g->sms && 4 * shell <= 113 * 1024) return polar(k_sep_theta32<4>, 4);
+  if (shells >= 3 * g->sms && 2 * shell <= 113 * 1024) return polar(k_sep_theta32<2>, 2);
+  return polar(k_sep_theta32<1>, 1);
 }
 
 }  // namespace yy

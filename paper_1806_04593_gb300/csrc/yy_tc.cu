@@ -95,6 +95,7 @@ __device__ __forceinline__ void split8(const float (&y)[8], typename F::elem *ba
 
 template <class F>
 __global__ void __launch_bounds__(256) k_pack_rows(PackBatch batch) {
+  pdl_begin();
   extern __shared__ float rowbuf[];
   __shared__ double red[4][256];
   const PackArgs &p = batch.job[blockIdx.y];
@@ -357,6 +358,7 @@ __device__ __forceinline__ void pack_store(const PackArgs &p, int row, const dou
 template <class F, int TPR, int P>
 __global__ void __launch_bounds__(TPR > 256 ? TPR : 256, (TPR <= 32 && P <= 6) ? 4 : ((TPR <= 32 && P <= 12) ? 3 : 1))
 k_pack_reg(PackBatch batch) {
+  pdl_begin();
   constexpr int TPB = TPR > 256 ? TPR : 256;
   __shared__ RowStats red[32];
   const PackArgs &p = batch.job[blockIdx.y];
@@ -415,6 +417,7 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
 
 template <class F>
 __global__ void __launch_bounds__(1024, 1) k_pack_stream(PackArgs p, int *err) {
+  pdl_begin();
   extern __shared__ __align__(16) double rowbuf_f64[];
   __shared__ RowStats red[32];
   __shared__ __align__(8) uint64_t bar;
@@ -976,6 +979,7 @@ __global__ void k_reduce_partials(int M, int N, int S, const float *__restrict__
                                   const double *__restrict__ rs, const double *__restrict__ cs,
                                   const double *__restrict__ mono, const double *__restrict__ mean,
                                   const double *__restrict__ colsum, double *__restrict__ A) {
+  pdl_begin();
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (size_t)M * N) return;
   const int row = (int)(e / N), col = (int)(e % N);
@@ -1063,6 +1067,7 @@ __device__ __forceinline__ void reduce_rotate_block(const ReduceRotateArgs &ra, 
 }
 
 __global__ void __launch_bounds__(256) k_reduce_rotate(ReduceRotateArgs r) {
+  pdl_begin();
   reduce_rotate_block(r, (int)blockIdx.x, (int)blockIdx.y);
 }
 
@@ -1248,7 +1253,7 @@ static size_t pack_smem(const PackBatch &b, int n) {
 }
 
 template <class F>
-static cudaError_t launch_pack(PackBatch &b, int n, cudaStream_t s) {
+static cudaError_t launch_pack(yy_grid *g, const char *name, PackBatch &b, int n, cudaStream_t s) {
   int rows = 0, kp = 0;
   for (int i = 0; i < n; ++i) {
     b.job[i].cache = b.job[i].K <= kPackCacheMax ? 1 : 0;
@@ -1258,43 +1263,38 @@ static cudaError_t launch_pack(PackBatch &b, int n, cudaStream_t s) {
   // register-resident forms where the row fits, else the two-pass kernel
   const unsigned wblocks = (unsigned)((rows + 7) / 8);
   if (kp <= 32 * 8)
-    k_pack_reg<F, 32, 4><<<dim3(wblocks, n), 256, 0, s>>>(b);
+    return launch_kernel(g, name, k_pack_reg<F, 32, 4>, dim3(wblocks, n), 256, 0, s, b);
   else if (kp <= 32 * 12)
-    k_pack_reg<F, 32, 6><<<dim3(wblocks, n), 256, 0, s>>>(b);
+    return launch_kernel(g, name, k_pack_reg<F, 32, 6>, dim3(wblocks, n), 256, 0, s, b);
   else if (kp <= 32 * 24)
-    k_pack_reg<F, 32, 12><<<dim3(wblocks, n), 256, 0, s>>>(b);
+    return launch_kernel(g, name, k_pack_reg<F, 32, 12>, dim3(wblocks, n), 256, 0, s, b);
   else if (kp <= 32 * 64)
-    k_pack_reg<F, 32, 32><<<dim3(wblocks, n), 256, 0, s>>>(b);
+    return launch_kernel(g, name, k_pack_reg<F, 32, 32>, dim3(wblocks, n), 256, 0, s, b);
   else if (kp <= 1024 * 8)
-    k_pack_reg<F, 1024, 4><<<dim3(rows, n), 1024, 0, s>>>(b);
+    return launch_kernel(g, name, k_pack_reg<F, 1024, 4>, dim3(rows, n), 1024, 0, s, b);
   else if (kp <= 1024 * 16)
-    k_pack_reg<F, 1024, 8><<<dim3(rows, n), 1024, 0, s>>>(b);
+    return launch_kernel(g, name, k_pack_reg<F, 1024, 8>, dim3(rows, n), 1024, 0, s, b);
   else if (kp <= 1024 * 24)
-    k_pack_reg<F, 1024, 12><<<dim3(rows, n), 1024, 0, s>>>(b);
+    return launch_kernel(g, name, k_pack_reg<F, 1024, 12>, dim3(rows, n), 1024, 0, s, b);
   else
-    k_pack_rows<F><<<dim3(rows, n), 256, pack_smem(b, n), s>>>(b);
-  return cudaGetLastError();
+    return launch_kernel(g, name, k_pack_rows<F>, dim3(rows, n), 256, pack_smem(b, n), s, b);
 }
 
 // One job of long density rows: the streaming form where its rules hold
 // (16-byte aligned rows of an even length, nothing left out), else
 // launch_pack.
 template <class F>
-static cudaError_t launch_pack_long(PackBatch &b, int *err, cudaStream_t s) {
+static cudaError_t launch_pack_long(yy_grid *g, const char *name, PackBatch &b, cudaStream_t s) {
   const PackArgs &p = b.job[0];
   const bool fits = ((uintptr_t)p.src0 % 16) == 0 && ((uintptr_t)p.src1 % 16) == 0 && (p.ld % 2) == 0 &&
                     (p.K % 2) == 0 && p.wrow == nullptr && p.row_add == nullptr && p.zero_k0 < 0 &&
                     p.zero_k1 < 0 && p.zero_row < 0 && (p.dot_vec == nullptr || (uintptr_t)p.dot_vec % 8 == 0);
-  if (!fits || p.K <= 32 * 64 || p.K > kStreamMaxK || p.k_pad > kStreamMaxK) return launch_pack<F>(b, 1, s);
-  int dev = 0, n_sm = 0;
-  cudaGetDevice(&dev);
-  if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n_sm < 1) n_sm = 1;
-  const int grid = std::min(p.rows_pad, n_sm);
-  k_pack_stream<F><<<grid, 1024, (size_t)p.K * sizeof(double), s>>>(p, err);
-  return cudaGetLastError();
+  if (!fits || p.K <= 32 * 64 || p.K > kStreamMaxK || p.k_pad > kStreamMaxK) return launch_pack<F>(g, name, b, 1, s);
+  return launch_kernel(g, name, k_pack_stream<F>, std::min(p.rows_pad, g->sms), 1024, (size_t)p.K * sizeof(double), s, p, g->err);
 }
 
-static cudaLaunchConfig_t pair_config(int pairs, int smem, cudaStream_t s, cudaLaunchAttribute *attr) {
+// attr: two entries; overlap: the launch may overlap the end of the kernel before it
+static cudaLaunchConfig_t pair_config(int pairs, int smem, cudaStream_t s, cudaLaunchAttribute *attr, bool overlap = false) {
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
@@ -1304,8 +1304,9 @@ static cudaLaunchConfig_t pair_config(int pairs, int smem, cudaStream_t s, cudaL
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
+  attr[1] = overlap_attribute();
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = overlap ? 2 : 1;
   return cfg;
 }
 
@@ -1313,9 +1314,9 @@ template <class F>
 static cudaError_t launch_pair(yy_grid *g, yy_tc_tables *t, const PairMaps &maps, const PairArgs &a, cudaStream_t s) {
   const int tiles = a.cell_tiles * a.row_tiles * a.k_splits * a.n_jobs;
   const int pairs = tiles < t->pair_slots ? tiles : t->pair_slots;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   const int smem = a.stages * pair_stage_bytes<F>(a.bn) + kSmemFixed + (a.out_mode >= 2 ? kEpiStageBytes : 0);
-  cudaLaunchConfig_t cfg = pair_config(pairs, smem, s, attr);
+  cudaLaunchConfig_t cfg = pair_config(pairs, smem, s, attr, overlap_allowed(g));
   const cudaError_t e = a.out_mode == 2   ? cudaLaunchKernelEx(&cfg, k_tc_pair<F, 2>, maps, a)
                         : a.out_mode == 1 ? cudaLaunchKernelEx(&cfg, k_tc_pair<F, 1>, maps, a)
                                           : cudaLaunchKernelEx(&cfg, k_tc_pair<F, 0>, maps, a);
@@ -1397,7 +1398,7 @@ static yy_status prepare_separable_synthesis(yy_grid *g, yy_tc_tables *t) {
   p.scale_out = t->sp_trigs;
   p.scale_out_f = t->sp_trigs_f;
   p.out = t->sp_trig;
-  if (e == cudaSuccess) e = launch_pack<F>(b, 1, 0);
+  if (e == cudaSuccess) e = launch_pack<F>(nullptr, "", b, 1, 0);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   cudaFree(trig_rows);
   if (e != cudaSuccess) return YY_ERR_CUDA;
@@ -1465,7 +1466,7 @@ static yy_status prepare_separable_analysis(yy_grid *g, yy_tc_tables *t) {
   p.scale_out = t->san_azs;
   p.scale_out_f = t->san_azsf;
   p.out = t->san_az;
-  if ((e = cudaGetLastError()) == cudaSuccess) e = launch_pack<F>(b, 1, 0);
+  if ((e = cudaGetLastError()) == cudaSuccess) e = launch_pack<F>(nullptr, "", b, 1, 0);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   cudaFree(az_rows);
   if (e != cudaSuccess) return YY_ERR_CUDA;
@@ -1490,7 +1491,7 @@ static yy_status prepare_form(yy_grid *g, yy_tc_tables *t) {
   t->rows_pad = t->row_tiles * t->bn;
   t->stages = pair_stages<F>(t->bn);
   {
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = pair_config(64, t->stages * pair_stage_bytes<F>(t->bn) + kSmemFixed, 0, attr);
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, (void *)k_tc_pair<F, 1>, &cfg) != cudaSuccess || n < 1) {
@@ -1561,7 +1562,7 @@ static yy_status prepare_form(yy_grid *g, yy_tc_tables *t) {
   p.zero_row = 0;
   p.scale_out = t->an_tabs;
   p.out = t->an_tab;
-  if ((e = launch_pack<F>(b, 1, 0)) != cudaSuccess) return YY_ERR_CUDA;
+  if ((e = launch_pack<F>(nullptr, "", b, 1, 0)) != cudaSuccess) return YY_ERR_CUDA;
   const double *tabs[3] = {g->ysyn, g->ysyn_t, g->ysyn_p};
   PackBatch bs = {};
   for (int c = 0; c < 3; ++c) {
@@ -1579,7 +1580,7 @@ static yy_status prepare_form(yy_grid *g, yy_tc_tables *t) {
     q.scale_out_f = t->sy_tabsf[c];
     q.out = t->sy_tab[c];
   }
-  if ((e = launch_pack<F>(bs, 3, 0)) != cudaSuccess) return YY_ERR_CUDA;
+  if ((e = launch_pack<F>(nullptr, "", bs, 3, 0)) != cudaSuccess) return YY_ERR_CUDA;
   if ((e = cudaDeviceSynchronize()) != cudaSuccess) return YY_ERR_CUDA;
 
   const int bh = t->bn / 2;
@@ -1754,8 +1755,7 @@ static cudaError_t analysis_form(yy_grid *g, yy_tc_tables *t, const double *ry, 
   PackBatch b = {};
   PairArgs a;
   analysis_args<F>(g, t, ry, rg, b.job[0], a);
-  cudaError_t e = launch_pack_long<F>(b, g->err, s);
-  note_launch(g, "k_pack_stream", s);
+  cudaError_t e = launch_pack_long<F>(g, "k_pack_stream", b, s);
   if (e != cudaSuccess) return e;
   if ((e = launch_pair<F>(g, t, t->an_maps, a, s)) != cudaSuccess) return e;
   if (g->n_patch == 2 && g->lmax <= kReduceRotateLmax) {
@@ -1763,18 +1763,13 @@ static cudaError_t analysis_form(yy_grid *g, yy_tc_tables *t, const double *ry, 
     ReduceRotateArgs r;
     reduce_rotate_args(g, t, r);
     const dim3 grid((unsigned)g->n_r, (unsigned)((g->n_lm + 255) / 256));
-    k_reduce_rotate<<<grid, 256, 0, s>>>(r);
-    note_launch(g, "k_reduce_rotate", s);
     g->atot_done = 1;
-    return cudaGetLastError();
+    return launch_kernel(g, "k_reduce_rotate", k_reduce_rotate, grid, 256, 0, s, r);
   }
   const int M = grid_rows(g);
   const size_t cnt = (size_t)M * g->n_lm;
-  k_reduce_partials<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(M, g->n_lm, t->an_segs, t->part, t->an_rhos,
-                                                                  t->an_tabs, t->an_mono, t->an_mean, t->an_colsum,
-                                                                  g->A);
-  note_launch(g, "k_reduce_partials", s);
-  return cudaGetLastError();
+  return launch_kernel(g, "k_reduce_partials", k_reduce_partials, (unsigned)((cnt + 255) / 256), 256, 0, s, M, g->n_lm, t->an_segs,
+                       t->part, t->an_rhos, t->an_tabs, t->an_mono, t->an_mean, t->an_colsum, g->A);
 }
 
 // The three coefficient sets' packing (Phi and g_r: the monopole, column 0,
@@ -1808,9 +1803,7 @@ template <class F>
 static cudaError_t pack_coefficients_form(yy_grid *g, yy_tc_tables *t, cudaStream_t s) {
   PackBatch b = {};
   coefficient_args(g, t, b.job);
-  cudaError_t e = launch_pack<F>(b, 3, s);
-  note_launch(g, "k_pack_reg/coefficients", s);
-  return e;
+  return launch_pack<F>(g, "k_pack_reg/coefficients", b, 3, s);
 }
 
 template <class F>
@@ -2014,8 +2007,7 @@ static cudaError_t separable_analysis_form(yy_grid *g, yy_tc_tables *t, const do
   p.out = t->san_x;
   p.wrow = g->sep_w32;            // rho w
   p.w_rows = g->n_theta;
-  cudaError_t e = launch_pack<F>(b, 1, s);
-  note_launch(g, "k_pack_reg/rho_rows", s);
+  cudaError_t e = launch_pack<F>(g, "k_pack_reg/rho_rows", b, 1, s);
   if (e != cudaSuccess) return e;
   PairArgs a = {};
   a.stages = t->san_stages;
@@ -2220,6 +2212,7 @@ constexpr int kQffShells = 8, kQffChunk = 512;
 constexpr size_t kQffOnePassSmem = 200 * 1024;
 
 __global__ void __launch_bounds__(512) k_q_ff(OzQffArgs a) {
+  pdl_begin();
   extern __shared__ float2 qrow[];                         // one_pass: [8][n_lm]; else [kQffChunk][8 + 1]
   __shared__ unsigned long long part[2][kQffShells];
   float2 (*tile)[kQffShells + 1] = reinterpret_cast<float2 (*)[kQffShells + 1]>(qrow);
@@ -2510,6 +2503,7 @@ inline size_t theta_ff_smem(int lmax, int gk) {
 // orders m at a time (m and l_max + 1 - m, about 2 (l_max + 1) terms).
 template <int NG>
 __global__ void __launch_bounds__(512, 2) k_theta_ff(OzThetaFFArgs a) {
+  pdl_begin();
   constexpr int TP = NG == 1 ? 2 : 1;
   constexpr int R = 2 * TP;
   extern __shared__ float4 ffsm4[];
@@ -2690,6 +2684,7 @@ static_assert(kSepFFShells == 2, "k_sep_theta_ff packs its two shells into one f
 __global__ void __launch_bounds__(512) k_sep_theta_ff(int n_shells, int n_theta, int n_lm, int nt, int nt_pad,
                                                       const float2 *__restrict__ tbf, const double *__restrict__ F,
                                                       double *__restrict__ A) {
+  pdl_begin();
   // [2][half][nt_pad]: S, then D, both shells' values as one packed pair
   // (hi of shell 0, hi of shell 1, lo of shell 0, lo of shell 1)
   extern __shared__ float4 sdf[];
@@ -2838,6 +2833,7 @@ constexpr int kRotRadii = 4;
 
 __global__ void __launch_bounds__(256) k_rotate_ff(int n_r, int n_lm, int lmax, const float2 *__restrict__ Df,
                                                    const double *__restrict__ A, double *__restrict__ Atot) {
+  pdl_begin();
   extern __shared__ float2 rsm[];                          // [w][w] D^l, then [kRotRadii][2 w] moment pairs
   __shared__ int rexp[kRotRadii];
   const int tiles = (n_r + kRotRadii - 1) / kRotRadii;
@@ -2933,6 +2929,7 @@ struct OzRhoArgs {
 // digits of one slice go out as one 32-bit store of their bf16 patterns.
 template <int C>
 __global__ void __launch_bounds__(256) k_rhow_ozaki(OzRhoArgs a) {
+  pdl_begin();
   const int row = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (row >= a.rows) return;
   const int shell = row / a.n_theta, j = row % a.n_theta;
@@ -3080,7 +3077,7 @@ static yy_status ozaki_prepare_analysis(yy_grid *g, yy_oz_tables *o) {
       cudaFuncSetAttribute(k_tc_pair<F, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess)
     return YY_OK;
   {
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg =
         pair_config(64, o->an_stages * pair_stage_bytes<F>(o->an_bn) + kSmemFixed + kEpiStageBytes, 0, attr);
     int n = 0;
@@ -3132,7 +3129,7 @@ static yy_status ozaki_prepare_analysis(yy_grid *g, yy_oz_tables *o) {
   if (nt <= kOzAnBN && make_map<F>(&o->an_maps2.a, o->an_x, o->an_kpad, F::kPA * o->rows_pad, kPairRows) &&
       make_map<F>(&o->an_maps2.b, o->an_az, o->an_kpad, F::kPB * o->an_b_rows_pad, kOzAnBN) &&
       cudaFuncSetAttribute(k_oz_analysis, cudaFuncAttributeMaxDynamicSharedMemorySize, kOzAnSmem) == cudaSuccess) {
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = pair_config(64, kOzAnSmem, 0, attr);
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, (void *)k_oz_analysis, &cfg) == cudaSuccess && n > 0) o->an_slots2 = n;
@@ -3147,10 +3144,9 @@ static cudaError_t ozaki_theta_analysis(yy_grid *g, cudaStream_t s) {
   const size_t smem = (size_t)kSepFFShells * 2 * half * g->sep_nt_pad * sizeof(float2);
   if (smem > 200 * 1024) return separable_theta_f64(g, s);
   const int shells = grid_rows(g);
-  k_sep_theta_ff<<<(unsigned)((shells + kSepFFShells - 1) / kSepFFShells), sep_theta_ff_threads(g->n_lm), smem, s>>>(
-      shells, g->n_theta, g->n_lm, 2 * g->lmax + 1, g->sep_nt_pad, g->oz->tbf, g->sep_F, g->A);
-  note_launch(g, "k_sep_theta_ff", s);
-  return cudaGetLastError();
+  return launch_kernel(g, "k_sep_theta_ff", k_sep_theta_ff, (unsigned)((shells + kSepFFShells - 1) / kSepFFShells),
+                       sep_theta_ff_threads(g->n_lm), smem, s, shells, g->n_theta, g->n_lm, 2 * g->lmax + 1, g->sep_nt_pad,
+                       g->oz->tbf, g->sep_F, g->A);
 }
 
 cudaError_t ozaki_analysis(yy_grid *g, const double *ry, const double *rg, cudaStream_t s) {
@@ -3171,12 +3167,7 @@ cudaError_t ozaki_analysis(yy_grid *g, const double *ry, const double *rg, cudaS
   ra.rexp = o->an_exp;
   const unsigned blocks = (unsigned)(((size_t)o->rows * 32 + 255) / 256);
   constexpr int kCmax = FormOzaki::kFillK * FormOzaki::kMaxFills / 64;
-  if (o->an_kpad <= 64 * 5)
-    k_rhow_ozaki<5><<<blocks, 256, 0, s>>>(ra);
-  else
-    k_rhow_ozaki<kCmax><<<blocks, 256, 0, s>>>(ra);
-  note_launch(g, "k_rhow_ozaki", s);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_kernel(g, "k_rhow_ozaki", o->an_kpad <= 64 * 5 ? k_rhow_ozaki<5> : k_rhow_ozaki<kCmax>, blocks, 256, 0, s, ra);
   if (e != cudaSuccess) return e;
   if (o->an_slots2 > 0) {
     OzAnalysisArgs z = {};
@@ -3192,8 +3183,8 @@ cudaError_t ozaki_analysis(yy_grid *g, const double *ry, const double *rg, cudaS
     z.cell_exp = o->an_exp;
     z.err = g->err;
     const int pairs = z.cell_tiles < o->an_slots2 ? z.cell_tiles : o->an_slots2;
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = pair_config(pairs, kOzAnSmem, s, attr);
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = pair_config(pairs, kOzAnSmem, s, attr, overlap_allowed(g));
     e = cudaLaunchKernelEx(&cfg, k_oz_analysis, o->an_maps2, z);
     note_launch(g, "k_oz_analysis", s);
     if (e != cudaSuccess) return e;
@@ -3224,9 +3215,9 @@ cudaError_t ozaki_analysis(yy_grid *g, const double *ry, const double *rg, cudaS
   a.job[0].tb = 0;
   const int tiles = a.cell_tiles * a.row_tiles;
   const int pairs = tiles < o->an_slots ? tiles : o->an_slots;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg =
-      pair_config(pairs, o->an_stages * pair_stage_bytes<F>(o->an_bn) + kSmemFixed + kEpiStageBytes, s, attr);
+      pair_config(pairs, o->an_stages * pair_stage_bytes<F>(o->an_bn) + kSmemFixed + kEpiStageBytes, s, attr, overlap_allowed(g));
   e = cudaLaunchKernelEx(&cfg, k_tc_pair<F, 3>, o->an_maps, a);
   note_launch(g, "k_tc_pair<FormOzaki,3>/analysis", s);
   if (e != cudaSuccess) return e;
@@ -3238,9 +3229,7 @@ cudaError_t ozaki_rotate(yy_grid *g, cudaStream_t s) {
   const int w = 2 * g->lmax + 1;
   const size_t smem = ((size_t)w * w + (size_t)kRotRadii * 2 * w) * sizeof(float2);
   const unsigned blocks = (unsigned)((g->lmax + 1) * ((g->n_r + kRotRadii - 1) / kRotRadii));
-  k_rotate_ff<<<blocks, 256, smem, s>>>(g->n_r, g->n_lm, g->lmax, g->oz->Df, g->A, g->Atot);
-  note_launch(g, "k_rotate_ff", s);
-  return cudaGetLastError();
+  return launch_kernel(g, "k_rotate_ff", k_rotate_ff, blocks, 256, smem, s, g->n_r, g->n_lm, g->lmax, g->oz->Df, g->A, g->Atot);
 }
 
 // balanced base-1024 digits of X <= 2^49 (most significant first): each in
@@ -3400,7 +3389,7 @@ yy_status ozaki_prepare(yy_grid *g) {
     const int smem = o->gk == 64 ? oz_synth_smem<2>() : oz_synth_smem<4>();
     int n = 0;
     if (ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess) {
-      cudaLaunchAttribute attr[1];
+      cudaLaunchAttribute attr[2];
       cudaLaunchConfig_t cfg = pair_config(64, smem, 0, attr);
       cfg.blockDim = dim3(kOzThreads);
       if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) n = 0;
@@ -3439,9 +3428,9 @@ cudaError_t ozaki_synthesis(yy_grid *g, double *py, double *pg, double *gy, doub
   qa.qexp = o->qexp;
   const size_t qff_smem = (size_t)kQffShells * g->n_lm * sizeof(float2);
   qa.one_pass = qff_smem <= kQffOnePassSmem ? 1 : 0;
-  k_q_ff<<<(unsigned)(n_q * (o->shells_pad / kQffShells)), 64 * kQffShells,
-           qa.one_pass ? qff_smem : (size_t)kQffChunk * (kQffShells + 1) * sizeof(float2), s>>>(qa);
-  note_launch(g, "k_q_ff", s);
+  cudaError_t e = launch_kernel(g, "k_q_ff", k_q_ff, (unsigned)(n_q * (o->shells_pad / kQffShells)), 64 * kQffShells,
+                                qa.one_pass ? qff_smem : (size_t)kQffChunk * (kQffShells + 1) * sizeof(float2), s, qa);
+  if (e != cudaSuccess) return e;
   OzThetaFFArgs fa = {};
   fa.n_shells = n_shells;
   fa.shells_pad = o->shells_pad;
@@ -3469,12 +3458,7 @@ cudaError_t ozaki_synthesis(yy_grid *g, double *py, double *pg, double *gy, doub
   const unsigned ff_blocks = (unsigned)(n_q * (o->shells_pad / 32) * ((fa.half + tp - 1) / tp));
   const unsigned ff_threads = (unsigned)(32 * (n_groups < 16 ? n_groups : 16));
   const size_t ff_smem = theta_ff_smem(g->lmax, o->gk);
-  if (o->gk == 64)
-    k_theta_ff<1><<<ff_blocks, ff_threads, ff_smem, s>>>(fa);
-  else
-    k_theta_ff<2><<<ff_blocks, ff_threads, ff_smem, s>>>(fa);
-  note_launch(g, "k_theta_ff", s);
-  cudaError_t e = cudaGetLastError();
+  e = launch_kernel(g, "k_theta_ff", o->gk == 64 ? k_theta_ff<1> : k_theta_ff<2>, ff_blocks, ff_threads, ff_smem, s, fa);
   if (e != cudaSuccess) return e;
   const size_t comp = (size_t)g->n_r * g->n_ang;
   double *o0[4] = {py, gy, gy ? gy + comp : nullptr, gy ? gy + 2 * comp : nullptr};
@@ -3500,8 +3484,8 @@ cudaError_t ozaki_synthesis(yy_grid *g, double *py, double *pg, double *gy, doub
   }
   const int tiles = z.cell_tiles * n_jobs;
   const int pairs = tiles < o->synth_slots ? tiles : o->synth_slots;
-  cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = pair_config(pairs, o->gk == 64 ? oz_synth_smem<2>() : oz_synth_smem<4>(), s, attr);
+  cudaLaunchAttribute attr[2];
+  cudaLaunchConfig_t cfg = pair_config(pairs, o->gk == 64 ? oz_synth_smem<2>() : oz_synth_smem<4>(), s, attr, overlap_allowed(g));
   cfg.blockDim = dim3(kOzThreads);
   e = o->gk == 64 ? cudaLaunchKernelEx(&cfg, k_oz_synth<2>, o->synth_maps, z)
                   : cudaLaunchKernelEx(&cfg, k_oz_synth<4>, o->synth_maps, z);
@@ -3714,7 +3698,7 @@ static yy_status group_build(yy_grid *const *grids, int n, yy_precision prec, co
         cudaFuncSetAttribute(k_tc_pair<F, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) !=
             cudaSuccess)
       return YY_ERR_NOT_SUPPORTED;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = pair_config(64, smem, 0, attr);
     if (cudaOccupancyMaxActiveClusters(&slots, (void *)k_tc_pair<F, 1, true>, &cfg) != cudaSuccess || slots < 1) {
       cudaGetLastError();
@@ -3735,7 +3719,7 @@ static cudaError_t group_run(const TcGroup *G, cudaStream_t s) {
   if (G->rs_nblocks > 0) k_pack_group<F, 32><<<G->rs_nblocks, 256, 0, s>>>(G->rs_jobs, G->rs_map, G->rs_class);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = pair_config(G->an_pairs, G->an_smem, s, attr);
   if ((e = cudaLaunchKernelEx(&cfg, k_tc_pair<F, 0, true>, none, G->an_top)) != cudaSuccess) return e;
   k_reduce_rotate_group<<<G->rr_nblocks, 256, 0, s>>>(G->rr, G->rr_map);

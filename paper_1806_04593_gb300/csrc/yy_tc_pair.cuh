@@ -497,6 +497,7 @@ __device__ __forceinline__ bool pair_tile_next(const PairArgs &a0, int pair, int
 template <class F, int OUT_MODE, bool GROUPED = false>
 __global__ void __launch_bounds__(kThreads, 1)
 k_tc_pair(const __grid_constant__ PairMaps maps0, const __grid_constant__ PairArgs a0) {
+  pdl_wait();
   constexpr int A_SLOT = kPairRows * kRowBytes;
   constexpr int KSTEP_BYTES = 32;
   constexpr int KSTEPS = kRowBytes / KSTEP_BYTES;
