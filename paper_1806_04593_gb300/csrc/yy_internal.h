@@ -112,13 +112,16 @@ struct yy_grid {
 
 namespace yy {
 
-// The azimuthal cells folded by their symmetries: column c < half stands for
-// cells first + c and its mirror n_phi - 1 - (first + c) about phi = 0 (phi = pi
-// on the polar grid).  Where pi is a whole number of cells, cells phi and
-// pi - phi are columns c and partner - c (partner = -1: they are not cells);
-// columns c < cols then stand for all of them.
+// The azimuthal cells folded by their symmetries.  A folded column c < half is
+// cell first + c, at an angle phi_c in [0, pi] from the mirror axis, and its mirror
+// n_phi - 1 - (first + c) at -phi_c (about phi = 0, phi = pi on the polar grid).
+// Where pi is a whole number of cells, pi - phi_c is column partner - c (else
+// partner = -1); where pi / 2 is, pi / 2 - phi_c and pi / 2 + phi_c are columns
+// quarter - odd - c and quarter + c (else quarter = 0; odd: cell centres at half
+// cells from the axis).  The columns c < cols stand for all of them (those whose
+// images are not cells of the grid, or are the column itself, for fewer).
 struct AzFold {
-  int half, cols, first, partner;
+  int half, cols, first, partner, quarter, odd;
 };
 AzFold az_fold(const yy_grid *g);
 
@@ -150,9 +153,11 @@ inline const double *moments_total(const yy_grid *g) { return g->n_patch == 2 ? 
 // idle, and the launch itself takes about a microsecond): every such kernel first
 // lets its successor do the same (pdl_begin) and then waits until its predecessor
 // has completed and its writes are visible.  Nothing is read or written before that.
-// The persistent tensor-core kernels only wait: their successors' blocks would
-// stay beside them for the whole run (134 us instead of 124 for a solve of 200
-// zones on 2-degree cells by YY_FP64_OZAKI; 133 without any overlap).
+// The persistent tensor-core kernels, and the ones that they follow, only wait: a
+// successor's blocks would stay beside the former for the whole run, and after the
+// latter the clusters would take the first SMs that come free (134 us instead of 124 for a solve of 200 zones on 2-degree
+// cells by YY_FP64_OZAKI, 133 without any overlap; 128 instead of 117 for 149 zones on a
+// 77 x 154 polar grid by YY_BF16X3, 122 without).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

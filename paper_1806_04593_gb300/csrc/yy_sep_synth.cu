@@ -38,13 +38,16 @@ struct SynthOut {
 //  - phi, where pi is a whole number of cells: cell phi also pairs with cell
 //    pi - phi, where cos(m phi) takes the sign (-1)^m and sin(m phi) -(-1)^m;
 //    the sums over even and odd m apart give up to four cells.
-// A column c stands for the cells at +-phi_c and, when partner >= 0 and
-// partner - c is another cell of the grid, at +-(pi - phi_c).  On the 1-degree
-// Yin-Yang grid 90 columns give the 270 cells: 18.7 float64 operations per
-// output at l_max 25 instead of 51.  Measured there, 550 zones, with the
-// gradient: 3.98 ms, 0.9 of the pipe's rate (1.9 a clock measured), against
-// 12.9 ms for one thread per four cells without the folds; 2-degree grid, 200
-// zones, l_max 15: 289 us against 707.
+//  - phi, where pi / 2 is one too: pi / 2 -+ phi.  Even orders keep their functions
+//    there up to signs that follow m mod 4, odd orders exchange cos and sin: sums
+//    of even m apart by m mod 4 (one product per slot) and of odd m with both
+//    functions (two per slot) give up to eight cells.
+// Columns and their images: AzFold.  On the 1-degree Yin-Yang grid 45 columns
+// give the 270 cells: 15.5 float64 operations per output at l_max 25 instead of
+// 51 (18.7 with pi - phi alone).  Measured there, 550 zones, with the gradient:
+// 3.27 ms, against 3.98 ms with pi - phi alone and 12.9 ms for one thread
+// per four cells without the folds; 2-degree grid, 200 zones, l_max 15: 246 us,
+// 289 and 707.
 struct Synth64 {
   int n_r, n_theta, n_phi, lmax, n_lm, chunks;
   AzFold fold;
@@ -54,14 +57,76 @@ struct Synth64 {
 };
 
 // rows of G in shared memory: (field, row pair of the chunk, side), padded to
-// the phi stage's groups of four
+// the phi stage's groups of four (two with the quarter fold)
 constexpr int kR64 = 4;
 __host__ __device__ constexpr int rows64(int nf, int jp) { return (2 * nf * jp + kR64 - 1) / kR64 * kR64; }
 // row stride of G: the theta stage's lanes write consecutive slots t, and two
 // more values than the rows keep those writes off one another's banks
 __host__ __device__ constexpr int stride_g(int rows) { return rows + 2; }
 
-template <int NF>
+// The phi stage of two rows at one column, every fold in use.
+__device__ __forceinline__ void phi_quarter(const Synth64 &a, const double *g, int ld, int c, double *const *dst) {
+  constexpr int R = 2;
+  // even m: cos and sin slots by m mod 4; odd m: cos slots with cos and with
+  // sigma sin, sin slots with sin and with sigma cos (sigma = +1, -1 for m mod 4 = 1, 3)
+  double c0[R] = {}, c2[R] = {}, s0[R] = {}, s2[R] = {}, cc[R] = {}, cs[R] = {}, ss[R] = {}, sc[R] = {};
+  const int nb = a.fold.cols;
+  const double *tr = a.tr + c;
+  auto even = [&](int m, double (&x)[R], double (&y)[R]) {
+    const double tc = tr[(size_t)(2 * m - 1) * nb], ts = tr[(size_t)(2 * m) * nb];
+    const double2 u = *reinterpret_cast<const double2 *>(g + (size_t)(2 * m - 1) * ld);
+    const double2 v = *reinterpret_cast<const double2 *>(g + (size_t)(2 * m) * ld);
+    x[0] = fma(u.x, tc, x[0]);
+    x[1] = fma(u.y, tc, x[1]);
+    y[0] = fma(v.x, ts, y[0]);
+    y[1] = fma(v.y, ts, y[1]);
+  };
+  auto odd = [&](int m, bool minus) {
+    const double tc = tr[(size_t)(2 * m - 1) * nb], ts = tr[(size_t)(2 * m) * nb];
+    const double xc = minus ? -tc : tc, xs = minus ? -ts : ts;
+    const double2 u = *reinterpret_cast<const double2 *>(g + (size_t)(2 * m - 1) * ld);
+    const double2 v = *reinterpret_cast<const double2 *>(g + (size_t)(2 * m) * ld);
+    cc[0] = fma(u.x, tc, cc[0]);
+    cc[1] = fma(u.y, tc, cc[1]);
+    cs[0] = fma(u.x, xs, cs[0]);
+    cs[1] = fma(u.y, xs, cs[1]);
+    ss[0] = fma(v.x, ts, ss[0]);
+    ss[1] = fma(v.y, ts, ss[1]);
+    sc[0] = fma(v.x, xc, sc[0]);
+    sc[1] = fma(v.y, xc, sc[1]);
+  };
+  int m = a.lmax;
+  if ((m & 3) == 3) odd(m--, true);
+  if ((m & 3) == 2) even(m--, c2, s2);
+  if ((m & 3) == 1) odd(m--, false);
+  for (; m > 0; m -= 4) {
+    even(m, c0, s0);
+    odd(m - 1, true);
+    even(m - 2, c2, s2);
+    odd(m - 3, false);
+  }
+  const int h = a.fold.half, first = a.fold.first, q = a.fold.quarter;
+  const int kb = q - a.fold.odd - c, kc = q + c, kd = a.fold.partner - c;   // pi/2 - phi, pi/2 + phi, pi - phi
+  const bool wb = kb != c && kb < h, wc = kc != kb && kc < h, wd = kd != kc && kd != c && kd < h;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    double *o = dst[r];
+    if (o == nullptr) continue;
+    const double cz = c0[r] + g[r];   // m = 0
+    const double e1 = cz + c2[r], e2 = cz - c2[r], f1 = s0[r] + s2[r], f2 = s0[r] - s2[r];
+    auto put = [&](int col, double C, double S) {
+      const int kp = first + col, km = a.n_phi - 1 - kp;
+      o[kp] = C + S;
+      if (km != kp) o[km] = C - S;
+    };
+    put(c, e1 + cc[r], f1 + ss[r]);
+    if (wb) put(kb, e2 + cs[r], sc[r] - f2);
+    if (wc) put(kc, e2 - cs[r], sc[r] + f2);
+    if (wd) put(kd, e1 - cc[r], ss[r] - f1);
+  }
+}
+
+template <int NF, bool QUARTER>
 __global__ void __launch_bounds__(256, 3) k_synth_f64(const Synth64 a, int jp) {
   pdl_begin();
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -121,8 +186,12 @@ __global__ void __launch_bounds__(256, 3) k_synth_f64(const Synth64 a, int jp) {
       Gs[(size_t)(e / (rp - 2 * NF * jp)) * ld + 2 * NF * jp + e % (rp - 2 * NF * jp)] = 0.0;
   __syncthreads();
 
-  // phi stage: one thread per (group of four rows, column)
+  // phi stage: one thread per (group of four rows, or two, and column)
   const int nb = a.fold.cols;
+  if constexpr (QUARTER) {
+    for (int e = threadIdx.x; e < rp / 2 * nb; e += blockDim.x) phi_quarter(a, Gs + e / nb * 2, ld, e % nb, dst + e / nb * 2);
+    return;
+  }
   for (int e = threadIdx.x; e < rp / kR64 * nb; e += blockDim.x) {
     const int r0 = e / nb * kR64, c = e % nb;
     double ce[kR64], co[kR64], se[kR64], so[kR64];   // cos / sin slots of even / odd m
@@ -457,7 +526,8 @@ cudaError_t run64(yy_grid *g, const Synth64 &a0, cudaStream_t s) {
   Synth64 a = a0;
   a.chunks = (pairs + jp - 1) / jp;
   jp = (pairs + a.chunks - 1) / a.chunks;   // even chunks
-  return launch_kernel(g, "k_synth_f64", k_synth_f64<NF>, (unsigned)(grid_rows(g) * a.chunks), 256, smem64<NF>(g->lmax, jp), s, a, jp);
+  return launch_kernel(g, "k_synth_f64", a.fold.quarter > 0 ? k_synth_f64<NF, true> : k_synth_f64<NF, false>,
+                       (unsigned)(grid_rows(g) * a.chunks), 256, smem64<NF>(g->lmax, jp), s, a, jp);
 }
 
 // Rows per tile of the fp32 form: multiples of eight whose items (eight rows x
@@ -521,15 +591,18 @@ AzFold az_fold(const yy_grid *g) {
   const bool polar = g->n_patch == 1;
   f.first = polar ? 0 : g->n_phi / 2;
   // cells to phi = pi from the mirror axis: whole when the quotient is one to rounding
-  f.partner = -1;
+  int whole = 0;
   if (polar) {
-    if (g->n_phi % 2 == 0) f.partner = g->n_phi / 2 - 1;
+    whole = g->n_phi % 2 == 0 ? g->n_phi / 2 : 0;
   } else {
-    const double cells = 3.141592653589793238462643383279502884 / g->dph, whole = rint(cells);
-    if (fabs(cells - whole) <= 4.0 * 2.220446049250313e-16 * whole && whole < 1e6)
-      f.partner = (int)whole - (g->n_phi % 2 == 0 ? 1 : 0);
+    const double cells = 3.141592653589793238462643383279502884 / g->dph, near = rint(cells);
+    if (fabs(cells - near) <= 4.0 * 2.220446049250313e-16 * near && near < 1e6) whole = (int)near;
   }
-  f.cols = f.partner >= 0 ? std::min(f.half, f.partner / 2 + 1) : f.half;
+  f.odd = polar || g->n_phi % 2 == 0 ? 1 : 0;
+  f.partner = whole > 0 ? whole - f.odd : -1;
+  f.quarter = whole > 0 && whole % 2 == 0 ? whole / 2 : 0;
+  f.cols = f.quarter > 0 ? (f.odd ? (f.quarter + 1) / 2 : f.quarter / 2 + 1) : f.partner >= 0 ? f.partner / 2 + 1 : f.half;
+  f.cols = std::min(f.half, f.cols);
   return f;
 }
 
@@ -541,7 +614,8 @@ cudaError_t synthesis_separable_prepare(yy_grid *g) {
   if (e != cudaSuccess) return e;
   k_fold_trig<<<(nt * f.cols + 255) / 256, 256>>>(nt, g->n_phi, f, g->sep_tr, g->sep_trf);
   k_inv_sin<<<(g->n_theta + 255) / 256, 256>>>(g->n_theta, g->th0, g->dth, g->sep_isin);
-  for (auto k : {(const void *)k_synth_f64<1>, (const void *)k_synth_f64<4>, (const void *)k_theta32<1>, (const void *)k_theta32<4>,
+  for (auto k : {(const void *)k_synth_f64<1, false>, (const void *)k_synth_f64<4, false>, (const void *)k_synth_f64<1, true>,
+                 (const void *)k_synth_f64<4, true>, (const void *)k_theta32<1>, (const void *)k_theta32<4>,
                  (const void *)k_phi32<true, true>, (const void *)k_phi32<true, false>,
                  (const void *)k_phi32<false, true>, (const void *)k_phi32<false, false>})
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);

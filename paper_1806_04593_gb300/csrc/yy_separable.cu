@@ -111,12 +111,16 @@ __device__ __forceinline__ void pair_fma(float &h, float &l, float ah, float al,
 // sets the time, so the cells are folded by their symmetries first (AzFold):
 // with E, O the sum and difference of a cell and its mirror, cos slots take E
 // and sin slots O over half the columns; where cells phi and pi - phi both
-// exist, E +- E' and O -+ O' serve the even and odd orders over a third of them
-// (on the 1-degree Yin-Yang grid 90 columns for 270 cells: 19.7 float64
-// operations per cell instead of 52; 0.97 ms there at 550 zones and l_max 25
-// against 3.02 ms without the folds, 72 against 214 us on the 2-degree grid of
-// 200 zones at l_max 15).  A block takes up to 16 consecutive rows
-// (shell, j); each thread then sums both slots of an order m for two rows.
+// exist, E +- E' and O -+ O' serve the even and odd orders over a third of them;
+// where pi / 2 is a whole number of cells, the columns at phi, pi / 2 -+ phi and
+// pi - phi (A, B, C, D) become one: even orders take sums of the four by m mod 4 with
+// one product per slot, odd orders A and D with their own function and B and C with
+// the other one (on the 1-degree Yin-Yang grid 45 columns for 270 cells: 16.2
+// float64 operations per cell instead of 52; 0.89 ms there at 550 zones and
+// l_max 25 against 0.97 ms with pi - phi alone and 3.02 ms without the folds,
+// 62 us, 72 and 214 on the 2-degree grid of 200 zones at l_max 15).  A
+// block takes up to 16 consecutive rows (shell, j); each thread then sums both
+// slots of an order m for two rows.
 constexpr int kR64 = 2;
 
 struct SepPhi64 {
@@ -127,63 +131,113 @@ struct SepPhi64 {
   double *F;
 };
 
+// planes of the staged, folded rows: [plane][column][per]
+//   pi - phi at most: E of even m, E of odd m, O of even m, O of odd m
+//   quarter fold: E of m mod 4 = 0, 2, O of m mod 4 = 0, 2, then of odd m: E_A - E_D,
+//   E_B - E_C, O_A + O_D, O_B + O_C
+constexpr int kPlanes = 4, kPlanesQuarter = 8;
+
 __global__ void k_sep_phi64(const SepPhi64 a) {
   pdl_begin();
   extern __shared__ __align__(16) unsigned char smraw[];
-  double *xs = reinterpret_cast<double *>(smraw);   // [E even m, E odd m, O even m, O odd m][column][per]
+  double *xs = reinterpret_cast<double *>(smraw);
   const int row0 = blockIdx.x * a.per, cols = a.fold.cols, plane = cols * a.per;
-  const int patch_rows = a.n_r * a.n_theta;
+  const int patch_rows = a.n_r * a.n_theta, h = a.fold.half;
+  const bool quarter = a.fold.quarter > 0;
   for (int e = threadIdx.x; e < plane; e += blockDim.x) {
     const int r = e / cols, c = e % cols, row = row0 + r;
-    double ee = 0.0, eo = 0.0, oe = 0.0, oo = 0.0;
-    if (row < a.rows) {
-      const double *x = (row >= patch_rows ? a.rho1 + (size_t)(row - patch_rows) * a.n_phi : a.rho0 + (size_t)row * a.n_phi);
-      const double *w = a.w + (size_t)(row % a.n_theta) * a.n_phi;
-      auto fold = [&](int kp, double &E, double &O) {
-        const int km = a.n_phi - 1 - kp;
-        const double u = x[kp] * w[kp];
-        if (km == kp) {
-          E = u;
-          O = 0.0;
-        } else {
-          const double v = x[km] * w[km];
-          E = u + v;
-          O = u - v;
-        }
-      };
-      fold(a.fold.first + c, ee, oe);
-      eo = ee;
-      oo = oe;
-      const int pc = a.fold.partner - c;
-      if (a.fold.partner >= 0 && pc > c && pc < a.fold.half) {
-        double E, O;
-        fold(a.fold.first + pc, E, O);
-        eo = ee - E;   // cos(m (pi - phi)) = (-1)^m cos(m phi)
-        ee = ee + E;
-        oo = oe + O;   // sin(m (pi - phi)) = -(-1)^m sin(m phi)
-        oe = oe - O;
-      }
-    }
     double *o = xs + c * a.per + r;
-    o[0] = ee;
-    o[plane] = eo;
-    o[2 * plane] = oe;
-    o[3 * plane] = oo;
+    const bool ok = row < a.rows;
+    const int rr = ok ? row : 0;
+    const double *x = (rr >= patch_rows ? a.rho1 + (size_t)(rr - patch_rows) * a.n_phi : a.rho0 + (size_t)rr * a.n_phi);
+    const double *w = a.w + (size_t)(rr % a.n_theta) * a.n_phi;
+    auto fold = [&](bool on, int col, double &E, double &O) {
+      E = O = 0.0;
+      if (!ok || !on) return;
+      const int kp = a.fold.first + col, km = a.n_phi - 1 - kp;
+      const double u = x[kp] * w[kp];
+      if (km == kp) {
+        E = u;
+      } else {
+        const double v = x[km] * w[km];
+        E = u + v;
+        O = u - v;
+      }
+    };
+    if (quarter) {
+      const int kb = a.fold.quarter - a.fold.odd - c, kc = a.fold.quarter + c, kd = a.fold.partner - c;
+      double ea, oa, eb, ob, ec, oc, ed, od;
+      fold(true, c, ea, oa);
+      fold(kb != c && kb < h, kb, eb, ob);
+      fold(kc != kb && kc < h, kc, ec, oc);
+      fold(kd != kc && kd != c && kd < h, kd, ed, od);
+      const double e1 = ea + ed, e2 = eb + ec, o1 = oa - od, o2 = ob - oc;
+      o[0] = e1 + e2;           // cos(m phi), m mod 4 = 0
+      o[plane] = e1 - e2;       // 2
+      o[2 * plane] = o1 - o2;   // sin(m phi), m mod 4 = 0
+      o[3 * plane] = o1 + o2;   // 2
+      o[4 * plane] = ea - ed;
+      o[5 * plane] = eb - ec;
+      o[6 * plane] = oa + od;
+      o[7 * plane] = ob + oc;
+    } else {
+      double ee, oe, E, O;
+      fold(true, c, ee, oe);
+      const int pc = a.fold.partner - c;
+      fold(a.fold.partner >= 0 && pc > c && pc < h, pc, E, O);
+      o[0] = ee + E;            // cos(m (pi - phi)) = (-1)^m cos(m phi)
+      o[plane] = ee - E;
+      o[2 * plane] = oe - O;    // sin(m (pi - phi)) = -(-1)^m sin(m phi)
+      o[3 * plane] = oe + O;
+    }
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < a.per / kR64 * a.m1; e += blockDim.x) {
-    const int r = e / a.m1 * kR64, m = e % a.m1;
-    const double *xe = xs + (m & 1 ? plane : 0) + r, *xo = xe + 2 * plane;
+  // items (pair of rows, order), the even orders first: with the quarter fold an
+  // odd order costs twice an even one, and a warp should not hold both
+  const int pairs = a.per / kR64, evens = (a.m1 + 1) / 2;
+  for (int e = threadIdx.x; e < pairs * a.m1; e += blockDim.x) {
+    const bool is_odd = e >= pairs * evens;
+    const int e1 = is_odd ? e - pairs * evens : e, n = is_odd ? a.m1 - evens : evens;
+    const int r = e1 / n * kR64, m = e1 % n * 2 + (is_odd ? 1 : 0);
     const double2 *az = a.az + m;
     double cs[kR64] = {0.0, 0.0}, sn[kR64] = {0.0, 0.0};
+    auto sum = [&](const double *xe, const double *xo) {
 #pragma unroll 4
-    for (int c = 0; c < cols; ++c) {
-      const double2 t = az[(size_t)c * a.m1];
-      const double2 u = *reinterpret_cast<const double2 *>(xe + c * a.per), v = *reinterpret_cast<const double2 *>(xo + c * a.per);
-      cs[0] = fma(u.x, t.x, cs[0]);
-      cs[1] = fma(u.y, t.x, cs[1]);
-      sn[0] = fma(v.x, t.y, sn[0]);
-      sn[1] = fma(v.y, t.y, sn[1]);
+      for (int c = 0; c < cols; ++c) {
+        const double2 t = az[(size_t)c * a.m1];
+        const double2 u = *reinterpret_cast<const double2 *>(xe + c * a.per), v = *reinterpret_cast<const double2 *>(xo + c * a.per);
+        cs[0] = fma(u.x, t.x, cs[0]);
+        cs[1] = fma(u.y, t.x, cs[1]);
+        sn[0] = fma(v.x, t.y, sn[0]);
+        sn[1] = fma(v.y, t.y, sn[1]);
+      }
+    };
+    if (!quarter) {
+      sum(xs + (is_odd ? plane : 0) + r, xs + (is_odd ? 3 : 2) * plane + r);
+    } else if (!is_odd) {
+      sum(xs + (m & 2 ? plane : 0) + r, xs + (m & 2 ? 3 : 2) * plane + r);
+    } else {
+      const double *ea = xs + 4 * plane + r, *eb = ea + plane, *oa = eb + plane, *ob = oa + plane;
+      double cq[kR64] = {0.0, 0.0}, sq[kR64] = {0.0, 0.0};   // B and C, with the other function
+#pragma unroll 2
+      for (int c = 0; c < cols; ++c) {
+        const double2 t = az[(size_t)c * a.m1];
+        const double2 u = *reinterpret_cast<const double2 *>(ea + c * a.per), v = *reinterpret_cast<const double2 *>(oa + c * a.per);
+        const double2 p = *reinterpret_cast<const double2 *>(eb + c * a.per), q = *reinterpret_cast<const double2 *>(ob + c * a.per);
+        cs[0] = fma(u.x, t.x, cs[0]);
+        cs[1] = fma(u.y, t.x, cs[1]);
+        sn[0] = fma(v.x, t.y, sn[0]);
+        sn[1] = fma(v.y, t.y, sn[1]);
+        cq[0] = fma(p.x, t.y, cq[0]);
+        cq[1] = fma(p.y, t.y, cq[1]);
+        sq[0] = fma(q.x, t.x, sq[0]);
+        sq[1] = fma(q.y, t.x, sq[1]);
+      }
+#pragma unroll
+      for (int i = 0; i < kR64; ++i) {   // sin(m pi / 2) = 1, -1 for m mod 4 = 1, 3
+        cs[i] += (m & 2) ? -cq[i] : cq[i];
+        sn[i] += (m & 2) ? -sq[i] : sq[i];
+      }
     }
 #pragma unroll
     for (int i = 0; i < kR64; ++i) {
@@ -540,7 +594,9 @@ __global__ void __launch_bounds__(256) k_sep_theta_partials(SepThetaPartials a, 
 // Rows per block of the float64 azimuthal stage: 16 (two blocks or more per SM
 // at the folded columns of one-degree cells), halved while the SMs are short of
 // blocks or the staged rows do not fit; 0: not even two rows fit.
-size_t phi64_smem(const AzFold &f, int rows) { return 4 * (size_t)f.cols * rows * sizeof(double); }
+size_t phi64_smem(const AzFold &f, int rows) {
+  return (size_t)(f.quarter > 0 ? kPlanesQuarter : kPlanes) * f.cols * rows * sizeof(double);
+}
 int phi64_rows(const yy_grid *g) {
   const AzFold f = az_fold(g);
   const long long rows = (long long)grid_rows(g) * g->n_theta;
