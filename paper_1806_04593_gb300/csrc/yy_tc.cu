@@ -95,7 +95,7 @@ __device__ __forceinline__ void split8(const float (&y)[8], typename F::elem *ba
 
 template <class F>
 __global__ void __launch_bounds__(256) k_pack_rows(PackBatch batch) {
-  pdl_begin();
+  pdl_wait();
   extern __shared__ float rowbuf[];
   __shared__ double red[4][256];
   const PackArgs &p = batch.job[blockIdx.y];
@@ -358,7 +358,7 @@ __device__ __forceinline__ void pack_store(const PackArgs &p, int row, const dou
 template <class F, int TPR, int P>
 __global__ void __launch_bounds__(TPR > 256 ? TPR : 256, (TPR <= 32 && P <= 6) ? 4 : ((TPR <= 32 && P <= 12) ? 3 : 1))
 k_pack_reg(PackBatch batch) {
-  pdl_begin();
+  pdl_wait();
   constexpr int TPB = TPR > 256 ? TPR : 256;
   __shared__ RowStats red[32];
   const PackArgs &p = batch.job[blockIdx.y];
@@ -417,7 +417,7 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
 
 template <class F>
 __global__ void __launch_bounds__(1024, 1) k_pack_stream(PackArgs p, int *err) {
-  pdl_begin();
+  pdl_wait();
   extern __shared__ __align__(16) double rowbuf_f64[];
   __shared__ RowStats red[32];
   __shared__ __align__(8) uint64_t bar;
@@ -2503,7 +2503,7 @@ inline size_t theta_ff_smem(int lmax, int gk) {
 // orders m at a time (m and l_max + 1 - m, about 2 (l_max + 1) terms).
 template <int NG>
 __global__ void __launch_bounds__(512, 2) k_theta_ff(OzThetaFFArgs a) {
-  pdl_begin();
+  pdl_wait();
   constexpr int TP = NG == 1 ? 2 : 1;
   constexpr int R = 2 * TP;
   extern __shared__ float4 ffsm4[];
@@ -2929,7 +2929,7 @@ struct OzRhoArgs {
 // digits of one slice go out as one 32-bit store of their bf16 patterns.
 template <int C>
 __global__ void __launch_bounds__(256) k_rhow_ozaki(OzRhoArgs a) {
-  pdl_begin();
+  pdl_wait();
   const int row = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (row >= a.rows) return;
   const int shell = row / a.n_theta, j = row % a.n_theta;
