@@ -2359,25 +2359,6 @@ __device__ __forceinline__ void ff_fma_x2(ulonglong2 q, ffx2 qn_hi, ulonglong2 p
   aH = s;
 }
 
-// The balanced base-256 digits of 0 <= X <= 2^47 in one step: with
-// Y = X + 127 (1 + 2^8 + ... + 2^32), the low five digits are Y's bytes less
-// 127 (each in [-127, 128], the carries done by the addition) and the top
-// one is Y >> 40.  Each digit comes out as the fp32 bit pattern of its
-// value, whose upper half is the bf16 pattern (an integer below 2^8 in
-// magnitude has sixteen zero low bits), most significant digit first: the
-// patterns of 2^23 + digit + 127 (the top one's of 2^23 + digit), from which
-// one fp32 subtraction each leaves the digit.
-__device__ __forceinline__ void x_digit_bits(unsigned long long X, uint32_t (&bits)[6]) {
-  const unsigned long long Y = X + 0x7F7F7F7F7Full;
-  const uint32_t ylo = (uint32_t)Y, yhi = (uint32_t)(Y >> 32);
-  bits[0] = __float_as_uint(__fsub_rn(__uint_as_float(0x4B000000u | (yhi >> 8)), 8388608.f));
-  bits[1] = __float_as_uint(__fsub_rn(__uint_as_float(__byte_perm(yhi, 0x4B000000u, 0x7540)), 8388735.f));
-  bits[2] = __float_as_uint(__fsub_rn(__uint_as_float(__byte_perm(ylo, 0x4B000000u, 0x7543)), 8388735.f));
-  bits[3] = __float_as_uint(__fsub_rn(__uint_as_float(__byte_perm(ylo, 0x4B000000u, 0x7542)), 8388735.f));
-  bits[4] = __float_as_uint(__fsub_rn(__uint_as_float(__byte_perm(ylo, 0x4B000000u, 0x7541)), 8388735.f));
-  bits[5] = __float_as_uint(__fsub_rn(__uint_as_float(__byte_perm(ylo, 0x4B000000u, 0x7540)), 8388735.f));
-}
-
 __device__ __forceinline__ ffx2 x2_pack(uint32_t lo, uint32_t hi) { return ((ffx2)hi << 32) | lo; }
 
 // Base-1024 digits (FormOzSynth) of two float-float values (hi, lo) at once, both
@@ -2911,23 +2892,40 @@ __global__ void __launch_bounds__(256) k_rotate_ff(int n_r, int n_lm, int lmax, 
   }
 }
 
-// The weighted densities of the separable analysis, rho w, as digit rows for
-// the analysis: one warp per row (shell, j); lane L takes the pairs
-// k = 2 L + 64 c.  rho w is the float64 product of the CUDA-core path; the
-// row's scale 2^e from its largest |rho w| (every value below 2^(e - 1)),
-// the digits of X = round(|rho w| 2^(48 - e)) taken from the float64 bits,
-// and the row exponent of a unit level-6 sum includes the table's scale 2^eb.
+// The weighted densities of the separable analysis, rho w, as digit rows for the
+// analysis: one warp per row (shell, j).  X = round(rho w 2^(48 - e)), |X| <= 2^47,
+// comes from one float64 multiply-add per cell, onto a constant whose last bit is
+// worth 2^(e - 48): its bits less the constant's are X.  The row's scale 2^e (every
+// |rho w| below 2^(e - 1)) is bounded from the operands' upper words: for a positive
+// float64, exponent + mantissa is its logarithm less at most 0.0861, so the
+// largest sum of the two words, plus 0.1723, bounds the largest product.  Rows
+// beyond 2^+-900 (or without a finite scale) take X from the bits of the products.
+// The digits of X (or of the sums below) are the bytes of X + 127 (1 + 2^8 + ... +
+// 2^32) + 2^50, signs included: five in [-127, 128] and the top one.
+//
+// kFold (k_oz_analysis): the digits are those of the sums and the differences of cell k
+// and its mirror n_phi - 1 - k (a middle cell enters the sums once, its differences
+// meet zeros of the table), for k < n_phi / 2 rounded up, first the sums: lanes 0-15 take the
+// cells k = 2 L + 32 c and then the sums, lanes 16-31 the mirrors and the differences
+// (mirror less cell), formed from the X, exactly, after one exchange.  |sum| <= 2^48
+// makes a top digit of at most 256 (exact in bf16).
+//
+// The integer pipe was the bound (86 percent busy with X taken from the bits of every
+// product and sign and magnitude kept apart; float64 additions for the folds, at two
+// operations per clock per SM, took 190 us); now memory is, 92 us at 6.0 TB/s on the
+// 1-degree grid at 550 zones (101 unfolded, of 320 columns) and 67 at 300 zones of a
+// 1-degree polar grid (91).
 struct OzRhoArgs {
   int n_r, n_theta, n_phi, rows, k_pad, rows_pad, eb;
   const double *rho0, *rho1;    // [n_r][n_theta][n_phi] per patch (rho1 NULL on a polar grid)
-  const double *w;              // [n_theta][n_phi]
+  const double *w;              // [n_theta][n_phi], nonnegative
   __nv_bfloat16 *X;             // [6][rows_pad][k_pad]
   int *rexp;                    // [rows_pad]
 };
 
-// C: 64-wide pieces of a row held per lane (k_pad <= 64 C).  Two cells'
-// digits of one slice go out as one 32-bit store of their bf16 patterns.
-template <int C>
+// C: pieces of a row, 64 of k_pad values or 32 of k_pad / 2 sums and differences.  Two values' digits of
+// one slice go out as one 32-bit store of their bf16 patterns.
+template <int C, bool kFold>
 __global__ void __launch_bounds__(256) k_rhow_ozaki(OzRhoArgs a) {
   pdl_wait();
   const int row = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
@@ -2936,59 +2934,110 @@ __global__ void __launch_bounds__(256) k_rhow_ozaki(OzRhoArgs a) {
   const int p = shell / a.n_r, i = shell % a.n_r;
   const double *rho = (p == 0 ? a.rho0 : a.rho1) + ((size_t)i * a.n_theta + j) * a.n_phi;
   const double *wj = a.w + (size_t)j * a.n_phi;
-  unsigned long long bits[C][2];
-  unsigned long long mb = 0ull;
+  const int cells = kFold ? (a.n_phi + 1) / 2 : a.n_phi;
+  const bool mirror = kFold && lane >= 16;
+  // a lane's two cells at, at + 1: columns k, k + 1, or k + 1, k of a mirror
+  double x[C][2], w[C][2];
+  unsigned int top = 0u, largest = 0u;
   // an even n_phi keeps every row on a 16-byte boundary (the densities are
-  // 16-byte aligned): a lane's two cells k, k + 1 in one load of each array
+  // 16-byte aligned): both cells in one load of each array
   const bool pairs = (a.n_phi & 1) == 0;
 #pragma unroll
   for (int c = 0; c < C; ++c) {
-    const int k = 2 * lane + 64 * c;
-    double v[2] = {0.0, 0.0};
-    if (pairs) {
-      if (k < a.n_phi) {
-        const double2 r2 = *reinterpret_cast<const double2 *>(rho + k);
-        const double2 w2 = *reinterpret_cast<const double2 *>(wj + k);
-        v[0] = r2.x * w2.x;
-        v[1] = r2.y * w2.y;
-      }
-    } else {
+    const int k = kFold ? 2 * (lane & 15) + 32 * c : 2 * lane + 64 * c;
+    const int at = mirror ? a.n_phi - 2 - k : k;
+    x[c][0] = x[c][1] = w[c][0] = w[c][1] = 0.0;
+    if (pairs && k + 1 < cells) {
+      const double2 r2 = *reinterpret_cast<const double2 *>(rho + at);
+      const double2 w2 = *reinterpret_cast<const double2 *>(wj + at);
+      x[c][0] = r2.x;
+      x[c][1] = r2.y;
+      w[c][0] = w2.x;
+      w[c][1] = w2.y;
+    } else if (k < cells) {
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
-        if (k + h < a.n_phi) v[h] = rho[k + h] * wj[k + h];
+      for (int h = 0; h < 2; ++h) {
+        const int col = mirror ? k + 1 - h : k + h;
+        if (col < cells && !(mirror && at + h == col)) {   // a middle cell: once
+          x[c][h] = rho[at + h];
+          w[c][h] = wj[at + h];
+        }
+      }
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      bits[c][h] = (unsigned long long)__double_as_longlong(v[h]);
-      mb = max(mb, bits[c][h] & 0x7FFFFFFFFFFFFFFFull);
+      const unsigned int u = (unsigned int)__double2hiint(x[c][h]) & 0x7FFFFFFFu;
+      top = max(top, u + (unsigned int)__double2hiint(w[c][h]));
+      largest = max(largest, u);   // infinities and NaN, also under a zero weight
     }
   }
+  top = __reduce_max_sync(0xffffffffu, top);
+  largest = __reduce_max_sync(0xffffffffu, largest);
+  int e = (int)((top + 180700u) >> 20) - 2044;   // 180700 > 0.1723 2^20; |rho w| < 2^(e - 1)
+  long long base = 0, X[C][2];
+  bool zero = false;
+  if (e >= -900 && e <= 900 && largest < 0x7FF00000u) {
+    const double magic = __hiloint2double((e + 4 + 1023) << 20 | 0x80000, 0);   // 1.5 2^(e + 4)
+    base = __double_as_longlong(magic);
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, off));
-  const int exm = (int)(mb >> 52);
-  const int e = exm - 1021;
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) X[c][h] = __double_as_longlong(fma(x[c][h], w[c][h], magic));
+  } else {
+    unsigned long long mb = 0ull;
+#pragma unroll
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        X[c][h] = __double_as_longlong(x[c][h] * w[c][h]);
+        mb = max(mb, (unsigned long long)X[c][h] & 0x7FFFFFFFFFFFFFFFull);
+      }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, off));
+    const int exm = (int)(mb >> 52);
+    zero = exm == 0;
+    e = exm - 1021;
+#pragma unroll
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const unsigned long long u = (unsigned long long)X[c][h];
+        const int ex = (int)((u >> 52) & 0x7FFu), sh = 1027 - ex + e;
+        long long v = 0;
+        if (exm != 0 && ex != 0 && sh < 64) v = (long long)(((((u & 0xFFFFFFFFFFFFFull) | (1ull << 52)) >> (sh - 1)) + 1ull) >> 1);
+        X[c][h] = X[c][h] < 0 ? -v : v;
+      }
+  }
+  // sums: own + other less both constants; differences: own - other = own + ~other + 1
+  const long long digits = 0x7F7F7F7F7Fll + (1ll << 50);
+  const long long bias = !kFold ? digits - base : mirror ? digits + 1 : digits - 2 * base;
+  const long long flip = mirror ? -1ll : 0ll;
+  const unsigned int order = mirror ? 0x3276u : 0x7632u;
   const size_t stride = (size_t)a.rows_pad * a.k_pad;
+  const int width = kFold ? a.k_pad / 2 : a.k_pad, k0 = kFold ? 2 * (lane & 15) : 2 * lane;
+  uint32_t *dst = reinterpret_cast<uint32_t *>(a.X + (size_t)row * a.k_pad + (mirror ? width : 0) + k0);
 #pragma unroll
   for (int c = 0; c < C; ++c) {
-    const int k0 = 2 * lane + 64 * c;
-    if (k0 >= a.k_pad) break;
+    if ((kFold ? 32 : 64) * c >= width) break;
     uint32_t d[2][6];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int ex = (int)((bits[c][h] >> 52) & 0x7FFu);
-      const int sh = 1027 - ex + e;
-      unsigned long long X = 0;
-      if (exm != 0 && ex != 0 && sh < 64)
-        X = ((((bits[c][h] & 0xFFFFFFFFFFFFFull) | (1ull << 52)) >> (sh - 1)) + 1ull) >> 1;
-      x_digit_bits(X, d[h]);
+      long long Y = X[c][h] + bias;
+      if constexpr (kFold) Y += __shfl_xor_sync(0xffffffffu, X[c][1 - h], 16) ^ flip;
+      const uint32_t ylo = (uint32_t)Y, yhi = (uint32_t)((unsigned long long)Y >> 32);
+      // the fp32 patterns of 2^23 + digit + 127 (top: + 1024), less the offset
+      d[h][0] = __float_as_uint(__fsub_rn(__uint_as_float(0x4B000000u | (yhi >> 8)), 8388608.f + 1024.f));
+      d[h][1] = __float_as_uint(__fsub_rn(__uint_as_float(__byte_perm(yhi, 0x4B000000u, 0x7540)), 8388735.f));
+      d[h][2] = __float_as_uint(__fsub_rn(__uint_as_float(__byte_perm(ylo, 0x4B000000u, 0x7543)), 8388735.f));
+      d[h][3] = __float_as_uint(__fsub_rn(__uint_as_float(__byte_perm(ylo, 0x4B000000u, 0x7542)), 8388735.f));
+      d[h][4] = __float_as_uint(__fsub_rn(__uint_as_float(__byte_perm(ylo, 0x4B000000u, 0x7541)), 8388735.f));
+      d[h][5] = __float_as_uint(__fsub_rn(__uint_as_float(__byte_perm(ylo, 0x4B000000u, 0x7540)), 8388735.f));
     }
-    // the signs on the bf16 patterns
-    const uint32_t sm = ((uint32_t)(bits[c][0] >> 63) << 15) | ((uint32_t)(bits[c][1] >> 63) << 31);
-    uint32_t *dst = reinterpret_cast<uint32_t *>(a.X + (size_t)row * a.k_pad + k0);
+    if (kFold && k0 + 32 * c >= width) continue;
 #pragma unroll
-    for (int sl = 0; sl < 6; ++sl) dst[sl * (stride / 2)] = __byte_perm(d[0][sl], d[1][sl], 0x7632) ^ sm;
+    for (int sl = 0; sl < 6; ++sl) dst[sl * (stride / 2) + (kFold ? 16 : 32) * c] = __byte_perm(d[0][sl], d[1][sl], order);
   }
-  if (lane == 0) a.rexp[row] = exm == 0 ? 0 : e + a.eb - 64;
+  if (lane == 0) a.rexp[row] = zero ? 0 : e + a.eb - 64;
 }
 
 }  // namespace yy
@@ -3015,10 +3064,10 @@ struct yy_oz_tables {
   int an_ok, an_kpad, an_bn, an_row_tiles, an_b_rows_pad, an_stages, an_slots, an_eb;
   void *an_x;                   // [6][rows_pad][an_kpad]
   int *an_exp;                  // [rows_pad]
-  void *an_az;                  // [6][an_b_rows_pad][an_kpad]
+  void *an_az;                  // [6][an_b_rows_pad][an_kpad, or folded: half of the cells, padded to 32]
   yy::PairMaps an_maps;
-  int an_slots2;                // resident clusters of k_oz_analysis (0: the pair kernel serves)
-  yy::OzAnalysisMaps an_maps2;  // its maps: density digits (box 128 rows), table digits (box 32 rows)
+  int an_slots2;                // resident clusters of k_oz_analysis, with folded rows (0: the pair kernel serves)
+  yy::OzAnalysisMaps an_maps2;  // its maps
 };
 
 namespace yy {
@@ -3068,15 +3117,27 @@ static yy_status ozaki_prepare_analysis(yy_grid *g, yy_oz_tables *o) {
   typedef FormOzaki F;
   const int nt = 2 * g->lmax + 1;
   if (g->n_phi > F::kFillK * F::kMaxFills || !g->sep_az || !g->sep_F) return YY_OK;
-  o->an_kpad = round_up(g->n_phi, kPadK);
+  // l_max <= 31: folded rows and k_oz_analysis; otherwise the pair kernel
+  o->an_slots2 = 0;
+  if (g->lmax < kOzAnBN &&
+      cudaFuncSetAttribute(k_oz_analysis, cudaFuncAttributeMaxDynamicSharedMemorySize, kOzAnSmem) == cudaSuccess) {
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = pair_config(64, kOzAnSmem, 0, attr);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, (void *)k_oz_analysis, &cfg) == cudaSuccess && n > 0) o->an_slots2 = n;
+  }
+  cudaGetLastError();
+  const bool fold = o->an_slots2 > 0;
+  const int half = (g->n_phi + 1) / 2, width = fold ? round_up(half, 32) : round_up(g->n_phi, kPadK);   // columns of the table
+  o->an_kpad = fold ? 2 * round_up(half, 16) : width;
   o->an_bn = 32;   // seven level accumulators of bn columns within one 256-column TMEM buffer
   o->an_row_tiles = (nt + o->an_bn - 1) / o->an_bn;
-  o->an_b_rows_pad = round_up(nt, kOzAnBN);   // tiles of an_bn (pair kernel) and kOzAnBN (k_oz_analysis)
+  o->an_b_rows_pad = fold ? 2 * kOzAnBN : round_up(nt, o->an_bn);
   o->an_stages = pair_stages<F>(o->an_bn, kEpiStageBytes);
-  if (o->an_stages < 2 ||
-      cudaFuncSetAttribute(k_tc_pair<F, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess)
-    return YY_OK;
-  {
+  if (!fold) {
+    if (o->an_stages < 2 ||
+        cudaFuncSetAttribute(k_tc_pair<F, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess)
+      return YY_OK;
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg =
         pair_config(64, o->an_stages * pair_stage_bytes<F>(o->an_bn) + kSmemFixed + kEpiStageBytes, 0, attr);
@@ -3092,13 +3153,14 @@ static yy_status ozaki_prepare_analysis(yy_grid *g, yy_oz_tables *o) {
     if (e == cudaSuccess) e = dmalloc(ptr, bytes);
   };
   const size_t x_bytes = (size_t)F::kPA * o->rows_pad * o->an_kpad * F::kElem;
-  const size_t b_elems = (size_t)F::kPB * o->an_b_rows_pad * o->an_kpad;
+  const size_t b_elems = (size_t)F::kPB * o->an_b_rows_pad * width;
   A(&o->an_x, x_bytes);
   A((void **)&o->an_exp, o->rows_pad * sizeof(int));
   A(&o->an_az, b_elems * F::kElem);
   if (e == cudaSuccess) e = cudaMemset(o->an_x, 0, x_bytes);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? YY_ERR_OOM : YY_ERR_CUDA;
-  // the azimuthal table az[k][t] (rows of sep_nt_pad) as operand B, rows t:
+  // the azimuthal table az[k][t] (rows of sep_nt_pad) as operand B, rows t, or the
+  // cos slots by order and then, 32 rows on, the sin slots of the folded cells:
   // one scale 2^eb for all of it (every row's largest value is about d_phi)
   const int ntp = g->sep_nt_pad;
   std::vector<double> az((size_t)g->n_phi * ntp);
@@ -3111,30 +3173,23 @@ static yy_status ozaki_prepare_analysis(yy_grid *g, yy_oz_tables *o) {
   int E2 = 0;
   frexp(mx, &E2);   // mx < 2^E2
   o->an_eb = E2 + 1;
-  for (int k = 0; k < g->n_phi && mx > 0.0; ++k)
+  for (int k = 0; k < (fold ? half : g->n_phi) && mx > 0.0; ++k)
     for (int t = 0; t < nt; ++t) {
-      const double y = ldexp(az[(size_t)k * ntp + t], -o->an_eb);   // |y| < 1/2
+      const bool sine = t > 0 && t % 2 == 0;
+      double y = ldexp(az[(size_t)k * ntp + t], -o->an_eb);   // |y| < 1/2
+      if (fold && sine) y = 2 * k + 1 == g->n_phi ? 0.0 : -y;   // the differences are mirror less cell
+      const int row = !fold ? t : (sine ? kOzAnBN : 0) + (t + 1) / 2;
       int d[6];
       oz_digits((unsigned long long)floor(ldexp(fabs(y), 48) + 0.5), d);
       for (int s2 = 0; s2 < F::kPB; ++s2)
-        sl[((size_t)s2 * o->an_b_rows_pad + t) * o->an_kpad + k] = bf16_int(y < 0 ? -d[s2] : d[s2]);
+        sl[((size_t)s2 * o->an_b_rows_pad + row) * width + k] = bf16_int(y < 0 ? -d[s2] : d[s2]);
     }
   if (cudaMemcpy(o->an_az, sl.data(), b_elems * F::kElem, cudaMemcpyHostToDevice) != cudaSuccess) return YY_ERR_CUDA;
-  if (!make_map<F>(&o->an_maps.a[0], o->an_x, o->an_kpad, F::kPA * o->rows_pad, kPairRows) ||
-      !make_map<F>(&o->an_maps.b[0], o->an_az, o->an_kpad, F::kPB * o->an_b_rows_pad, o->an_bn / 2))
+  CUtensorMap *ma = fold ? &o->an_maps2.a : &o->an_maps.a[0], *mb = fold ? &o->an_maps2.b : &o->an_maps.b[0];
+  if (!make_map<F>(ma, o->an_x, o->an_kpad, F::kPA * o->rows_pad, kPairRows) ||
+      !make_map<F>(mb, o->an_az, width, F::kPB * o->an_b_rows_pad, fold ? kOzAnBN : o->an_bn / 2))
     return YY_ERR_NOT_SUPPORTED;
   o->an_ok = 1;
-  // the analysis kernel with all slots in one MMA
-  o->an_slots2 = 0;
-  if (nt <= kOzAnBN && make_map<F>(&o->an_maps2.a, o->an_x, o->an_kpad, F::kPA * o->rows_pad, kPairRows) &&
-      make_map<F>(&o->an_maps2.b, o->an_az, o->an_kpad, F::kPB * o->an_b_rows_pad, kOzAnBN) &&
-      cudaFuncSetAttribute(k_oz_analysis, cudaFuncAttributeMaxDynamicSharedMemorySize, kOzAnSmem) == cudaSuccess) {
-    cudaLaunchAttribute attr[2];
-    cudaLaunchConfig_t cfg = pair_config(64, kOzAnSmem, 0, attr);
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, (void *)k_oz_analysis, &cfg) == cudaSuccess && n > 0) o->an_slots2 = n;
-  }
-  cudaGetLastError();
   return YY_OK;
 }
 
@@ -3167,15 +3222,22 @@ cudaError_t ozaki_analysis(yy_grid *g, const double *ry, const double *rg, cudaS
   ra.rexp = o->an_exp;
   const unsigned blocks = (unsigned)(((size_t)o->rows * 32 + 255) / 256);
   constexpr int kCmax = FormOzaki::kFillK * FormOzaki::kMaxFills / 64;
-  cudaError_t e = launch_kernel(g, "k_rhow_ozaki", o->an_kpad <= 64 * 5 ? k_rhow_ozaki<5> : k_rhow_ozaki<kCmax>, blocks, 256, 0, s, ra);
+  auto rhow = o->an_slots2 > 0 ? (o->an_kpad <= 64 * 5   ? k_rhow_ozaki<5, true>
+                                  : o->an_kpad <= 64 * 6 ? k_rhow_ozaki<6, true>
+                                                         : k_rhow_ozaki<kCmax, true>)
+                               : (o->an_kpad <= 64 * 5 ? k_rhow_ozaki<5, false> : k_rhow_ozaki<kCmax, false>);
+  cudaError_t e = launch_kernel(g, "k_rhow_ozaki", rhow, blocks, 256, 0, s, ra);
   if (e != cudaSuccess) return e;
   if (o->an_slots2 > 0) {
     OzAnalysisArgs z = {};
     z.cells = o->rows;
     z.cell_tiles = o->rows_pad / (2 * kPairRows);
     z.cols = 2 * g->lmax + 1;
-    z.kb_total = o->an_kpad * F::kElem / kRowBytes;
-    z.kb_fill = F::kFillK * F::kElem / kRowBytes;   // exact level sums per fill; the epilogue adds the fills
+    z.width = o->an_kpad / 2;
+    z.kb_class = (z.width + 31) / 32;
+    // exact level sums per fill (the epilogue adds the fills): a folded top digit is up
+    // to 256, so a level sum over K columns is at most 7 K 2^14, below 2^24 for K <= 146
+    z.kb_fill = (g->n_phi + 1) / 2 <= 146 ? 5 : 4;
     z.a_rows = o->rows_pad;
     z.b_rows = o->an_b_rows_pad;
     z.ldo = g->sep_nt_pad;
