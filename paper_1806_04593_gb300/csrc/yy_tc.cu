@@ -376,16 +376,20 @@ k_pack_reg(PackBatch batch) {
 }
 
 // Streaming form for long rows of densities: a persistent block of 1024
-// threads per SM walks the rows blockIdx.x, blockIdx.x + gridDim.x, ...  One
-// thread starts the bulk copy of the block's next float64 row into shared
-// memory as soon as every thread holds the current one in registers, so that
-// row's reads stay in flight while the block reduces and stores the current
-// one.  Only the density job takes this form (no columns or rows left out, no
+// threads per SM walks the rows blockIdx.x, blockIdx.x + gridDim.x, ...  A row is
+// copied to shared memory in three pieces with a barrier each, and one thread starts
+// the copy of the next row's piece as soon as every thread holds the current one's in
+// registers: the next row is in flight while the rest of this one is read, reduced
+// and stored.  1100 rows of 24300 cells: 74 us in FormFP16x2, 79 in FormBF16x3 (87 and
+// 91 with the next row started after the whole one); each SM takes seven or eight rows.
+// Only the density job takes this form (no columns or rows left out, no
 // weight rows, an even row length, 16-byte aligned rows; the launcher checks),
 // so its predicates are per pair of elements; the arithmetic and its order are
 // those of k_pack_reg<F, 1024, kStreamP>.
 constexpr int kStreamP = 12;
 constexpr int kStreamMaxK = 2 * kStreamP * 1024;
+constexpr int kStreamRun = 4;        // pairs of a thread in one piece
+constexpr int kStreamPieces = kStreamP / kStreamRun, kStreamPiece = 2 * kStreamRun * 1024;   // doubles
 constexpr int kStreamChunk = 4096;   // doubles per bulk copy
 
 // float64 -> fp32, round to nearest even, for values in fp32's normal range:
@@ -415,104 +419,127 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
       : "memory");
 }
 
+// The row buffer's barriers: phase bits, and the pieces in flight (thread 0's copy).
+struct StreamState {
+  uint64_t *bar;
+  uint32_t phases, flying;
+};
+
+// start the copy of piece i of row r (one thread)
+__device__ __forceinline__ void stream_issue(const PackArgs &p, int r, int i, double *rowbuf, StreamState &st) {
+  const double *src = (r < p.split_row) ? p.src0 + (size_t)r * p.ld : p.src1 + (size_t)(r - p.split_row) * p.ld;
+  const int k0 = i * kStreamPiece, k1 = min(p.K, k0 + kStreamPiece);
+  if (k0 >= k1) return;
+  mbar_expect_tx(&st.bar[i], (uint32_t)(k1 - k0) * 8u);
+  for (int k = k0; k < k1; k += kStreamChunk)
+    bulk_load(smem_u32(rowbuf + k), src + k, (uint32_t)min(kStreamChunk, k1 - k) * 8u, &st.bar[i]);
+  st.flying |= 1u << i;
+}
+
+// One row: next(i) starts the copy of piece i of the block's next row (one thread).
+// False when a copy did not arrive in time.
+template <class F, class Next>
+__device__ __forceinline__ bool stream_row(const PackArgs &p, int row, double *rowbuf, StreamState &state, RowStats *red, int *err,
+                                           Next next) {
+  typedef typename F::elem E;
+  const int tid = threadIdx.x;
+  const int K = p.K;
+  const size_t piece_stride = (size_t)p.rows_pad * p.k_pad;
+  const bool valid = row < p.rows;
+  // the row in fp32 registers and its statistics (runs of 4 pairs for the dot product)
+  float x[2 * kStreamP];
+  RowStats st = {0.f, 0.f, 0.f, INFINITY, -INFINITY};
+#pragma unroll
+  for (int i = 0; i < kStreamPieces; ++i) {
+    const int c0 = i * kStreamRun;
+    float2 d[kStreamRun];
+#pragma unroll
+    for (int c = 0; c < kStreamRun; ++c) {
+      const int k = 2 * ((c0 + c) * 1024 + tid);
+      d[c] = valid && k < K && p.dot_vec ? *(const float2 *)(p.dot_vec + k) : make_float2(0.0f, 0.0f);
+    }
+    if (valid && i * kStreamPiece < K) {
+      const bool ok = mbar_wait(&state.bar[i], (state.phases >> i) & 1u, err);
+      if (__syncthreads_or(!ok)) {   // timed out: let the copies finish (bounded), then leave
+        for (int q = 0; q < kStreamPieces && tid == 0; ++q)
+          if (state.flying >> q & 1u) mbar_wait(&state.bar[q], (state.phases >> q) & 1u, err);
+        return false;
+      }
+      state.phases ^= 1u << i;
+      state.flying &= ~(1u << i);
+    }
+    float run = 0.0f;
+#pragma unroll
+    for (int c = c0; c < c0 + kStreamRun; ++c) {
+      const int k = 2 * (c * 1024 + tid);
+      float v0 = 0.0f, v1 = 0.0f;
+      if (valid && k < K) {
+        const double2 t = *(const double2 *)(rowbuf + k);
+        v0 = f64_to_f32_rn(t.x);
+        v1 = f64_to_f32_rn(t.y);
+        st.mn = fminf(st.mn, fminf(v0, v1));
+        st.mx = fmaxf(st.mx, fmaxf(v0, v1));
+      }
+      x[2 * c] = v0;
+      x[2 * c + 1] = v1;
+      st.s += v0;
+      st.s += v1;
+      run = fmaf(v0, d[c - c0].x, run);
+      run = fmaf(v1, d[c - c0].y, run);
+    }
+    if (p.dot_vec) two_sum_add(st.dh, st.dl, run, 0.0f);
+    __syncthreads();   // every thread holds the piece: its part of the buffer is free
+    if (tid == 0) next(i);
+  }
+  row_stats<1024>(st, red);
+  float mean = 0.0f;
+  if (p.mean_out && valid) mean = st.s / (float)K;
+  float amax = 0.0f;
+  if (valid) amax = fmaxf(st.mx - mean, mean - st.mn);
+  float scf = 1.0f;
+  if (amax > 0.0f && isfinite(amax)) scf = ldexpf(1.0f, 14 - ilogbf(amax));
+  if (tid == 0) {
+    p.scale_out[row] = (double)(1.0f / scf);   // a power of two: exact in fp32
+    if (p.scale_out_f) p.scale_out_f[row] = 1.0f / scf;
+    if (p.mean_out) p.mean_out[row] = (double)mean;
+    if (p.dot_vec && valid) p.dot_out[row] = (double)st.dh + (double)st.dl;
+  }
+  // (x - mean) scf as one rounding: scf is a power of two
+  const float off = -mean * scf;
+  E *orow = (E *)p.out + (size_t)row * p.k_pad;
+#pragma unroll
+  for (int c = 0; c < kStreamP; ++c) {
+    const int k = 2 * (c * 1024 + tid);
+    if (k >= p.k_pad) break;
+    const bool u = valid && k < K;
+    split2<F>(u ? fmaf(x[2 * c], scf, off) : 0.0f, u ? fmaf(x[2 * c + 1], scf, off) : 0.0f, orow + k,
+              piece_stride);
+  }
+  return true;
+}
+
+__device__ __forceinline__ StreamState stream_begin(uint64_t *bar) {
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kStreamPieces; ++i) mbar_init(&bar[i], 1);
+    fence_barrier_init();
+  }
+  __syncthreads();
+  return {bar, 0u, 0u};
+}
+
 template <class F>
 __global__ void __launch_bounds__(1024, 1) k_pack_stream(PackArgs p, int *err) {
   pdl_wait();
   extern __shared__ __align__(16) double rowbuf_f64[];
   __shared__ RowStats red[32];
-  __shared__ __align__(8) uint64_t bar;
-  typedef typename F::elem E;
-  const int tid = threadIdx.x;
-  const int K = p.K;
-  const size_t piece_stride = (size_t)p.rows_pad * p.k_pad;
-  auto row_src = [&](int r) {
-    return (r < p.split_row) ? p.src0 + (size_t)r * p.ld : p.src1 + (size_t)(r - p.split_row) * p.ld;
+  __shared__ __align__(8) uint64_t bar[kStreamPieces];
+  StreamState state = stream_begin(bar);
+  auto issue = [&](int r, int i) {
+    if (r < p.rows) stream_issue(p, r, i, rowbuf_f64, state);
   };
-  auto issue = [&](int r) {   // one thread
-    const double *src = row_src(r);
-    mbar_expect_tx(&bar, (uint32_t)K * 8u);
-    for (int k0 = 0; k0 < K; k0 += kStreamChunk) {
-      const int n = min(kStreamChunk, K - k0);
-      bulk_load(smem_u32(rowbuf_f64 + k0), src + k0, (uint32_t)n * 8u, &bar);
-    }
-  };
-  if (tid == 0) {
-    mbar_init(&bar, 1);
-    fence_barrier_init();
-  }
-  __syncthreads();
-  int row = blockIdx.x;
-  if (tid == 0 && row < p.rows) issue(row);
-  uint32_t phase = 0;
-  for (; row < p.rows_pad; row += gridDim.x) {
-    const bool valid = row < p.rows;
-    if (valid) {
-      const bool ok = mbar_wait(&bar, phase, err);
-      phase ^= 1u;
-      if (__syncthreads_or(!ok)) {   // timed out: let the copy finish (bounded), then leave
-        if (tid == 0) mbar_wait(&bar, phase ^ 1u, err);
-        return;
-      }
-    }
-    // the row in fp32 registers and its statistics (runs of 4 pairs for the dot product)
-    float x[2 * kStreamP];
-    RowStats st = {0.f, 0.f, 0.f, INFINITY, -INFINITY};
-#pragma unroll
-    for (int c0 = 0; c0 < kStreamP; c0 += 4) {
-      float run = 0.0f;
-#pragma unroll
-      for (int c = c0; c < c0 + 4; ++c) {
-        const int k = 2 * (c * 1024 + tid);
-        float v0 = 0.0f, v1 = 0.0f, d0 = 0.0f, d1 = 0.0f;
-        if (valid && k < K) {
-          const double2 t = *(const double2 *)(rowbuf_f64 + k);
-          v0 = f64_to_f32_rn(t.x);
-          v1 = f64_to_f32_rn(t.y);
-          st.mn = fminf(st.mn, fminf(v0, v1));
-          st.mx = fmaxf(st.mx, fmaxf(v0, v1));
-          if (p.dot_vec) {
-            const float2 d = *(const float2 *)(p.dot_vec + k);
-            d0 = d.x;
-            d1 = d.y;
-          }
-        }
-        x[2 * c] = v0;
-        x[2 * c + 1] = v1;
-        st.s += v0;
-        st.s += v1;
-        run = fmaf(v0, d0, run);
-        run = fmaf(v1, d1, run);
-      }
-      if (p.dot_vec) two_sum_add(st.dh, st.dl, run, 0.0f);
-    }
-    __syncthreads();   // every thread holds the row: the buffer is free
-    const int next = row + gridDim.x;
-    if (tid == 0 && next < p.rows) issue(next);
-    row_stats<1024>(st, red);
-    float mean = 0.0f;
-    if (p.mean_out && valid) mean = st.s / (float)K;
-    float amax = 0.0f;
-    if (valid) amax = fmaxf(st.mx - mean, mean - st.mn);
-    float scf = 1.0f;
-    if (amax > 0.0f && isfinite(amax)) scf = ldexpf(1.0f, 14 - ilogbf(amax));
-    if (tid == 0) {
-      p.scale_out[row] = (double)(1.0f / scf);   // a power of two: exact in fp32
-      if (p.scale_out_f) p.scale_out_f[row] = 1.0f / scf;
-      if (p.mean_out) p.mean_out[row] = (double)mean;
-      if (p.dot_vec && valid) p.dot_out[row] = (double)st.dh + (double)st.dl;
-    }
-    // (x - mean) scf as one rounding: scf is a power of two
-    const float off = -mean * scf;
-    E *orow = (E *)p.out + (size_t)row * p.k_pad;
-#pragma unroll
-    for (int c = 0; c < kStreamP; ++c) {
-      const int k = 2 * (c * 1024 + tid);
-      if (k >= p.k_pad) break;
-      const bool u = valid && k < K;
-      split2<F>(u ? fmaf(x[2 * c], scf, off) : 0.0f, u ? fmaf(x[2 * c + 1], scf, off) : 0.0f, orow + k,
-                piece_stride);
-    }
-  }
+  for (int i = 0; i < kStreamPieces && threadIdx.x == 0; ++i) issue((int)blockIdx.x, i);
+  for (int row = blockIdx.x; row < p.rows_pad; row += gridDim.x)
+    if (!stream_row<F>(p, row, rowbuf_f64, state, red, err, [&](int i) { issue(row + (int)gridDim.x, i); })) return;
 }
 
 // The streaming form over the long, even rows of many jobs: the grid walks
@@ -524,111 +551,21 @@ __global__ void __launch_bounds__(1024, 1)
 k_pack_stream_group(const PackArgs *__restrict__ jobs, const uint32_t *__restrict__ row_map, int n_rows, int *err) {
   extern __shared__ __align__(16) double rowbuf_f64[];
   __shared__ RowStats red[32];
-  __shared__ __align__(8) uint64_t bar;
-  typedef typename F::elem E;
-  const int tid = threadIdx.x;
-  auto issue = [&](const PackArgs &q, int r) {   // one thread
-    const double *src = (r < q.split_row) ? q.src0 + (size_t)r * q.ld : q.src1 + (size_t)(r - q.split_row) * q.ld;
-    mbar_expect_tx(&bar, (uint32_t)q.K * 8u);
-    for (int k0 = 0; k0 < q.K; k0 += kStreamChunk) {
-      const int n = min(kStreamChunk, q.K - k0);
-      bulk_load(smem_u32(rowbuf_f64 + k0), src + k0, (uint32_t)n * 8u, &bar);
-    }
+  __shared__ __align__(8) uint64_t bar[kStreamPieces];
+  StreamState state = stream_begin(bar);
+  auto issue = [&](int gi, int i) {
+    if (gi >= n_rows) return;
+    const uint32_t m = row_map[gi];
+    const PackArgs &q = jobs[m >> 24];
+    const int r = (int)(m & 0xFFFFFFu);
+    if (r < q.rows) stream_issue(q, r, i, rowbuf_f64, state);
   };
-  // the job and row of global row i, and whether it carries data
-  auto at = [&](int i, int &job, int &r) {
-    const uint32_t m = row_map[i];
-    job = (int)(m >> 24);
-    r = (int)(m & 0xFFFFFFu);
-  };
-  if (tid == 0) {
-    mbar_init(&bar, 1);
-    fence_barrier_init();
-  }
-  __syncthreads();
-  if (tid == 0 && (int)blockIdx.x < n_rows) {
-    int j0, r0;
-    at((int)blockIdx.x, j0, r0);
-    if (r0 < jobs[j0].rows) issue(jobs[j0], r0);
-  }
-  uint32_t phase = 0;
+  for (int i = 0; i < kStreamPieces && threadIdx.x == 0; ++i) issue((int)blockIdx.x, i);
   for (int gi = blockIdx.x; gi < n_rows; gi += gridDim.x) {
-    int jb, row;
-    at(gi, jb, row);
-    const PackArgs &p = jobs[jb];
-    const int K = p.K;
-    const size_t piece_stride = (size_t)p.rows_pad * p.k_pad;
-    const bool valid = row < p.rows;
-    if (valid) {
-      const bool ok = mbar_wait(&bar, phase, err);
-      phase ^= 1u;
-      if (__syncthreads_or(!ok)) {   // timed out: let the copy finish (bounded), then leave
-        if (tid == 0) mbar_wait(&bar, phase ^ 1u, err);
-        return;
-      }
-    }
-    // the row in fp32 registers and its statistics (runs of 4 pairs for the dot product)
-    float x[2 * kStreamP];
-    RowStats st = {0.f, 0.f, 0.f, INFINITY, -INFINITY};
-#pragma unroll
-    for (int c0 = 0; c0 < kStreamP; c0 += 4) {
-      float run = 0.0f;
-#pragma unroll
-      for (int c = c0; c < c0 + 4; ++c) {
-        const int k = 2 * (c * 1024 + tid);
-        float v0 = 0.0f, v1 = 0.0f, d0 = 0.0f, d1 = 0.0f;
-        if (valid && k < K) {
-          const double2 t = *(const double2 *)(rowbuf_f64 + k);
-          v0 = f64_to_f32_rn(t.x);
-          v1 = f64_to_f32_rn(t.y);
-          st.mn = fminf(st.mn, fminf(v0, v1));
-          st.mx = fmaxf(st.mx, fmaxf(v0, v1));
-          if (p.dot_vec) {
-            const float2 d = *(const float2 *)(p.dot_vec + k);
-            d0 = d.x;
-            d1 = d.y;
-          }
-        }
-        x[2 * c] = v0;
-        x[2 * c + 1] = v1;
-        st.s += v0;
-        st.s += v1;
-        run = fmaf(v0, d0, run);
-        run = fmaf(v1, d1, run);
-      }
-      if (p.dot_vec) two_sum_add(st.dh, st.dl, run, 0.0f);
-    }
-    __syncthreads();   // every thread holds the row: the buffer is free
-    const int next = gi + gridDim.x;
-    if (tid == 0 && next < n_rows) {
-      int jn, rn;
-      at(next, jn, rn);
-      if (rn < jobs[jn].rows) issue(jobs[jn], rn);
-    }
-    row_stats<1024>(st, red);
-    float mean = 0.0f;
-    if (p.mean_out && valid) mean = st.s / (float)K;
-    float amax = 0.0f;
-    if (valid) amax = fmaxf(st.mx - mean, mean - st.mn);
-    float scf = 1.0f;
-    if (amax > 0.0f && isfinite(amax)) scf = ldexpf(1.0f, 14 - ilogbf(amax));
-    if (tid == 0) {
-      p.scale_out[row] = (double)(1.0f / scf);   // a power of two: exact in fp32
-      if (p.scale_out_f) p.scale_out_f[row] = 1.0f / scf;
-      if (p.mean_out) p.mean_out[row] = (double)mean;
-      if (p.dot_vec && valid) p.dot_out[row] = (double)st.dh + (double)st.dl;
-    }
-    // (x - mean) scf as one rounding: scf is a power of two
-    const float off = -mean * scf;
-    E *orow = (E *)p.out + (size_t)row * p.k_pad;
-#pragma unroll
-    for (int c = 0; c < kStreamP; ++c) {
-      const int k = 2 * (c * 1024 + tid);
-      if (k >= p.k_pad) break;
-      const bool u = valid && k < K;
-      split2<F>(u ? fmaf(x[2 * c], scf, off) : 0.0f, u ? fmaf(x[2 * c + 1], scf, off) : 0.0f, orow + k,
-                piece_stride);
-    }
+    const uint32_t m = row_map[gi];
+    if (!stream_row<F>(jobs[m >> 24], (int)(m & 0xFFFFFFu), rowbuf_f64, state, red, err,
+                       [&](int i) { issue(gi + (int)gridDim.x, i); }))
+      return;
   }
 }
 
