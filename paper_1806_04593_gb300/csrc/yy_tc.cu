@@ -2588,7 +2588,7 @@ __global__ void __launch_bounds__(512, 2) k_theta_ff(OzThetaFFArgs a) {
 // The polar stage of the analysis in float-float arithmetic (the Ozaki
 // path): A[lm] = sum_{j < ceil(n_theta / 2)} T_j[lm] (F_j + s F_j')[t], with
 // s = +1 for even l + m and -1 for odd (the cell integrals of P_l^m sin theta
-// have the parity of l + m; a middle row enters once), as in k_sep_theta.
+// have the parity of l + m; a middle row enters once), as in k_sep_theta64.
 // One block per shell: its F rows scaled by a power of two (the shell's
 // largest |F| below 1) and split into fp32 pairs, the mirrored sums and
 // differences formed in float-float and staged in shared memory, then one
@@ -2836,7 +2836,8 @@ __global__ void __launch_bounds__(256) k_rotate_ff(int n_r, int n_lm, int lmax, 
 // |rho w| below 2^(e - 1)) is bounded from the operands' upper words: for a positive
 // float64, exponent + mantissa is its logarithm less at most 0.0861, so the
 // largest sum of the two words, plus 0.1723, bounds the largest product.  Rows
-// beyond 2^+-900 (or without a finite scale) take X from the bits of the products.
+// beyond 2^+-900 are brought back by a power of two first, so that rho 2^k has the
+// digits of rho everywhere.
 // The digits of X (or of the sums below) are the bytes of X + 127 (1 + 2^8 + ... +
 // 2^32) + 2^50, signs included: five in [-127, 128] and the top one.
 //
@@ -2910,39 +2911,32 @@ __global__ void __launch_bounds__(256) k_rhow_ozaki(OzRhoArgs a) {
   }
   top = __reduce_max_sync(0xffffffffu, top);
   largest = __reduce_max_sync(0xffffffffu, largest);
-  int e = (int)((top + 180700u) >> 20) - 2044;   // 180700 > 0.1723 2^20; |rho w| < 2^(e - 1)
+  int e = max((int)((top + 180700u) >> 20) - 2044, -1400);   // 180700 > 0.1723 2^20; |rho w| < 2^(e - 1)
   long long base = 0, X[C][2];
-  bool zero = false;
-  if (e >= -900 && e <= 900 && largest < 0x7FF00000u) {
-    const double magic = __hiloint2double((e + 4 + 1023) << 20 | 0x80000, 0);   // 1.5 2^(e + 4)
+  auto take = [&](int exponent, auto value) {   // X from the products in units of 2^(exponent - 48)
+    const double magic = __hiloint2double((exponent + 4 + 1023) << 20 | 0x80000, 0);   // 1.5 2^(exponent + 4)
     base = __double_as_longlong(magic);
 #pragma unroll
     for (int c = 0; c < C; ++c)
 #pragma unroll
-      for (int h = 0; h < 2; ++h) X[c][h] = __double_as_longlong(fma(x[c][h], w[c][h], magic));
-  } else {
-    unsigned long long mb = 0ull;
+      for (int h = 0; h < 2; ++h) X[c][h] = __double_as_longlong(fma(value(x[c][h]), w[c][h], magic));
+  };
+  if (e >= -900 && e <= 900 && largest < 0x7FF00000u) {
+    take(e, [](double v) { return v; });
+  } else if (largest < 0x7FF00000u) {
+    const int far = e > 0 ? 600 : -600;
+    const double back = __hiloint2double((1023 - far) << 20, 0);
+    take(e - far, [&](double v) { return v * back; });
+  } else {   // a value without a finite magnitude: the row at the top of the range, integers of 48 bits from any bits
+    e = 1026;
 #pragma unroll
     for (int c = 0; c < C; ++c)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        X[c][h] = __double_as_longlong(x[c][h] * w[c][h]);
-        mb = max(mb, (unsigned long long)X[c][h] & 0x7FFFFFFFFFFFFFFFull);
-      }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, off));
-    const int exm = (int)(mb >> 52);
-    zero = exm == 0;
-    e = exm - 1021;
-#pragma unroll
-    for (int c = 0; c < C; ++c)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const unsigned long long u = (unsigned long long)X[c][h];
-        const int ex = (int)((u >> 52) & 0x7FFu), sh = 1027 - ex + e;
-        long long v = 0;
-        if (exm != 0 && ex != 0 && sh < 64) v = (long long)(((((u & 0xFFFFFFFFFFFFFull) | (1ull << 52)) >> (sh - 1)) + 1ull) >> 1);
-        X[c][h] = X[c][h] < 0 ? -v : v;
+        const long long u = __double_as_longlong(x[c][h] * w[c][h]);
+        const int sh = 1027 - (int)((u >> 52) & 0x7FF) + e;
+        const long long v = sh < 64 ? (((u & 0xFFFFFFFFFFFFFll) | (1ll << 52)) >> (sh - 1)) + 1 >> 1 : 0;
+        X[c][h] = u < 0 ? -v : v;
       }
   }
   // sums: own + other less both constants; differences: own - other = own + ~other + 1
@@ -2974,7 +2968,7 @@ __global__ void __launch_bounds__(256) k_rhow_ozaki(OzRhoArgs a) {
 #pragma unroll
     for (int sl = 0; sl < 6; ++sl) dst[sl * (stride / 2) + (kFold ? 16 : 32) * c] = __byte_perm(d[0][sl], d[1][sl], order);
   }
-  if (lane == 0) a.rexp[row] = zero ? 0 : e + a.eb - 64;
+  if (lane == 0) a.rexp[row] = e + a.eb - 64;
 }
 
 }  // namespace yy

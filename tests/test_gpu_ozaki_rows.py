@@ -80,3 +80,19 @@ def test_scales(case, scale):
     g.prepare("fp64_ozaki")
     compare(g, rho, scale)
     g.close()
+
+
+@pytest.mark.parametrize("power", [-940, -880, 880, 940])
+def test_scale_is_exact_across_the_far_rows(power):
+    """rho 2^k gives 2^k times the result, bit for bit, also where rows are brought back
+    by a power of two before their digits are taken (beyond 2^+-900)."""
+    require_gpu()
+    yy = lib()
+    spec, rho = build((True, 4, 8, 65, 7), 1.0)
+    g = yy.Grid.from_spec(spec)
+    g.prepare("fp64_ozaki")
+    one = solve(g, rho, "fp64_ozaki")
+    far = solve(g, [np.ldexp(x, power) for x in rho], "fp64_ozaki")
+    for key in one:
+        assert np.array_equal(np.ldexp(one[key], power), far[key]), key
+    g.close()
