@@ -349,10 +349,9 @@ def kernel_work(name, spec, n_lm, gradient, prec):
         gk = 64 if L <= 31 else 128
         w = {"flop": rows * spec.n_phi * nt * J, "flop_kind": "tensor", "products": "ozaki_synth",
              "bytes": out_bytes + J * rows * gk * 5 * 2}
-    elif name.startswith("k_tc_pair<FormOzaki,3>/analysis") or name == "k_oz_analysis":
-        # l_max <= 31: sums and differences of mirrored cells, half of the slots each
-        k_pad = -(-spec.n_phi // 32) * 32 if L <= 31 else -(-spec.n_phi // 64) * 64
-        w = {"flop": (1.0 if L <= 31 else 2.0) * rows * spec.n_phi * nt, "flop_kind": "tensor", "products": "ozaki",
+    elif name == "k_oz_analysis":   # sums and differences of mirrored cells, half of the slots each
+        k_pad = -(-spec.n_phi // 32) * 32
+        w = {"flop": 1.0 * rows * spec.n_phi * nt, "flop_kind": "tensor", "products": "ozaki",
              "bytes": rows * k_pad * 6 * 2}
     elif name == "k_theta_ff":
         # float-float multiply-adds of Phi, g_r and g_theta (g_phi is formed
@@ -364,7 +363,7 @@ def kernel_work(name, spec, n_lm, gradient, prec):
     elif name == "k_q_ff":
         w = {"bytes": 2 * min(J, 3) * n_r2 * n_lm * f64}
     elif name == "k_rhow_ozaki":
-        k_pad = -(-spec.n_phi // 32) * 32 if L <= 31 else -(-spec.n_phi // 64) * 64
+        k_pad = -(-spec.n_phi // 32) * 32
         w = {"bytes": n_r2 * spec.n_ang * f64 + rows * k_pad * 6 * 2}
     elif name == "k_sep_theta_ff":
         nt_pad = -(-nt // 4) * 4

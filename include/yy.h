@@ -76,12 +76,15 @@ typedef enum {
  *             fp32 accumulation per K chunk, chunks summed in float64.
  *   YY_FP64_OZAKI  float64 results (the YY_FP64 tolerance) with the
  *             azimuthal stages of the separable analysis and synthesis on
- *             tcgen05 tensor cores by the Ozaki scheme: the rows (rho w, the
- *             polar-stage sums G) and the azimuthal / trig tables written as
- *             six balanced 8-bit digits (integers exact in bf16) under a
- *             power-of-two scale per row, the 26 digit products of levels
- *             <= 6 accumulated exactly in fp32 per level, levels combined in
- *             integers and rounded once to float64.  The polar stages and
+ *             tcgen05 tensor cores by the Ozaki scheme, over longitudes folded
+ *             by their mirror symmetry: the rows and the azimuthal / trig
+ *             tables written as balanced digits under a power-of-two scale per
+ *             row (analysis: sums and differences of mirrored cells of rho w,
+ *             six 8-bit digits in bf16, the 26 products of levels <= 6;
+ *             synthesis: the polar-stage sums G, five 10-bit digits in fp16,
+ *             the 15 products of levels <= 4), accumulated exactly in fp32
+ *             per level, levels combined in integers and rounded once to
+ *             float64.  The polar stages and
  *             the combination of the patches run in float-float arithmetic
  *             (unevaluated pairs of fp32 values, about 48 bits: exact
  *             products by fused multiply-add and exact sums by TwoSum) on the
@@ -91,9 +94,8 @@ typedef enum {
  *             than 640 cells per row).  Multiplying rho by a power of two
  *             multiplies every result by the same power exactly.
  *             Needs yy_grid_prepare and 2 l_max + 1 <= 127 (l_max <= 63);
- *             above l_max 30 the contractions take their general kernels
- *             (no spare bias columns in G rows of 64 slots, rows of 128
- *             slots past l_max 31, the analysis in tiles of 32 slots). */
+ *             above l_max 31 rows of G hold 128 slots and the analysis's
+ *             classes 64 slots each. */
 typedef enum {
   YY_FP64 = 0,
   YY_FP32 = 1,

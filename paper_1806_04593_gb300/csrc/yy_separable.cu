@@ -12,9 +12,9 @@
 //
 // which costs 2 N_ang (2 l_max + 1) + 2 n_theta n_lm flops per shell instead of
 // 2 N_ang n_lm for the dense contraction (12.6 times fewer at the 1-degree grid
-// with l_max = 25).  T = double computes everything in float64.  T = float
-// computes the azimuthal stage in fp32 on CUDA cores (it is bound by reading
-// the density), except that the m = 0 sums, which carry the monopole and so
+// with l_max = 25).  The float64 kernels (k_sep_phi64, k_sep_theta64) fold the cells by
+// the symmetries of both angles.  The fp32 ones (k_sep_phi32, k_sep_theta32) sum
+// in order, except that the m = 0 sums, which carry the monopole and so
 // dominate Phi, are compensated fp32 pairs in the azimuthal stage and float64
 // in the polar stage.
 #include <math.h>

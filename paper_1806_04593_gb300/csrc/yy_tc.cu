@@ -2838,10 +2838,10 @@ __global__ void __launch_bounds__(256) k_rotate_ff(int n_r, int n_lm, int lmax, 
 // largest sum of the two words, plus 0.1723, bounds the largest product.  Rows
 // beyond 2^+-900 are brought back by a power of two first, so that rho 2^k has the
 // digits of rho everywhere.
-// The digits of X (or of the sums below) are the bytes of X + 127 (1 + 2^8 + ... +
+// The digits of a sum are the bytes of it + 127 (1 + 2^8 + ... +
 // 2^32) + 2^50, signs included: five in [-127, 128] and the top one.
 //
-// kFold (k_oz_analysis): the digits are those of the sums and the differences of cell k
+// The digits are those of the sums and the differences of cell k
 // and its mirror n_phi - 1 - k (a middle cell enters the sums once, its differences
 // meet zeros of the table), for k < n_phi / 2 rounded up, first the sums: lanes 0-15 take the
 // cells k = 2 L + 32 c and then the sums, lanes 16-31 the mirrors and the differences
@@ -2861,9 +2861,9 @@ struct OzRhoArgs {
   int *rexp;                    // [rows_pad]
 };
 
-// C: pieces of a row, 64 of k_pad values or 32 of k_pad / 2 sums and differences.  Two values' digits of
+// C: pieces of a row, 32 of the k_pad / 2 sums and as many differences.  Two values' digits of
 // one slice go out as one 32-bit store of their bf16 patterns.
-template <int C, bool kFold>
+template <int C>
 __global__ void __launch_bounds__(256) k_rhow_ozaki(OzRhoArgs a) {
   pdl_wait();
   const int row = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
@@ -2872,8 +2872,8 @@ __global__ void __launch_bounds__(256) k_rhow_ozaki(OzRhoArgs a) {
   const int p = shell / a.n_r, i = shell % a.n_r;
   const double *rho = (p == 0 ? a.rho0 : a.rho1) + ((size_t)i * a.n_theta + j) * a.n_phi;
   const double *wj = a.w + (size_t)j * a.n_phi;
-  const int cells = kFold ? (a.n_phi + 1) / 2 : a.n_phi;
-  const bool mirror = kFold && lane >= 16;
+  const int cells = (a.n_phi + 1) / 2;
+  const bool mirror = lane >= 16;
   // a lane's two cells at, at + 1: columns k, k + 1, or k + 1, k of a mirror
   double x[C][2], w[C][2];
   unsigned int top = 0u, largest = 0u;
@@ -2882,7 +2882,7 @@ __global__ void __launch_bounds__(256) k_rhow_ozaki(OzRhoArgs a) {
   const bool pairs = (a.n_phi & 1) == 0;
 #pragma unroll
   for (int c = 0; c < C; ++c) {
-    const int k = kFold ? 2 * (lane & 15) + 32 * c : 2 * lane + 64 * c;
+    const int k = 2 * (lane & 15) + 32 * c;
     const int at = mirror ? a.n_phi - 2 - k : k;
     x[c][0] = x[c][1] = w[c][0] = w[c][1] = 0.0;
     if (pairs && k + 1 < cells) {
@@ -2941,20 +2941,19 @@ __global__ void __launch_bounds__(256) k_rhow_ozaki(OzRhoArgs a) {
   }
   // sums: own + other less both constants; differences: own - other = own + ~other + 1
   const long long digits = 0x7F7F7F7F7Fll + (1ll << 50);
-  const long long bias = !kFold ? digits - base : mirror ? digits + 1 : digits - 2 * base;
+  const long long bias = mirror ? digits + 1 : digits - 2 * base;
   const long long flip = mirror ? -1ll : 0ll;
   const unsigned int order = mirror ? 0x3276u : 0x7632u;
   const size_t stride = (size_t)a.rows_pad * a.k_pad;
-  const int width = kFold ? a.k_pad / 2 : a.k_pad, k0 = kFold ? 2 * (lane & 15) : 2 * lane;
+  const int width = a.k_pad / 2, k0 = 2 * (lane & 15);
   uint32_t *dst = reinterpret_cast<uint32_t *>(a.X + (size_t)row * a.k_pad + (mirror ? width : 0) + k0);
 #pragma unroll
   for (int c = 0; c < C; ++c) {
-    if ((kFold ? 32 : 64) * c >= width) break;
+    if (32 * c >= width) break;
     uint32_t d[2][6];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      long long Y = X[c][h] + bias;
-      if constexpr (kFold) Y += __shfl_xor_sync(0xffffffffu, X[c][1 - h], 16) ^ flip;
+      const long long Y = X[c][h] + bias + (__shfl_xor_sync(0xffffffffu, X[c][1 - h], 16) ^ flip);
       const uint32_t ylo = (uint32_t)Y, yhi = (uint32_t)((unsigned long long)Y >> 32);
       // the fp32 patterns of 2^23 + digit + 127 (top: + 1024), less the offset
       d[h][0] = __float_as_uint(__fsub_rn(__uint_as_float(0x4B000000u | (yhi >> 8)), 8388608.f + 1024.f));
@@ -2964,9 +2963,9 @@ __global__ void __launch_bounds__(256) k_rhow_ozaki(OzRhoArgs a) {
       d[h][4] = __float_as_uint(__fsub_rn(__uint_as_float(__byte_perm(ylo, 0x4B000000u, 0x7541)), 8388735.f));
       d[h][5] = __float_as_uint(__fsub_rn(__uint_as_float(__byte_perm(ylo, 0x4B000000u, 0x7540)), 8388735.f));
     }
-    if (kFold && k0 + 32 * c >= width) continue;
+    if (k0 + 32 * c >= width) continue;
 #pragma unroll
-    for (int sl = 0; sl < 6; ++sl) dst[sl * (stride / 2) + (kFold ? 16 : 32) * c] = __byte_perm(d[0][sl], d[1][sl], order);
+    for (int sl = 0; sl < 6; ++sl) dst[sl * (stride / 2) + 16 * c] = __byte_perm(d[0][sl], d[1][sl], order);
   }
   if (lane == 0) a.rexp[row] = e + a.eb - 64;
 }
@@ -2991,14 +2990,12 @@ struct yy_oz_tables {
   float2 *tbf;                  // [ceil(n_theta / 2)][n_lm]: the analysis table T as fp32 pairs
   float2 *Df;                   // [sum_l (2l+1)^2]: the rotation D^l as fp32 pairs (two patches)
   void *trig;                   // digit slices of trig 2^-qt: [9][b_rows_pad][gk]
-  // analysis (FormOzaki in fills of kFillK): rho w digit rows as operand A, the azimuthal table as operand B
-  int an_ok, an_kpad, an_bn, an_row_tiles, an_b_rows_pad, an_stages, an_slots, an_eb;
+  // analysis: folded rho w digit rows as operand A, the azimuthal table as operand B
+  int an_ok, an_kpad, an_b_rows_pad, an_slots, an_eb;   // an_slots: resident clusters of k_oz_analysis
   void *an_x;                   // [6][rows_pad][an_kpad]
   int *an_exp;                  // [rows_pad]
-  void *an_az;                  // [6][an_b_rows_pad][an_kpad, or folded: half of the cells, padded to 32]
-  yy::PairMaps an_maps;
-  int an_slots2;                // resident clusters of k_oz_analysis, with folded rows (0: the pair kernel serves)
-  yy::OzAnalysisMaps an_maps2;  // its maps
+  void *an_az;                  // [6][an_b_rows_pad][half of the cells, padded to 32]
+  yy::OzAnalysisMaps an_maps;
 };
 
 namespace yy {
@@ -3043,42 +3040,32 @@ static uint16_t bf16_int(int v) {
 }
 
 // Tables of the analysis by the Ozaki scheme; leaves an_ok = 0 (the float64
-// analysis serves) where the rows are longer than four fills.
+// analysis serves) where the rows are longer than 640 cells.
 static yy_status ozaki_prepare_analysis(yy_grid *g, yy_oz_tables *o) {
   typedef FormOzaki F;
   const int nt = 2 * g->lmax + 1;
-  if (g->n_phi > F::kFillK * F::kMaxFills || !g->sep_az || !g->sep_F) return YY_OK;
-  // l_max <= 31: folded rows and k_oz_analysis; otherwise the pair kernel
-  o->an_slots2 = 0;
-  if (g->lmax < kOzAnBN &&
-      cudaFuncSetAttribute(k_oz_analysis, cudaFuncAttributeMaxDynamicSharedMemorySize, kOzAnSmem) == cudaSuccess) {
-    cudaLaunchAttribute attr[2];
-    cudaLaunchConfig_t cfg = pair_config(64, kOzAnSmem, 0, attr);
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, (void *)k_oz_analysis, &cfg) == cudaSuccess && n > 0) o->an_slots2 = n;
+  if (g->n_phi > F::kMaxK || !g->sep_az || !g->sep_F) return YY_OK;
+  // classes of 32 slots up to l_max 31, of 64 up to 63
+  const int BN = g->lmax < 32 ? 32 : 64;
+  const auto kernel = BN == 32 ? k_oz_analysis<32> : k_oz_analysis<64>;
+  const int smem = BN == 32 ? OzAn<32>::kSmem : OzAn<64>::kSmem;
+  if (g->lmax >= 64 || cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return YY_OK;
   }
-  cudaGetLastError();
-  const bool fold = o->an_slots2 > 0;
-  const int half = (g->n_phi + 1) / 2, width = fold ? round_up(half, 32) : round_up(g->n_phi, kPadK);   // columns of the table
-  o->an_kpad = fold ? 2 * round_up(half, 16) : width;
-  o->an_bn = 32;   // seven level accumulators of bn columns within one 256-column TMEM buffer
-  o->an_row_tiles = (nt + o->an_bn - 1) / o->an_bn;
-  o->an_b_rows_pad = fold ? 2 * kOzAnBN : round_up(nt, o->an_bn);
-  o->an_stages = pair_stages<F>(o->an_bn, kEpiStageBytes);
-  if (!fold) {
-    if (o->an_stages < 2 ||
-        cudaFuncSetAttribute(k_tc_pair<F, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess)
-      return YY_OK;
+  {
     cudaLaunchAttribute attr[2];
-    cudaLaunchConfig_t cfg =
-        pair_config(64, o->an_stages * pair_stage_bytes<F>(o->an_bn) + kSmemFixed + kEpiStageBytes, 0, attr);
+    cudaLaunchConfig_t cfg = pair_config(64, smem, 0, attr);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, (void *)k_tc_pair<F, 3>, &cfg) != cudaSuccess || n < 1) {
+    if (cudaOccupancyMaxActiveClusters(&n, (void *)kernel, &cfg) != cudaSuccess || n < 1) {
       cudaGetLastError();
       return YY_OK;
     }
     o->an_slots = n;
   }
+  const int half = (g->n_phi + 1) / 2, width = round_up(half, 32);   // columns of the table
+  o->an_kpad = 2 * round_up(half, 16);
+  o->an_b_rows_pad = 2 * BN;
   cudaError_t e = cudaSuccess;
   auto A = [&](void **ptr, size_t bytes) {
     if (e == cudaSuccess) e = dmalloc(ptr, bytes);
@@ -3090,8 +3077,8 @@ static yy_status ozaki_prepare_analysis(yy_grid *g, yy_oz_tables *o) {
   A(&o->an_az, b_elems * F::kElem);
   if (e == cudaSuccess) e = cudaMemset(o->an_x, 0, x_bytes);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? YY_ERR_OOM : YY_ERR_CUDA;
-  // the azimuthal table az[k][t] (rows of sep_nt_pad) as operand B, rows t, or the
-  // cos slots by order and then, 32 rows on, the sin slots of the folded cells:
+  // the azimuthal table az[k][t] (rows of sep_nt_pad) of the folded cells as operand B:
+  // the cos slots by order and then, BN rows on, the sin slots, under
   // one scale 2^eb for all of it (every row's largest value is about d_phi)
   const int ntp = g->sep_nt_pad;
   std::vector<double> az((size_t)g->n_phi * ntp);
@@ -3104,21 +3091,20 @@ static yy_status ozaki_prepare_analysis(yy_grid *g, yy_oz_tables *o) {
   int E2 = 0;
   frexp(mx, &E2);   // mx < 2^E2
   o->an_eb = E2 + 1;
-  for (int k = 0; k < (fold ? half : g->n_phi) && mx > 0.0; ++k)
+  for (int k = 0; k < half && mx > 0.0; ++k)
     for (int t = 0; t < nt; ++t) {
       const bool sine = t > 0 && t % 2 == 0;
       double y = ldexp(az[(size_t)k * ntp + t], -o->an_eb);   // |y| < 1/2
-      if (fold && sine) y = 2 * k + 1 == g->n_phi ? 0.0 : -y;   // the differences are mirror less cell
-      const int row = !fold ? t : (sine ? kOzAnBN : 0) + (t + 1) / 2;
+      if (sine) y = 2 * k + 1 == g->n_phi ? 0.0 : -y;   // the differences are mirror less cell
+      const int row = (sine ? BN : 0) + (t + 1) / 2;
       int d[6];
       oz_digits((unsigned long long)floor(ldexp(fabs(y), 48) + 0.5), d);
       for (int s2 = 0; s2 < F::kPB; ++s2)
         sl[((size_t)s2 * o->an_b_rows_pad + row) * width + k] = bf16_int(y < 0 ? -d[s2] : d[s2]);
     }
   if (cudaMemcpy(o->an_az, sl.data(), b_elems * F::kElem, cudaMemcpyHostToDevice) != cudaSuccess) return YY_ERR_CUDA;
-  CUtensorMap *ma = fold ? &o->an_maps2.a : &o->an_maps.a[0], *mb = fold ? &o->an_maps2.b : &o->an_maps.b[0];
-  if (!make_map<F>(ma, o->an_x, o->an_kpad, F::kPA * o->rows_pad, kPairRows) ||
-      !make_map<F>(mb, o->an_az, width, F::kPB * o->an_b_rows_pad, fold ? kOzAnBN : o->an_bn / 2))
+  if (!make_map<F>(&o->an_maps.a, o->an_x, o->an_kpad, F::kPA * o->rows_pad, kPairRows) ||
+      !make_map<F>(&o->an_maps.b, o->an_az, width, F::kPB * o->an_b_rows_pad, BN))
     return YY_ERR_NOT_SUPPORTED;
   o->an_ok = 1;
   return YY_OK;
@@ -3152,67 +3138,31 @@ cudaError_t ozaki_analysis(yy_grid *g, const double *ry, const double *rg, cudaS
   ra.X = (__nv_bfloat16 *)o->an_x;
   ra.rexp = o->an_exp;
   const unsigned blocks = (unsigned)(((size_t)o->rows * 32 + 255) / 256);
-  constexpr int kCmax = FormOzaki::kFillK * FormOzaki::kMaxFills / 64;
-  auto rhow = o->an_slots2 > 0 ? (o->an_kpad <= 64 * 5   ? k_rhow_ozaki<5, true>
-                                  : o->an_kpad <= 64 * 6 ? k_rhow_ozaki<6, true>
-                                                         : k_rhow_ozaki<kCmax, true>)
-                               : (o->an_kpad <= 64 * 5 ? k_rhow_ozaki<5, false> : k_rhow_ozaki<kCmax, false>);
+  constexpr int kCmax = F::kMaxK / 64;
+  auto rhow = o->an_kpad <= 64 * 5 ? k_rhow_ozaki<5> : o->an_kpad <= 64 * 6 ? k_rhow_ozaki<6> : k_rhow_ozaki<kCmax>;
   cudaError_t e = launch_kernel(g, "k_rhow_ozaki", rhow, blocks, 256, 0, s, ra);
   if (e != cudaSuccess) return e;
-  if (o->an_slots2 > 0) {
-    OzAnalysisArgs z = {};
-    z.cells = o->rows;
-    z.cell_tiles = o->rows_pad / (2 * kPairRows);
-    z.cols = 2 * g->lmax + 1;
-    z.width = o->an_kpad / 2;
-    z.kb_class = (z.width + 31) / 32;
-    // exact level sums per fill (the epilogue adds the fills): a folded top digit is up
-    // to 256, so a level sum over K columns is at most 7 K 2^14, below 2^24 for K <= 146
-    z.kb_fill = (g->n_phi + 1) / 2 <= 146 ? 5 : 4;
-    z.a_rows = o->rows_pad;
-    z.b_rows = o->an_b_rows_pad;
-    z.ldo = g->sep_nt_pad;
-    z.out = g->sep_F;
-    z.cell_exp = o->an_exp;
-    z.err = g->err;
-    const int pairs = z.cell_tiles < o->an_slots2 ? z.cell_tiles : o->an_slots2;
-    cudaLaunchAttribute attr[2];
-    cudaLaunchConfig_t cfg = pair_config(pairs, kOzAnSmem, s, attr, overlap_allowed(g));
-    e = cudaLaunchKernelEx(&cfg, k_oz_analysis, o->an_maps2, z);
-    note_launch(g, "k_oz_analysis", s);
-    if (e != cudaSuccess) return e;
-    return ozaki_theta_analysis(g, s);
-  }
-  PairArgs a = {};
-  a.stages = o->an_stages;
-  a.cells = o->rows;
-  a.cell_tiles = o->rows_pad / (2 * kPairRows);
-  a.rows = 2 * g->lmax + 1;
-  a.row_tiles = o->an_row_tiles;
-  a.bn = o->an_bn;
-  a.kb_total = o->an_kpad * F::kElem / kRowBytes;
-  a.kb_chunk = F::kFillK * F::kElem / kRowBytes;   // exact level sums per fill; the epilogue adds the fills
-  a.k_splits = 1;
-  a.kb_per_split = a.kb_total;
-  a.a_rows = o->rows_pad;
-  a.b_rows = o->an_b_rows_pad;
-  a.out_mode = 3;
-  a.out_split = o->rows;
-  a.ldo = g->sep_nt_pad;
-  a.n_jobs = 1;
-  a.err = g->err;
-  a.job[0].out0 = g->sep_F;
-  a.job[0].out1 = g->sep_F;
-  a.job[0].cell_exp = o->an_exp;
-  a.job[0].ta = 0;
-  a.job[0].tb = 0;
-  const int tiles = a.cell_tiles * a.row_tiles;
-  const int pairs = tiles < o->an_slots ? tiles : o->an_slots;
+  OzAnalysisArgs z = {};
+  z.cells = o->rows;
+  z.cell_tiles = o->rows_pad / (2 * kPairRows);
+  z.cols = 2 * g->lmax + 1;
+  z.width = o->an_kpad / 2;
+  z.kb_class = (z.width + 31) / 32;
+  // exact level sums per fill (the epilogue adds the fills): a folded top digit is up
+  // to 256, so a level sum over K columns is at most 7 K 2^14, below 2^24 for K <= 146
+  z.kb_fill = (g->n_phi + 1) / 2 <= 146 ? 5 : 4;
+  z.a_rows = o->rows_pad;
+  z.b_rows = o->an_b_rows_pad;
+  z.ldo = g->sep_nt_pad;
+  z.out = g->sep_F;
+  z.cell_exp = o->an_exp;
+  z.err = g->err;
+  const int pairs = z.cell_tiles < o->an_slots ? z.cell_tiles : o->an_slots;
+  const bool small = o->an_b_rows_pad == 64;
   cudaLaunchAttribute attr[2];
-  cudaLaunchConfig_t cfg =
-      pair_config(pairs, o->an_stages * pair_stage_bytes<F>(o->an_bn) + kSmemFixed + kEpiStageBytes, s, attr, overlap_allowed(g));
-  e = cudaLaunchKernelEx(&cfg, k_tc_pair<F, 3>, o->an_maps, a);
-  note_launch(g, "k_tc_pair<FormOzaki,3>/analysis", s);
+  cudaLaunchConfig_t cfg = pair_config(pairs, small ? OzAn<32>::kSmem : OzAn<64>::kSmem, s, attr, overlap_allowed(g));
+  e = cudaLaunchKernelEx(&cfg, small ? k_oz_analysis<32> : k_oz_analysis<64>, o->an_maps, z);
+  note_launch(g, "k_oz_analysis", s);
   if (e != cudaSuccess) return e;
   return ozaki_theta_analysis(g, s);
 }

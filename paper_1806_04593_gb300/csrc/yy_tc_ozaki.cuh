@@ -1,48 +1,27 @@
-// The Ozaki form of the pair kernel: float64 results from exact products of
-// bf16 digits (output mode 3 of k_tc_pair), and its epilogue.  Included by
-// yy_tc_pair.cuh after the PTX wrappers it uses.
+// The analysis's Ozaki form: float64 results from exact products of bf16 digits,
+// and the sums of its levels (k_oz_analysis).  Included by yy_tc_pair.cuh after the
+// PTX wrappers it uses.
 #pragma once
 
 namespace yy {
 
 // Float64 results by the Ozaki scheme: each operand row is scaled by a power
 // of two to |x| <= 1/2 and written with six balanced base-256 digits,
-// x = sum_s a_s 2^(-8 (s + 1)) + r, integers |a_s| <= 128 (exact in bf16),
-// |r| <= 2^-49: the digits of round(|x| 2^48), each taken in [-127, 128]
-// with a carry into the next.  The products of digit levels L = s + t <= 6
-// (26 of the 36) are kept; the dropped ones add up to below 2^-56.  A
-// product sum over K <= 160 is at most 160 * 128^2 < 2^21.4, and a level has
-// at most 6 products, so every level accumulates in one TMEM accumulator
-// below 2^24 over a fill of up to 160: exact in fp32.  Longer K runs in
-// several fills, which the epilogue adds.  The epilogue combines levels 0-3
-// in int64 and the three lowest in fp32, and rounds once to float64.  The
+// x = sum_s a_s 2^(-8 (s + 1)) + r, integers |a_s| <= 128 (the first up to 256 for the sums
+// of two cells; exact in bf16), |r| <= 2^-49: the digits of round(x 2^48), each in
+// [-127, 128] with a carry into the next.  The products of digit levels
+// L = s + t <= 6 (26 of the 36) are kept; the dropped ones add up to below 2^-56.  A
+// level has at most 6 products, one with a first digit of the cells, so over K <= 146
+// columns it stays below 7 * 146 * 2^14 < 2^24 and accumulates exactly in fp32.
+// Longer K runs in several fills, which the epilogue adds.  The epilogue combines
+// levels 0-3 in int64 and the three lowest in fp32, and rounds once to float64.  The
 // digits are rounded to nearest, so their representation errors take either
 // sign and grow like sqrt(K) along K rather than like K.
-// Products in level order; level L has s = max(0, L - 5) .. min(L, 5).
 struct FormOzaki {
   typedef __nv_bfloat16 elem;
-  static constexpr int kKind = KIND_BF16, kElem = 2, kPA = 6, kPB = 6, kPairs = 26, kAccs = 7;
-  // K per accumulator fill (a level sum stays below 6 * 160 * 2^14 < 2^24), and
-  // the longest K taken: the epilogue adds up to four fills in int64 / fp32
-  static constexpr int kFillK = 160, kMaxFills = 4;
-  __host__ __device__ static constexpr int s_lo(int L) { return L > 5 ? L - 5 : 0; }
-  // first product of level L (levels hold 1, 2, 3, 4, 5, 6, 5 products)
-  __host__ __device__ static constexpr int start(int L) {
-    return L <= 0 ? 0 : L == 1 ? 1 : L == 2 ? 3 : L == 3 ? 6 : L == 4 ? 10 : L == 5 ? 15 : L == 6 ? 21 : 26;
-  }
-  __host__ __device__ static constexpr int level(int i) {
-    return i < 1 ? 0 : i < 3 ? 1 : i < 6 ? 2 : i < 10 ? 3 : i < 15 ? 4 : i < 21 ? 5 : 6;
-  }
-  __host__ __device__ static constexpr int pa(int i) { return s_lo(level(i)) + i - start(level(i)); }
-  __host__ __device__ static constexpr int pb(int i) { return level(i) - pa(i); }
-  __host__ __device__ static constexpr int acc(int i) { return level(i); }
-  __host__ __device__ static constexpr bool first(int i) { return i == start(level(i)); }
+  static constexpr int kKind = KIND_BF16, kElem = 2, kPA = 6, kPB = 6, kAccs = 7;
+  static constexpr int kMaxK = 640;   // cells of the longest row taken: up to three fills a class
 };
-
-static_assert(FormOzaki::start(7) == 26 && FormOzaki::level(25) == 6 && FormOzaki::pa(25) == 5 &&
-                  FormOzaki::pb(25) == 1 && FormOzaki::pa(21) == 1 && FormOzaki::first(21) &&
-                  FormOzaki::pa(20) == 5 && FormOzaki::pb(20) == 0 && !FormOzaki::first(20),
-              "Ozaki product table");
 
 // v 2^e exactly, for |v| < 2^53 and a result in the normal range, built
 // from the bits: |v| shifted so that its top bit lands on bit 52 (the

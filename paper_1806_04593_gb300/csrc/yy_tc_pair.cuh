@@ -367,7 +367,7 @@ __device__ __forceinline__ float f64_to_f32(double x) {
 }  // namespace yy
 
 // the Ozaki forms (float64 results from exact bf16 digit products) and their
-// epilogue, for out_mode 3
+// epilogue
 #include "yy_tc_ozaki.cuh"
 
 namespace yy {
@@ -396,7 +396,6 @@ struct PairJob {
                                 // (out_mode 2: cell c < out_split -> out0 + c ldo, ...)
   const float *cell_scale, *row_scale, *row_add;
   const float *cell_add;        // out_mode 2: added to every value of the cell
-  const int *cell_exp;          // out_mode 3: power of two of a unit level-6 sum in the cell's row
   int ta, tb;                   // operand maps of this job
 };
 
@@ -413,8 +412,7 @@ struct PairArgs {
                                 // sums go out as one partial
   int a_rows, b_rows;           // rows of one piece in the stacked A / B operands
   int out_mode;                 // 1: scaled float64 job outputs; 0: raw fp32 partial sums;
-                                // 2: scaled float64 outputs stored along the rows of each cell;
-                                // 3: as 2, from the exact level sums of FormOzaki;
+                                // 2: scaled float64 outputs stored along the rows of each cell
   float *part;                  // mode 0: part[(segment rows + row) part_ld + cell]
   int part_ld;
   int out_split;
@@ -597,7 +595,7 @@ k_tc_pair(const __grid_constant__ PairMaps maps0, const __grid_constant__ PairAr
         const PairArgs &a = GROUPED ? a0.group[f_] : a0;
         const int per_job = a.cell_tiles * a.row_tiles * a.k_splits;
         // K blocks per accumulator fill (modes 0 and 3 add the fills in the epilogue)
-        const int chunk = ((OUT_MODE == 0 || OUT_MODE == 3) && a.kb_chunk > 0) ? a.kb_chunk : a.kb_total;
+        const int chunk = (OUT_MODE == 0 && a.kb_chunk > 0) ? a.kb_chunk : a.kb_total;
         const uint32_t idesc = instr_desc_pair<F>(a.bn);
         const int tl = t % per_job;
         TileFills tf(a, tl / (a.row_tiles * a.cell_tiles));
@@ -667,7 +665,7 @@ k_tc_pair(const __grid_constant__ PairMaps maps0, const __grid_constant__ PairAr
         const PairArgs &a = GROUPED ? a0.group[f_] : a0;
         const int per_job = a.cell_tiles * a.row_tiles * a.k_splits;
         // K blocks per accumulator fill (modes 0 and 3 add the fills in the epilogue)
-        const int chunk = ((OUT_MODE == 0 || OUT_MODE == 3) && a.kb_chunk > 0) ? a.kb_chunk : a.kb_total;
+        const int chunk = (OUT_MODE == 0 && a.kb_chunk > 0) ? a.kb_chunk : a.kb_total;
         const int n_chunks = a.bn / kEpiCols;
         const int tl = t % per_job;
         const int rt = tl % a.row_tiles, ct = (tl / a.row_tiles) % a.cell_tiles;
@@ -726,97 +724,20 @@ k_tc_pair(const __grid_constant__ PairMaps maps0, const __grid_constant__ PairAr
         }
         if (!ok) break;
       }
-    } else if constexpr (OUT_MODE == 2 || OUT_MODE == 3) {
+    } else if constexpr (OUT_MODE == 2) {
       // Cells are rows of the output arrays (stride ldo) and the accumulator
       // columns run along them: each lane holds 16 consecutive values of its
       // cell's row.  They go through this warp's shared-memory block, and the
       // warp then writes two cells' 16-value runs per store instruction.
-      // Mode 3 forms the values from FormOzaki's level accumulators.
       static_assert(!GROUPED, "grouped launches take output modes 0 and 1");
       const PairArgs &a = a0;
       const int per_job = a.cell_tiles * a.row_tiles * a.k_splits;
       const int total = per_job * a.n_jobs;
-      const int chunk = (OUT_MODE == 3 && a.kb_chunk > 0) ? a.kb_chunk : a.kb_total;
       const int n_chunks = a.bn / kEpiCols;
       uint8_t *wbuf = smem + S * STAGE + 512 + (size_t)(warp - 2) * kEpiWarpBytes;
       double *ebuf = reinterpret_cast<double *>(wbuf);                          // [32][kEpiPad]
       double **rowp = reinterpret_cast<double **>(wbuf + 32 * kEpiPad * 8);     // [32] output rows
       const bool vec = (a.ldo & 1) == 0;   // rows start on 16-byte boundaries (with 16-byte aligned bases)
-      if constexpr (OUT_MODE == 3) {
-        // FormOzaki: the tile's fills (kb_chunk K blocks each) are added in
-        // registers, level by level; this warp owns the 8-column chunk sub
-        // (bn <= 8 kEpiPerQuarter), and the values are formed after the last fill.
-        const int k = sub;
-        const bool mine = k < a.bn / 8;
-        for (int t = pair; t < total; t += n_pairs) {
-          const PairJob &J = a.job[t / per_job];
-          const int tl = t % per_job;
-          const int rt = tl % a.row_tiles, ct = (tl / a.row_tiles) % a.cell_tiles;
-          TileFills tf(a, tl / (a.row_tiles * a.cell_tiles));
-          const int nkb = tf.nkb;
-          const int cell = (2 * ct + rank) * kPairRows + quarter * 32 + lane;
-          const bool cell_ok = cell < a.cells;
-          const int ce = cell_ok ? J.cell_exp[cell] : 0;
-          __syncwarp();   // the previous tile's row pointers are no longer read
-          rowp[lane] = !cell_ok ? nullptr
-                       : (cell < a.out_split) ? J.out0 + (size_t)cell * a.ldo
-                                              : J.out1 + (size_t)(cell - a.out_split) * a.ldo;
-          long long hi[8];
-          float lo[8];
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            hi[j] = 0;
-            lo[j] = 0.0f;
-          }
-          bool ok = true;
-          for (int c0 = 0, c1 = 0; c0 < nkb; c0 = c1, ++it) {
-            c1 = tf.fill_end(c0, chunk);
-            tf.advance(a, c1);
-            const int b = it & 1;
-            if (!mbar_wait_cluster(&tfull[b], (it >> 1) & 1, a.err)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-            const uint32_t tbase = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * 256);
-            if (mine) ozaki_accumulate(tbase + (uint32_t)(k * 8), a.bn, hi, lo);
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster_relaxed(tempty_even + (uint32_t)(b * sizeof(uint64_t)));
-          }
-          if (!ok) break;
-          if (mine) {
-            const int row0 = rt * a.bn + k * 8;
-            ozaki_finish(hi, lo, ce, ebuf + lane * kEpiPad);
-            __syncwarp();
-            if (vec) {
-              // lanes 4 c' + e: cell 8 q + c', values 2 e and 2 e + 1 of the run
-              const int e = lane & 3, row = row0 + 2 * e;
-#pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                const int c = 8 * q + (lane >> 2);
-                double *orow = rowp[c];
-                const double2 val = *reinterpret_cast<const double2 *>(ebuf + c * kEpiPad + 2 * e);
-                if (orow != nullptr) {
-                  if (row + 1 < a.rows)
-                    *reinterpret_cast<double2 *>(orow + row) = val;
-                  else if (row < a.rows)
-                    orow[row] = val.x;
-                }
-              }
-            } else {
-              const int e = lane & 7, row = row0 + e;
-#pragma unroll
-              for (int q = 0; q < 8; ++q) {
-                const int c = 4 * q + (lane >> 3);
-                double *orow = rowp[c];
-                if (orow != nullptr && row < a.rows) orow[row] = ebuf[c * kEpiPad + e];
-              }
-            }
-            __syncwarp();
-          }
-        }
-      } else
       for (int t = pair; t < total; t += n_pairs, ++it) {
         const int b = it & 1;
         const PairJob &J = a.job[t / per_job];
