@@ -20,6 +20,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "yy_internal.h"
 
@@ -268,9 +269,12 @@ __global__ void k_fold_az(int m1, int nt_pad, AzFold f, const double *__restrict
 // each, lane = k), round and weight it and write it transposed; all threads sum
 // it, R rows x 4 functions each, the table's piece in shared memory beside it
 // (through L1 it came from L2: the staged rows leave L1 little room).  On the
-// 1-degree grid, 550 zones, l_max 25: 167 us (300 us with whole shells staged and
-// the table read per 16 products), about 70 of them instruction issue; 23 us
-// against 48 on the 2-degree grid of 200 zones at l_max 15.  The row's compensated sum (the m = 0
+// 1-degree grid, 550 zones, l_max 25: 155 us (300 us with whole shells staged and
+// the table read per 16 products), bound by instruction issue; 22 us
+// against 48 on the 2-degree grid of 200 zones at l_max 15.  Every other row is narrowed
+// by the conversion instruction, on the float64 pipe, idle here (same rounding: all by
+// integer operations 168 us, all by the instruction 161); whole pieces of whole blocks
+// take no checks per value (162 without).  The row's compensated sum (the m = 0
 // azimuthal sum without the factor d_phi) is formed by the lanes as they convert:
 // lane L adds k = L, L + 32, ... to an unevaluated fp32 pair, and shuffles add the
 // lanes' pairs.
@@ -317,11 +321,18 @@ __global__ void k_sep_phi32(const SepPhi32 a) {
   auto fetch = [&](int p) {
     const int k = p * kPiece + lane;
     if (loads && k < a.n_phi) {
+      const double *x = src + q * a.n_phi + k;
+      if (rows == kRows32) {
 #pragma unroll
-      for (int i = 0; i < kLoadRows; ++i) {
-        if (q + i >= rows) break;
-        copy_async(&raw[q + i][lane], src + (q + i) * a.n_phi + k);
-        copy_async(&wts[q + i][lane], a.w + wrow[i] + k);
+        for (int i = 0; i < kLoadRows; ++i) {
+          copy_async(&raw[q + i][lane], x + i * a.n_phi);
+          copy_async(&wts[q + i][lane], a.w + wrow[i] + k);
+        }
+      } else {
+        for (int i = 0; i < kLoadRows && q + i < rows; ++i) {
+          copy_async(&raw[q + i][lane], x + i * a.n_phi);
+          copy_async(&wts[q + i][lane], a.w + (j0 + q + i) % a.n_theta * a.n_phi + k);
+        }
       }
     }
     const int n = min(kPiece, a.n_phi - p * kPiece) * a.nt_pad;
@@ -341,16 +352,23 @@ __global__ void k_sep_phi32(const SepPhi32 a) {
   for (int p = 0; p < pieces; ++p) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (loads) {
-      const bool in = p * kPiece + lane < a.n_phi;
       float v[kLoadRows];
+      auto convert = [&](auto whole) {
 #pragma unroll
-      for (int i = 0; i < kLoadRows; ++i) {
-        v[i] = 0.0f;
-        if (in && q + i < rows) {
-          v[i] = __fmul_rn(narrow(raw[q + i][lane]), wts[q + i][lane]);   // rounded before the pair's sum
-          pair_add(h[i], l[i], v[i]);
+        for (int i = 0; i < kLoadRows; ++i) {
+          v[i] = 0.0f;
+          if (decltype(whole)::value || (p * kPiece + lane < a.n_phi && q + i < rows)) {
+            const double x = raw[q + i][lane];
+            // rounded before the pair's sum
+            v[i] = __fmul_rn(i & 1 ? __double2float_rn(x) : narrow(x), wts[q + i][lane]);
+            pair_add(h[i], l[i], v[i]);
+          }
         }
-      }
+      };
+      if (rows == kRows32 && (p + 1) * kPiece <= a.n_phi)
+        convert(std::true_type());
+      else
+        convert(std::false_type());
       float4 *to = reinterpret_cast<float4 *>(&xs[p & 1][lane * kLd32 + q]);
       to[0] = make_float4(v[0], v[1], v[2], v[3]);
       to[1] = make_float4(v[4], v[5], v[6], v[7]);

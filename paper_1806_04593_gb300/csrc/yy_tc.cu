@@ -380,8 +380,11 @@ k_pack_reg(PackBatch batch) {
 // copied to shared memory in three pieces with a barrier each, and one thread starts
 // the copy of the next row's piece as soon as every thread holds the current one's in
 // registers: the next row is in flight while the rest of this one is read, reduced
-// and stored.  1100 rows of 24300 cells: 74 us in FormFP16x2, 79 in FormBF16x3 (87 and
+// and stored.  1100 rows of 24300 cells: 72 us in FormFP16x2, 78 in FormBF16x3 (87 and
 // 91 with the next row started after the whole one); each SM takes seven or eight rows.
+// Bound by instruction issue: a quarter of the values is narrowed by the conversion
+// instruction on the idle float64 pipe (same rounding; 75 and 79 with none, 74 and 79
+// with half of them).
 // Only the density job takes this form (no columns or rows left out, no
 // weight rows, an even row length, 16-byte aligned rows; the launcher checks),
 // so its predicates are per pair of elements; the arithmetic and its order are
@@ -476,7 +479,7 @@ __device__ __forceinline__ bool stream_row(const PackArgs &p, int row, double *r
       if (valid && k < K) {
         const double2 t = *(const double2 *)(rowbuf + k);
         v0 = f64_to_f32_rn(t.x);
-        v1 = f64_to_f32_rn(t.y);
+        v1 = c & 1 ? __double2float_rn(t.y) : f64_to_f32_rn(t.y);
         st.mn = fminf(st.mn, fminf(v0, v1));
         st.mx = fmaxf(st.mx, fmaxf(v0, v1));
       }
