@@ -42,12 +42,15 @@ struct SynthOut {
 //    there up to signs that follow m mod 4, odd orders exchange cos and sin: sums
 //    of even m apart by m mod 4 (one product per slot) and of odd m with both
 //    functions (two per slot) give up to eight cells.
+// The monopole (l = 0 of slot 0, then slot 0) is added last, to each row and to each
+// cell apart: two roundings at the size of Phi and g_r.  (Inside the folded sums it
+// took up to six: 4.7 units of 2^-53 at worst instead of 2, rms 1.05e-16 instead of 6.8e-17.)
 // Columns and their images: AzFold.  On the 1-degree Yin-Yang grid 45 columns
-// give the 270 cells: 15.5 float64 operations per output at l_max 25 instead of
-// 51 (18.7 with pi - phi alone).  Measured there, 550 zones, with the gradient:
-// 3.27 ms, against 3.98 ms with pi - phi alone and 12.9 ms for one thread
-// per four cells without the folds; 2-degree grid, 200 zones, l_max 15: 246 us,
-// 289 and 707.
+// give the 270 cells: 16.4 float64 operations per output at l_max 25 instead of
+// 51.  Measured there, 550 zones, with the gradient: 3.47 ms, against 12.9 ms for one
+// thread per four cells without the folds; 2-degree grid, 200 zones, l_max 15: 254 us
+// and 707.  (With the monopole inside the sums, 15.5 operations: 3.27 ms and 246 us, and
+// with pi - phi alone, 18.7: 3.98 ms and 289 us.)
 struct Synth64 {
   int n_r, n_theta, n_phi, lmax, n_lm, chunks;
   AzFold fold;
@@ -112,12 +115,12 @@ __device__ __forceinline__ void phi_quarter(const Synth64 &a, const double *g, i
   for (int r = 0; r < R; ++r) {
     double *o = dst[r];
     if (o == nullptr) continue;
-    const double cz = c0[r] + g[r];   // m = 0
-    const double e1 = cz + c2[r], e2 = cz - c2[r], f1 = s0[r] + s2[r], f2 = s0[r] - s2[r];
+    const double z = g[r];   // m = 0, added last
+    const double e1 = c0[r] + c2[r], e2 = c0[r] - c2[r], f1 = s0[r] + s2[r], f2 = s0[r] - s2[r];
     auto put = [&](int col, double C, double S) {
       const int kp = first + col, km = a.n_phi - 1 - kp;
-      o[kp] = C + S;
-      if (km != kp) o[km] = C - S;
+      o[kp] = z + (C + S);
+      if (km != kp) o[km] = z + (C - S);
     };
     put(c, e1 + cc[r], f1 + ss[r]);
     if (wb) put(kb, e2 + cs[r], sc[r] - f2);
@@ -162,19 +165,31 @@ __global__ void __launch_bounds__(256, 3) k_synth_f64(const Synth64 a, int jp) {
         s[2] = fma(q[2 * a.qsz + at], a.dP[row + at], s[2]);
       }
     };
+    const int least = t == 0 ? 1 : m;   // the monopole is added last
     int l = a.lmax;
-    for (; l > m; l -= 2) {
+    for (; l > least; l -= 2) {
       term(l, x);
       term(l - 1, y);
     }
-    if (l == m) term(l, x);
+    if (l == least) term(l, x);
     const bool odd = ((a.lmax + m) & 1) != 0;   // parity of x's terms
     double *g = Gs + (size_t)t * ld + 2 * jj;
     auto put = [&](double *at, double v0, double v1) { *reinterpret_cast<double2 *>(at) = make_double2(ok ? v0 : 0.0, ok ? v1 : 0.0); };
-    const double up = x[0] + y[0], um = odd ? y[0] - x[0] : x[0] - y[0];
+    auto sides = [&](const double *coef, double u, double v, double &plus, double &minus) {
+      plus = u + v;
+      minus = odd ? v - u : u - v;
+      if (t == 0) {
+        plus = fma(coef[0], a.P[row], plus);
+        minus = fma(coef[0], a.P[row], minus);
+      }
+    };
+    double up, um;
+    sides(q, x[0], y[0], up, um);
     put(g, up, um);
     if constexpr (NF == 4) {
-      put(g + 2 * jp, x[1] + y[1], odd ? y[1] - x[1] : x[1] - y[1]);
+      double radial_p, radial_m;
+      sides(q + a.qsz, x[1], y[1], radial_p, radial_m);
+      put(g + 2 * jp, radial_p, radial_m);
       put(g + 4 * jp, x[2] + y[2], odd ? x[2] - y[2] : y[2] - x[2]);   // dP has the other parity
       const int to = t == 0 ? 0 : ((t & 1) ? t + 1 : t - 1);
       const double fac = (t & 1 ? 1.0 : -1.0) * m * a.isin[ok ? j : 0] * inv_r;
@@ -225,14 +240,14 @@ __global__ void __launch_bounds__(256, 3) k_synth_f64(const Synth64 a, int jp) {
     for (int r = 0; r < kR64; ++r) {
       double *o = dst[r0 + r];
       if (o == nullptr) continue;
-      const double cz = ce[r] + g[r];   // m = 0
-      const double C = cz + co[r], S = se[r] + so[r];
-      o[kp] = C + S;
-      if (km != kp) o[km] = C - S;
+      const double z = g[r];   // m = 0, added last
+      const double C = ce[r] + co[r], S = se[r] + so[r];
+      o[kp] = z + (C + S);
+      if (km != kp) o[km] = z + (C - S);
       if (pair) {
-        const double Cq = cz - co[r], Sq = so[r] - se[r];
-        o[kq] = Cq + Sq;
-        if (a.n_phi - 1 - kq != kq) o[a.n_phi - 1 - kq] = Cq - Sq;
+        const double Cq = ce[r] - co[r], Sq = so[r] - se[r];
+        o[kq] = z + (Cq + Sq);
+        if (a.n_phi - 1 - kq != kq) o[a.n_phi - 1 - kq] = z + (Cq - Sq);
       }
     }
   }
