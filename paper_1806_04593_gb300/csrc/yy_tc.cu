@@ -2838,8 +2838,9 @@ __global__ void __launch_bounds__(256) k_rotate_ff(int n_r, int n_lm, int lmax, 
 // worth 2^(e - 48): its bits less the constant's are X.  The row's scale 2^e (every
 // |rho w| below 2^(e - 1)) is bounded from the operands' upper words: for a positive
 // float64, exponent + mantissa is its logarithm less at most 0.0861, so the
-// largest sum of the two words, plus 0.1723, bounds the largest product.  Rows
-// beyond 2^+-900 are brought back by a power of two first, so that rho 2^k has the
+// largest sum of the two words, plus 0.1723, bounds the largest product.  Where that
+// crosses a power of two (17 percent of the mantissas) the row's products decide, so that
+// every row enters with 48 bits.  Rows beyond 2^+-900 are brought back by a power of two first, so that rho 2^k has the
 // digits of rho everywhere.
 // The digits of a sum are the bytes of it + 127 (1 + 2^8 + ... +
 // 2^32) + 2^50, signs included: five in [-127, 128] and the top one.
@@ -2853,9 +2854,9 @@ __global__ void __launch_bounds__(256) k_rotate_ff(int n_r, int n_lm, int lmax, 
 //
 // The integer pipe was the bound (86 percent busy with X taken from the bits of every
 // product and sign and magnitude kept apart; float64 additions for the folds, at two
-// operations per clock per SM, took 190 us); now memory is, 92 us at 6.0 TB/s on the
-// 1-degree grid at 550 zones (101 unfolded, of 320 columns) and 67 at 300 zones of a
-// 1-degree polar grid (91).
+// operations per clock per SM, took 190 us); now memory is, 95 us at 5.8 TB/s on the
+// 1-degree grid at 550 zones (101 unfolded, of 320 columns; 92 with the bound alone as the
+// scale) and 67 at 300 zones of a 1-degree polar grid (91).
 struct OzRhoArgs {
   int n_r, n_theta, n_phi, rows, k_pad, rows_pad, eb;
   const double *rho0, *rho1;    // [n_r][n_theta][n_phi] per patch (rho1 NULL on a polar grid)
@@ -2915,6 +2916,15 @@ __global__ void __launch_bounds__(256) k_rhow_ozaki(OzRhoArgs a) {
   top = __reduce_max_sync(0xffffffffu, top);
   largest = __reduce_max_sync(0xffffffffu, largest);
   int e = max((int)((top + 180700u) >> 20) - 2044, -1400);   // 180700 > 0.1723 2^20; |rho w| < 2^(e - 1)
+  if ((top + 180700u) >> 20 != top >> 20) {   // the bound may be one power too large: from the products themselves
+    unsigned int most = 0u;
+#pragma unroll
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) most = max(most, (unsigned int)__double2hiint(x[c][h] * w[c][h]) & 0x7FFFFFFFu);
+    most = __reduce_max_sync(0xffffffffu, most) >> 20;
+    if (most > 0u && most < 0x7FFu) e = (int)most - 1021;
+  }
   long long base = 0, X[C][2];
   auto take = [&](int exponent, auto value) {   // X from the products in units of 2^(exponent - 48)
     const double magic = __hiloint2double((exponent + 4 + 1023) << 20 | 0x80000, 0);   // 1.5 2^(exponent + 4)
