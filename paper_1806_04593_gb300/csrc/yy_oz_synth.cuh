@@ -27,7 +27,7 @@
 // (Six base-256 digits in bf16 with the whole row in one class: seven accumulators
 // per cell, 26 products over 64 slots and all longitudes, 511 us on the 1-degree
 // grid at l_max 25 with the gradient; this form 348; 180 x 360 polar grid of 300 zones: 377 and 260; l_max 40 on 61 x
-// 185 cells, 317 zones: 412 and 213.)
+// 185 cells, 317 zones: 412 and 217.)
 //
 // Schedule: a CTA pair (cluster of two, cta_group::2, M = 256 rows) takes a
 // cell tile of 256 rows of one field, loads its G digits once and runs every tile
@@ -398,13 +398,13 @@ k_oz_synth(const __grid_constant__ OzSynthMaps maps, const __grid_constant__ OzS
                   // half of the values through the float64 pipe's conversion,
                   // half by integer formatting: the epilogue's issue slots are its
                   // limit, and with more the float64 pipe (six of eight: 356
-                  // against 352 us, all: 379).  The formatting takes values below
-                  // 2^53: four classes halve theirs for it.
+                  // against 352 us, all: 379).  Values of four classes
+                  // may reach 2^54.
 #pragma unroll
                   for (int j = 0; j < 8; ++j) {
                     const long long V = sg ? vc[g + j] - v[j] : vc[g + j] + v[j];
                     ebuf[lane * kOzEpiPad + (sg ? 7 - j : j)] = (j & 1) == 0 ? i64_ldexp_row_cvt(V, ce)
-                                                                : NCLS == 4  ? i64_ldexp_row(V >> 1, ce + 1)
+                                                                : NCLS == 4  ? i64_ldexp_row54(V, ce)
                                                                              : i64_ldexp_row(V, ce);
                   }
                 } else {

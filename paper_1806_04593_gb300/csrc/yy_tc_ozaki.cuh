@@ -50,7 +50,19 @@ __device__ __forceinline__ double i64_ldexp_row(long long v, int e) {
   return __longlong_as_double((long long)(u == 0ull ? 0ull : b));
 }
 
-// The same through the float64 pipe's conversion (exact: |v| < 2^53) and an
+// i64_ldexp_row for |v| < 2^54, rounded to nearest even (e in [-1022, 970]): the
+// top bit on bit 53, so that the bit below the last one decides.
+__device__ __forceinline__ double i64_ldexp_row54(long long v, int e) {
+  const unsigned long long s = (unsigned long long)(v >> 63);
+  const unsigned long long u = ((unsigned long long)v ^ s) - s;
+  const int lz = __clzll((long long)u);
+  const unsigned long long t = u << ((lz - 10) & 63);
+  const unsigned long long m = (t + ((t >> 1) & 1)) >> 1;   // a carry into bit 53 steps the exponent
+  const unsigned long long b = (m + ((unsigned long long)(1085 - lz + e) << 52)) | (s << 63);
+  return __longlong_as_double((long long)(u == 0ull ? 0ull : b));
+}
+
+// The same through the float64 pipe's conversion (to nearest; exact for |v| < 2^53) and an
 // exponent add: a few issue slots instead of the integer formatting, for
 // callers that spread their values over both pipes.
 __device__ __forceinline__ double i64_ldexp_row_cvt(long long v, int e) {
