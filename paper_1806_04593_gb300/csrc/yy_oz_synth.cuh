@@ -333,8 +333,8 @@ k_oz_synth(const __grid_constant__ OzSynthMaps maps, const __grid_constant__ OzS
       const int cell = (2 * ct + rank) * kPairRows + quarter * 32 + lane;
       const bool cell_ok = cell < a.cells;
       const int ce = cell_ok ? J.cell_exp[cell] : 0;
-      // the whole warp's rows stay in the normal range (a sum may reach 2^54 with four classes)
-      const bool rows_ok = __all_sync(0xffffffffu, i64_ldexp_row_ok(NCLS == 4 ? ce + 1 : ce));
+      // the whole warp's rows stay in the normal range, a sum of 1 as well as one of four classes, up to 2^54
+      const bool rows_ok = __all_sync(0xffffffffu, i64_ldexp_row_ok(ce) && (NCLS == 2 || i64_ldexp_row_ok(ce + 1)));
       __syncwarp();   // the previous tile's row pointers are no longer read
       rowp[lane] = !cell_ok ? nullptr
                    : (cell < a.out_split) ? J.out0 + (size_t)cell * a.ldo

@@ -42,3 +42,30 @@ def test_odd_multiples_in_every_column(n_phi, lmax):
     place = last_places(v)
     odd = place == place.min(axis=1, keepdims=True)
     assert odd.any(axis=0).all(), np.nonzero(~odd.any(axis=0))[0]
+
+
+@pytest.mark.parametrize("lmax", [40, 63])
+def test_single_units_at_the_bottom_of_the_range(lmax):
+    """Rows whose unit is 2^-1023, below the normal range: a value of one unit stays one.
+
+    A density that alternates along its rows excites the sine of order 32, whose derivative
+    vanishes at the cells: g_phi is a few units there, of rounding alone (one row per shell, at
+    the equator, so that neighbouring rows have about the same unit).  Rows are written 32
+    at a time, by a quick form where all of them allow it.  The density is stepped by powers
+    of two, so that the smallest unit of each group passes 2^-1023; at that step, and at
+    those around it, some of these rows' values are a single unit."""
+    require_gpu()
+    yy = lib()
+    g = yy.Grid.from_spec(inputs.polar_grid(np.logspace(-1, 0, 481), 1, 64, lmax))
+    g.prepare("fp64_ozaki")
+    rho = (1.0 - 2.0 * (np.arange(64) % 2)) * (1.0 + np.random.default_rng(6).random((480, 1, 1)))
+    groups = lambda v: v[-480:].reshape(15, 32, 64)  # noqa: E731  (g_phi)
+    least = last_places(groups(rows(g, rho))).min(axis=(1, 2))
+    single = {at: 0 for at in range(-1025, -1020)}
+    for power in range(-1026 - int(least.max()), -1019 - int(least.min())):
+        v = groups(rows(g, np.ldexp(rho, power)))
+        for at in single:
+            single[at] += int((np.abs(v[least + power == at]) == 2.0 ** at).sum())
+    assert yy.yy_last_device_status(g.handle) == yy.YY_OK
+    g.close()
+    assert all(single[at] > 0 for at in single), single
