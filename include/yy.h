@@ -90,8 +90,9 @@ typedef enum {
  *             products by fused multiply-add and exact sums by TwoSum) on the
  *             CUDA cores' fp32 pipe, each input scaled by a power of two that
  *             follows the data; the radial scans are float64 as for YY_FP64
- *             (and so is the analysis with YY_ANALYSIS_DENSE, or with more
- *             than 640 cells per row).  Multiplying rho by a power of two
+ *             (and so is the analysis with YY_ANALYSIS_DENSE, with more
+ *             than 640 cells per row, or on grids too tall for both polar
+ *             stages: from 227 polar rows at l_max 63).  Multiplying rho by a power of two
  *             multiplies every result by the same power exactly.
  *             Needs yy_grid_prepare and 2 l_max + 1 <= 127 (l_max <= 63);
  *             above l_max 31 rows of G hold 128 slots and the analysis's

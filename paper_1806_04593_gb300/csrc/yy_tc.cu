@@ -3052,12 +3052,19 @@ static uint16_t bf16_int(int v) {
   return (uint16_t)(u >> 16);
 }
 
+// shared memory of k_sep_theta_ff; grids beyond its limit take the float64 polar stage
+static size_t sep_theta_ff_smem(const yy_grid *g) {
+  return (size_t)kSepFFShells * 2 * ((g->n_theta + 1) / 2) * g->sep_nt_pad * sizeof(float2);
+}
+static bool sep_theta_ff_fits(const yy_grid *g) { return sep_theta_ff_smem(g) <= 200 * 1024; }
+
 // Tables of the analysis by the Ozaki scheme; leaves an_ok = 0 (the float64
-// analysis serves) where the rows are longer than 640 cells.
+// analysis serves) where the rows are longer than 640 cells or neither polar stage fits.
 static yy_status ozaki_prepare_analysis(yy_grid *g, yy_oz_tables *o) {
   typedef FormOzaki F;
   const int nt = 2 * g->lmax + 1;
   if (g->n_phi > F::kMaxK || !g->sep_az || !g->sep_F) return YY_OK;
+  if (!sep_theta_ff_fits(g) && !(g->sep_ok & 2)) return YY_OK;
   // classes of 32 slots up to l_max 31, of 64 up to 63
   const int BN = g->lmax < 32 ? 32 : 64;
   const auto kernel = BN == 32 ? k_oz_analysis<32> : k_oz_analysis<64>;
@@ -3125,9 +3132,8 @@ static yy_status ozaki_prepare_analysis(yy_grid *g, yy_oz_tables *o) {
 
 // the polar stage of the analysis after the Ozaki azimuthal stage
 static cudaError_t ozaki_theta_analysis(yy_grid *g, cudaStream_t s) {
-  const int half = (g->n_theta + 1) / 2;
-  const size_t smem = (size_t)kSepFFShells * 2 * half * g->sep_nt_pad * sizeof(float2);
-  if (smem > 200 * 1024) return separable_theta_f64(g, s);
+  if (!sep_theta_ff_fits(g)) return separable_theta_f64(g, s);
+  const size_t smem = sep_theta_ff_smem(g);
   const int shells = grid_rows(g);
   return launch_kernel(g, "k_sep_theta_ff", k_sep_theta_ff, (unsigned)((shells + kSepFFShells - 1) / kSepFFShells),
                        sep_theta_ff_threads(g->n_lm), smem, s, shells, g->n_theta, g->n_lm, 2 * g->lmax + 1, g->sep_nt_pad,
