@@ -46,8 +46,16 @@ static void gauss_legendre01(int n, double *x, double *w) {
   }
 }
 
+// A call that fails takes its CUDA error with it: the runtime keeps the error of a
+// refused launch for the next cudaGetLastError, which may be another call's.
+static yy_status settled(yy_status st) {
+  if (st != YY_OK) cudaGetLastError();
+  return st;
+}
+
 static yy_status from_cuda(cudaError_t e) {
   if (e == cudaSuccess) return YY_OK;
+  cudaGetLastError();
   if (e == cudaErrorMemoryAllocation) return YY_ERR_OOM;
   return YY_ERR_CUDA;
 }
@@ -204,7 +212,6 @@ static yy_status create_grid(const double *r_edges, int n_r, int n_theta, int n_
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     const yy_status st = from_cuda(e);
-    cudaGetLastError();
     free_all(g);
     delete g;
     return st;
@@ -237,7 +244,7 @@ yy_status yy_grid_set_analysis(yy_grid *g, yy_analysis method) {
   g->analysis_method = (int)method;
   if (method == YY_ANALYSIS_SEPARABLE)   // the separable tensor-core tables of the prepared forms
     for (yy_precision p : {YY_TF32, YY_BF16X3, YY_FP16X2}) {
-      const yy_status st = tc_build_separable(g, p);
+      const yy_status st = settled(tc_build_separable(g, p));
       if (st != YY_OK) return st;
     }
   return YY_OK;
@@ -292,9 +299,9 @@ yy_status yy_grid_prepare(yy_grid *g, yy_precision prec) {
     }
     case YY_TF32:
     case YY_BF16X3:
-    case YY_FP16X2: return tc_prepare(g, prec);
+    case YY_FP16X2: return settled(tc_prepare(g, prec));
     case YY_FP64_OZAKI: {
-      const yy_status st = ozaki_prepare(g);
+      const yy_status st = settled(ozaki_prepare(g));
       return st == YY_OK ? from_cuda(cudaDeviceSynchronize()) : st;
     }
   }

@@ -62,6 +62,7 @@ namespace {
 
 yy_status to_status(cudaError_t e) {
   if (e == cudaSuccess) return YY_OK;
+  cudaGetLastError();   // the error goes with this call, not with the next one
   if (e == cudaErrorMemoryAllocation) return YY_ERR_OOM;
   return YY_ERR_CUDA;
 }
