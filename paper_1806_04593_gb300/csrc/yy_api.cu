@@ -106,6 +106,10 @@ extern "C" {
 
 void yy_debug_fail_alloc_after(int n) { g_fail_alloc_countdown = n; }
 
+int yy_debug_oz_trig_scale(const double *trig, int l_max, int columns) {
+  return trig == nullptr || l_max < 0 || l_max > 63 || columns < 1 ? -2 : oz_trig_scale(trig, l_max, columns);
+}
+
 const char *yy_status_string(yy_status s) {
   switch (s) {
     case YY_OK: return "ok";

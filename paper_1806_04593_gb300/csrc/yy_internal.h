@@ -349,6 +349,7 @@ cudaError_t tc_synthesis(yy_grid *g, yy_precision prec, double *phi_yin,
 // float64 synthesis with its azimuthal stage on the tensor cores by the Ozaki
 // scheme (yy_tc.cu): tables once (2 l_max + 1 <= 64), then per solve
 yy_status ozaki_prepare(yy_grid *g);
+int oz_trig_scale(const double *trig, int lmax, int columns);   // yy_debug_oz_trig_scale
 void ozaki_free(yy_grid *g);
 bool ozaki_ready(const yy_grid *g);
 // the separable analysis with its azimuthal stage by the same scheme (n_phi <= 640)

@@ -10,15 +10,16 @@
 //
 // Digits (FormOzSynth): x = sum_s a_s 2^(-10 (s + 1)), five balanced base-1024
 // digits |a_s| <= 512 (528 for one of G's), exact in fp16; rows of G scaled to |x| <= 1/2, the trig
-// table to |y| <= 1/4 (1/8 above l_max 31).  The products of digit levels L = s + t
+// table to |y| <= 1/4.  The products of digit levels L = s + t
 // <= 4 are kept, the dropped ones add up to below 2^-50 of the scales.  A class
 // (the cos or sin slots; above l_max 31 those of even and of odd m apart) has at
-// most 32 slots, so a level sum S_L of L <= 3 stays below 2^24 for the trig
-// tables in use (512 times the sum of up to four products' trig digits, checked
-// on the host for L <= 2 and close to it for L = 3) and accumulates exactly in
-// fp32.  Level 4 enters the accumulator of level 3 first, its trig digits scaled
+// most 32 slots, and a level sum S_L of L <= 2 stays below 2^24 (528 times the sum of
+// the trig digits, checked on the host) and accumulates exactly in fp32.  Level 4
+// enters the accumulator of level 3 first, its trig digits scaled
 // by 2^-10 (still exact in fp16): S_4 2^-10 is exact in fp32, and what the additions
-// of level 3 round off it is some 2^-3 of a level-3 unit.  So four
+// of level 3 round off it is some 2^-3 of a level-3 unit.  Level 3 itself is not
+// checked: were all of its products of one sign and every digit of G at its largest, it
+// could reach 1.15 2^24, where an addition rounds to 2 units.  So four
 // accumulators hold a class, and
 //   V = S_0 2^30 + S_1 2^20 + S_2 2^10 + round(S_3 + S_4 2^-10)
 // is the class's sum in level-3 units, 2^-50 of the two rows' scales.  V_C + V_S

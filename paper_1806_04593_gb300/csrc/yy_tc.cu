@@ -3217,37 +3217,56 @@ static uint16_t half_bits(float v) {
   return u;
 }
 
+// The columns of the synthesis that trig digits are written for (ozaki_prepare).
+struct OzTrigColumns {
+  int lmax, n_phi, first, half, shift;   // columns: shift, then half folded ones
+  int rows_pad, gk;                      // rows of a slice, slots of a row
+};
+
 // Trig digit slices (FormOzSynth): digits 0..3 of y = trig 2^-qt, then digits
 // 0..4 scaled by 2^-10, rows = columns of the fold, slots by class.  False: a
 // level sum of levels 0..2 could reach 2^24 at some column (|G digit| <= 528).
 template <int NG>
-static bool oz_trig_digits(const yy_grid *g, const yy_oz_tables *o, const std::vector<double> &tr, int qt,
-                           std::vector<uint16_t> &sl) {
+static bool oz_trig_digits(const OzTrigColumns &o, const double *tr, int qt, std::vector<uint16_t> &sl) {
   typedef FormOzSynth F;
   std::fill(sl.begin(), sl.end(), (uint16_t)0);
   bool exact = true;
-  for (int c = 0; c < o->fold.half + o->shift; ++c) {
+  for (int c = 0; c < o.half + o.shift; ++c) {
     // a column before the first repeats that one's mirror cell
-    const bool mirror = c < o->shift;
-    const int k = o->fold.first + (mirror ? 0 : c - o->shift);
+    const bool mirror = c < o.shift;
+    const int k = o.first + (mirror ? 0 : c - o.shift);
     long long asum[4][3] = {};   // per class, of the three top digits
-    for (int m = 0; m <= g->lmax; ++m)
+    for (int m = 0; m <= o.lmax; ++m)
       for (int sine = 0; sine < (m > 0 ? 2 : 1); ++sine) {
         const int t = oz_slot<NG>(m, sine);
-        const double x = tr[(size_t)(m == 0 ? 0 : 2 * m - 1 + sine) * g->n_phi + k];
+        const double x = tr[(size_t)(m == 0 ? 0 : 2 * m - 1 + sine) * o.n_phi + k];
         const double y = ldexp(mirror && sine ? -x : x, -qt);
         int d[5];
         oz_digits1024((unsigned long long)floor(ldexp(fabs(y), 50) + 0.5), d);
         for (int s = 0; s < 5; ++s) {
           const float v = (float)(y < 0 ? -d[s] : d[s]);
-          if (s < F::kTrigScaled) sl[((size_t)s * o->b_rows_pad + c) * o->gk + t] = half_bits(v);
-          sl[((size_t)(F::kTrigScaled + s) * o->b_rows_pad + c) * o->gk + t] = half_bits(ldexpf(v, -10));
+          if (s < F::kTrigScaled) sl[((size_t)s * o.rows_pad + c) * o.gk + t] = half_bits(v);
+          sl[((size_t)(F::kTrigScaled + s) * o.rows_pad + c) * o.gk + t] = half_bits(ldexpf(v, -10));
           if (s < 3) asum[t / F::kClassSlots][s] += abs(d[s]);
         }
       }
     for (auto &u : asum) exact = exact && 528 * (u[0] + u[1] + u[2]) < (1ll << 24);
   }
   return exact;
+}
+
+// The digits of trig / 4, or of a smaller scale, whose digits are others, where a
+// column's sums come out too large (on no grid of up to 639 cells).  The power of
+// the scale, -1 where none of three is exact.
+static int oz_trig_scale(const OzTrigColumns &o, const double *tr, std::vector<uint16_t> &sl) {
+  for (int q = 2; q <= 4; ++q)
+    if (o.gk == 64 ? oz_trig_digits<1>(o, tr, q, sl) : oz_trig_digits<2>(o, tr, q, sl)) return q;
+  return -1;
+}
+int oz_trig_scale(const double *tr, int lmax, int columns) {
+  const OzTrigColumns o = {lmax, columns, 0, columns, 0, columns, lmax <= 31 ? 64 : 128};
+  std::vector<uint16_t> sl((size_t)FormOzSynth::kTrig * o.rows_pad * o.gk);
+  return oz_trig_scale(o, tr, sl);
 }
 
 yy_status ozaki_prepare(yy_grid *g) {
@@ -3331,15 +3350,15 @@ yy_status ozaki_prepare(yy_grid *g) {
     if (e != cudaSuccess) st = e == cudaErrorMemoryAllocation ? YY_ERR_OOM : YY_ERR_CUDA;
   }
   if (st == YY_OK) {
-    // trig digits on the host, of trig / 4; a smaller scale has other digits,
-    // should a column's sums come out too large
+    // trig digits on the host
     std::vector<double> tr((size_t)nt * g->n_phi);
     std::vector<uint16_t> sl(t_elems);
     if (cudaMemcpy(tr.data(), g->sep_tr, tr.size() * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
       st = YY_ERR_CUDA;
-    const int q0 = 2;
-    auto digits = [&](int q) { return o->gk == 64 ? oz_trig_digits<1>(g, o, tr, q, sl) : oz_trig_digits<2>(g, o, tr, q, sl); };
-    for (o->qt = q0; st == YY_OK && !digits(o->qt) && o->qt < q0 + 2;) ++o->qt;
+    if (st == YY_OK) {
+      o->qt = oz_trig_scale({g->lmax, g->n_phi, o->fold.first, o->fold.half, o->shift, o->b_rows_pad, o->gk}, tr.data(), sl);
+      if (o->qt < 0) st = YY_ERR_NOT_SUPPORTED;
+    }
     if (st == YY_OK && cudaMemcpy(o->trig, sl.data(), t_elems * F::kElem, cudaMemcpyHostToDevice) != cudaSuccess)
       st = YY_ERR_CUDA;
   }

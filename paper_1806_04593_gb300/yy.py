@@ -111,6 +111,8 @@ def load():
     lib.yy_grid_kernel_ms.restype = I
     lib.yy_debug_fail_alloc_after.argtypes = [I]
     lib.yy_debug_fail_alloc_after.restype = None
+    lib.yy_debug_oz_trig_scale.argtypes = [P, I, I]
+    lib.yy_debug_oz_trig_scale.restype = I
     lib.yy_batch_create.argtypes = [P, I, ctypes.POINTER(P)]
     lib.yy_batch_create.restype = I
     lib.yy_batch_prepare.argtypes = [P, I]
@@ -297,6 +299,11 @@ def yy_grid_kernels_ms(handle):
 
 def yy_debug_fail_alloc_after(n):
     load().yy_debug_fail_alloc_after(int(n))
+
+
+def yy_debug_oz_trig_scale(trig):
+    t = np.ascontiguousarray(trig, dtype=np.float64)
+    return load().yy_debug_oz_trig_scale(_ptr(t), (t.shape[0] - 1) // 2, t.shape[1])
 
 
 class FieldDesc(ctypes.Structure):
