@@ -244,15 +244,27 @@ cudaError_t synthesis_simt(yy_grid *g, double *phi_yin, double *phi_yang, double
 cudaError_t convert_tables_f32(yy_grid *g) {
   const size_t n_ban = (size_t)g->n_lm * g->n_ang;
   const size_t n_syn = (size_t)g->n_ang * g->n_lm;
-  cudaError_t err;
-  if ((err = dmalloc((void **)&g->ban32, n_ban * sizeof(float))) != cudaSuccess) return err;
-  if ((err = dmalloc((void **)&g->ysyn32, n_syn * sizeof(float))) != cudaSuccess) return err;
-  if ((err = dmalloc((void **)&g->ysyn_t32, n_syn * sizeof(float))) != cudaSuccess) return err;
-  if ((err = dmalloc((void **)&g->ysyn_p32, n_syn * sizeof(float))) != cudaSuccess) return err;
-  if ((err = dmalloc((void **)&g->rho32, (size_t)grid_rows(g) * g->n_ang * sizeof(float))) != cudaSuccess)
+  // all of them or none: a solve takes ban32 for the others (Q32 may be there for another form)
+  struct {
+    float **p;
+    size_t n;
+  } const bufs[] = {{&g->ban32, n_ban}, {&g->ysyn32, n_syn}, {&g->ysyn_t32, n_syn}, {&g->ysyn_p32, n_syn},
+                    {&g->rho32, (size_t)grid_rows(g) * g->n_ang}, {&g->Q32, 3 * (size_t)grid_rows(g) * g->n_lm}};
+  float **made[6] = {};
+  int n_made = 0;
+  for (const auto &b : bufs) {
+    if (*b.p) continue;
+    const cudaError_t err = dmalloc((void **)b.p, b.n * sizeof(float));
+    if (err == cudaSuccess) {
+      made[n_made++] = b.p;
+      continue;
+    }
+    while (n_made > 0) {
+      cudaFree(*made[--n_made]);
+      *made[n_made] = nullptr;
+    }
     return err;
-  if ((err = dmalloc((void **)&g->Q32, 3 * (size_t)grid_rows(g) * g->n_lm * sizeof(float))) != cudaSuccess)
-    return err;
+  }
   k_to_f32<<<(unsigned)((n_ban + 255) / 256), 256>>>(n_ban, g->ban, g->ban32);
   k_to_f32<<<(unsigned)((n_syn + 255) / 256), 256>>>(n_syn, g->ysyn, g->ysyn32);
   k_to_f32<<<(unsigned)((n_syn + 255) / 256), 256>>>(n_syn, g->ysyn_t, g->ysyn_t32);
