@@ -647,6 +647,7 @@ cudaError_t synthesis_separable_prepare(yy_grid *g) {
 }
 
 cudaError_t synthesis_separable_prepare_f32(yy_grid *g) {
+  if (!(g->sep_syn_ok & 1)) return cudaSuccess;   // the dense contraction serves
   const size_t n_p = (size_t)g->n_theta * g->n_lm, rows = (size_t)grid_rows(g) * g->n_theta;
   const float *src[3] = {g->sep_P32, g->sep_dP32, g->sep_Qs32};
   cudaError_t e = cudaSuccess;
