@@ -332,12 +332,32 @@ def cpu_baseline(spec, ry, rg, gradient):
 # algorithmic work per kernel (roofline)
 # ---------------------------------------------------------------------------
 
+def fold_columns(spec):
+    """(columns, quarter): the columns of the float64 stages' azimuthal folds, and whether
+    they fold at pi / 2 -+ phi too (at pi - phi alone, or at -phi alone, otherwise)."""
+    half = (spec.n_phi + 1) // 2
+    cells = spec.n_phi / 2 if spec.polar else math.pi / ((1.5 * math.pi + 2 * spec.delta_phi) / spec.n_phi)
+    whole = round(cells) if abs(cells - round(cells)) < 1e-12 * cells else 0   # cells to pi, where a whole number
+    odd = 1 if spec.polar or spec.n_phi % 2 == 0 else 0                        # centres at half cells from the axis
+    if whole and whole % 2 == 0:
+        q = whole // 2
+        return min(half, (q + 1) // 2 if odd else q // 2 + 1), True
+    return min(half, (whole - odd) // 2 + 1 if whole else half), False
+
+
+def fold_products(spec, zeroth):
+    """Multiply-adds of one row over its folded columns: one per slot, two per slot of an
+    odd order with the quarter fold; zeroth: those of slot 0."""
+    cols, quarter = fold_columns(spec)
+    return cols * (zeroth + 2 * (spec.lmax // 2) + (4 if quarter else 2) * ((spec.lmax + 1) // 2))
+
+
 def kernel_work(name, spec, n_lm, gradient, prec):
     """Algorithmic work of one launch of a named kernel of the solve:
     {"flop": ..., "flop_kind": "tensor"|"fp64"|"fp32", "bytes": ...} (the
     entries that apply), each counted from the sizes of the workload."""
     L = spec.lmax
-    n_r2 = 2 * spec.n_r                       # rows of both patches
+    n_r2 = (1 if spec.polar else 2) * spec.n_r   # rows of all patches
     J = 4 if gradient else 1                  # Phi and the three gradient components
     nt = 2 * L + 1
     half = (spec.n_theta + 1) // 2
@@ -387,19 +407,17 @@ def kernel_work(name, spec, n_lm, gradient, prec):
         w = {"bytes": n_r2 * spec.n_ang * f64 + n_r2 * spec.n_ang * {"fp16x2": 4, "bf16x3": 6, "tf32": 4}.get(prec, 4)}
     elif name in ("k_synth_f64", "k_phi32", "k_theta32", "k_sep_phi64", "k_sep_phi32"):
         # separable sums; the float64 kernels run them over the cells folded by
-        # their symmetries: the operations of the folded sums
+        # their symmetries: the multiply-adds of the folded sums (their additions apart)
         kind = "fp64" if name.endswith("64") else "fp32"
-        cols = spec.n_phi
-        if kind == "fp64":
-            whole = math.pi / ((1.5 * math.pi + 2 * spec.delta_phi) / spec.n_phi)
-            cols = spec.n_phi / 3 if abs(whole - round(whole)) < 1e-9 else spec.n_phi / 2
+        # multiply-adds per row: the float64 synthesis adds slot 0 without one
+        per_row = fold_products(spec, 0 if name == "k_synth_f64" else 1) if kind == "fp64" else spec.n_phi * nt
         if name.startswith("k_sep_phi"):
-            w = {"flop": 2.0 * rows * cols * nt, "bytes": n_r2 * spec.n_ang * f64}
+            w = {"flop": 2.0 * rows * per_row, "bytes": n_r2 * spec.n_ang * f64}
         elif name == "k_theta32":
             w = {"flop": J * 2.0 * rows * n_lm, "bytes": J * rows * nt * 4}
         else:
             theta = 0.0 if name == "k_phi32" else min(J, 3) * 2.0 * n_r2 * half * n_lm
-            w = {"flop": theta + J * 2.0 * rows * cols * nt, "bytes": out_bytes}
+            w = {"flop": theta + J * 2.0 * rows * per_row, "bytes": out_bytes}
         w["flop_kind"] = kind
     return w
 
