@@ -403,7 +403,7 @@ def kernel_work(name, spec, n_lm, gradient, prec):
              "bytes": out_bytes}
     elif name == "k_tc_pair/split-K":
         w = {"flop": 2.0 * n_r2 * n_lm * spec.n_ang, "flop_kind": "tensor", "products": prec}
-    elif name == "k_pack_stream":
+    elif name in ("k_pack_stream", "k_pack_reg/densities"):
         w = {"bytes": n_r2 * spec.n_ang * f64 + n_r2 * spec.n_ang * {"fp16x2": 4, "bf16x3": 6, "tf32": 4}.get(prec, 4)}
     elif name in ("k_synth_f64", "k_phi32", "k_theta32", "k_sep_phi64", "k_sep_phi32"):
         # separable sums; the float64 kernels run them over the cells folded by

@@ -1224,13 +1224,13 @@ static cudaError_t launch_pack(yy_grid *g, const char *name, PackBatch &b, int n
 // (16-byte aligned rows of an even length, nothing left out), else
 // launch_pack.
 template <class F>
-static cudaError_t launch_pack_long(yy_grid *g, const char *name, PackBatch &b, cudaStream_t s) {
+static cudaError_t launch_pack_long(yy_grid *g, PackBatch &b, cudaStream_t s) {
   const PackArgs &p = b.job[0];
   const bool fits = ((uintptr_t)p.src0 % 16) == 0 && ((uintptr_t)p.src1 % 16) == 0 && (p.ld % 2) == 0 &&
                     (p.K % 2) == 0 && p.wrow == nullptr && p.row_add == nullptr && p.zero_k0 < 0 &&
                     p.zero_k1 < 0 && p.zero_row < 0 && (p.dot_vec == nullptr || (uintptr_t)p.dot_vec % 8 == 0);
-  if (!fits || p.K <= 32 * 64 || p.K > kStreamMaxK || p.k_pad > kStreamMaxK) return launch_pack<F>(g, name, b, 1, s);
-  return launch_kernel(g, name, k_pack_stream<F>, std::min(p.rows_pad, g->sms), 1024, (size_t)p.K * sizeof(double), s, p, g->err);
+  if (!fits || p.K <= 32 * 64 || p.K > kStreamMaxK || p.k_pad > kStreamMaxK) return launch_pack<F>(g, "k_pack_reg/densities", b, 1, s);
+  return launch_kernel(g, "k_pack_stream", k_pack_stream<F>, std::min(p.rows_pad, g->sms), 1024, (size_t)p.K * sizeof(double), s, p, g->err);
 }
 
 // attr: two entries; overlap: the launch may overlap the end of the kernel before it
@@ -1695,7 +1695,7 @@ static cudaError_t analysis_form(yy_grid *g, yy_tc_tables *t, const double *ry, 
   PackBatch b = {};
   PairArgs a;
   analysis_args<F>(g, t, ry, rg, b.job[0], a);
-  cudaError_t e = launch_pack_long<F>(g, "k_pack_stream", b, s);
+  cudaError_t e = launch_pack_long<F>(g, b, s);
   if (e != cudaSuccess) return e;
   if ((e = launch_pair<F>(g, t, t->an_maps, a, s)) != cudaSuccess) return e;
   if (g->n_patch == 2 && g->lmax <= kReduceRotateLmax) {
