@@ -203,7 +203,9 @@ k_rotate_moments(int n_r, int n_lm, const T *__restrict__ rot, const double *__r
 }
 
 // Radial scans with one thread per (patch, mode, chunk of radii): 32 chunks of
-// ch = ceil(n_r / 32) <= CH radii, held in registers.  Each recurrence is folded
+// ch = ceil(n_r / 32) <= CH radii, held in registers (with three blocks per SM the form of
+// 24 radii, and the grouped kernel, which has every form, spill some 60 values each to local memory;
+// 577 to 768 zones at l_max 25 take 37 to 41 us so, 47 to 55 with a warp per mode).  Each recurrence is folded
 // into one affine map per chunk, the maps are composed across the chunks in
 // shared memory (prefix for the inner sums, suffix for the outer ones, both in
 // the same five steps), and each thread then replays its radii from the composed

@@ -594,7 +594,7 @@ k_tc_pair(const __grid_constant__ PairMaps maps0, const __grid_constant__ PairAr
            t += n_pairs) {
         const PairArgs &a = GROUPED ? a0.group[f_] : a0;
         const int per_job = a.cell_tiles * a.row_tiles * a.k_splits;
-        // K blocks per accumulator fill (modes 0 and 3 add the fills in the epilogue)
+        // K blocks per accumulator fill (mode 0 adds the fills in the epilogue)
         const int chunk = (OUT_MODE == 0 && a.kb_chunk > 0) ? a.kb_chunk : a.kb_total;
         const uint32_t idesc = instr_desc_pair<F>(a.bn);
         const int tl = t % per_job;
@@ -664,7 +664,7 @@ k_tc_pair(const __grid_constant__ PairMaps maps0, const __grid_constant__ PairAr
       for (int f_ = 0, base_ = 0, t = pair; pair_tile_next<GROUPED>(a0, pair, n_pairs, f_, base_, t); t += n_pairs) {
         const PairArgs &a = GROUPED ? a0.group[f_] : a0;
         const int per_job = a.cell_tiles * a.row_tiles * a.k_splits;
-        // K blocks per accumulator fill (modes 0 and 3 add the fills in the epilogue)
+        // K blocks per accumulator fill (mode 0 adds the fills in the epilogue)
         const int chunk = (OUT_MODE == 0 && a.kb_chunk > 0) ? a.kb_chunk : a.kb_total;
         const int n_chunks = a.bn / kEpiCols;
         const int tl = t % per_job;
