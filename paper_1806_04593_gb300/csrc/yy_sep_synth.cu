@@ -499,9 +499,19 @@ __global__ void k_transpose_f32(int n_theta, int n_lm, const float *__restrict__
   if (e < (size_t)n_theta * n_lm) dst[e] = src[(e % n_theta) * n_lm + e / n_theta];
 }
 
-__global__ void k_fold_trig(int nt, int n_phi, AzFold f, const double *__restrict__ tr, double *__restrict__ out) {
+// 1, cos, sin at the folded columns
+__global__ void k_fold_trig(int m1, AzFold f, double dph, double dph_low, double *__restrict__ out) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < nt * f.cols) out[e] = tr[(size_t)(e / f.cols) * n_phi + f.first + e % f.cols];
+  if (e >= m1 * f.cols) return;
+  const int m = e / f.cols, c = e % f.cols;
+  double sn, cs;
+  fold_sincos(f, dph, dph_low, c, m, &sn, &cs);
+  if (m == 0) {
+    out[c] = 1.0;
+  } else {
+    out[(size_t)(2 * m - 1) * f.cols + c] = cs;
+    out[(size_t)(2 * m) * f.cols + c] = sn;
+  }
 }
 
 __global__ void k_inv_sin(int n_theta, double th0, double dth, double *__restrict__ isin) {
@@ -621,13 +631,24 @@ AzFold az_fold(const yy_grid *g) {
   return f;
 }
 
+// The cell width is (3 pi / 2 + 2 delta_phi) / n_phi (2 pi / n_phi on the polar grid), with pi
+// beyond its double: pi / 4 is kQ + kQLow to 107 bits.
+double fold_dph_low(const yy_grid *g) {
+  const double kQ = 0.78539816339744830962, kQLow = 3.0616169978683829431e-17;
+  const double n = g->n_phi, quarters = g->n_patch == 1 ? 8.0 : 6.0, d = 2.0 * g->delta_phi;
+  const double range = quarters * kQ, low = fma(quarters, kQ, -range) + quarters * kQLow;
+  const double sum = range + d, b = sum - range, err = (range - (sum - b)) + (d - b);   // exact: sum + err
+  return (fma(-g->dph, n, sum) + (err + low)) / n;
+}
+
 cudaError_t synthesis_separable_prepare(yy_grid *g) {
   const int nt = 2 * g->lmax + 1;
   const AzFold f = az_fold(g);
   cudaError_t e = dmalloc((void **)&g->sep_trf, (size_t)nt * f.cols * sizeof(double));
   if (e == cudaSuccess) e = dmalloc((void **)&g->sep_isin, (size_t)g->n_theta * sizeof(double));
   if (e != cudaSuccess) return e;
-  k_fold_trig<<<(nt * f.cols + 255) / 256, 256>>>(nt, g->n_phi, f, g->sep_tr, g->sep_trf);
+  const int m1 = g->lmax + 1;
+  k_fold_trig<<<(m1 * f.cols + 255) / 256, 256>>>(m1, f, g->dph, fold_dph_low(g), g->sep_trf);
   k_inv_sin<<<(g->n_theta + 255) / 256, 256>>>(g->n_theta, g->th0, g->dth, g->sep_isin);
   for (auto k : {(const void *)k_synth_f64<1, false>, (const void *)k_synth_f64<4, false>, (const void *)k_synth_f64<1, true>,
                  (const void *)k_synth_f64<4, true>, (const void *)k_theta32<1>, (const void *)k_theta32<4>,

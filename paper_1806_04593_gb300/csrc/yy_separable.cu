@@ -255,12 +255,14 @@ __global__ void k_sep_phi64(const SepPhi64 a) {
 }
 
 // az[column][m] = the cell integrals of cos and sin (m phi) at the folded columns
-__global__ void k_fold_az(int m1, int nt_pad, AzFold f, const double *__restrict__ az, double2 *__restrict__ out) {
+__global__ void k_fold_az(int m1, AzFold f, double dph, double dph_low, double2 *__restrict__ out) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= m1 * f.cols) return;
   const int c = e / m1, m = e % m1;
-  const double *row = az + (size_t)(f.first + c) * nt_pad;
-  out[e] = m == 0 ? make_double2(row[0], 0.0) : make_double2(row[2 * m - 1], row[2 * m]);
+  double sn, cs;
+  fold_sincos(f, dph, dph_low, c, m, &sn, &cs);
+  const double width = m == 0 ? dph : 2.0 * sin(0.5 * m * dph) / m;
+  out[e] = make_double2(cs * width, sn * width);
 }
 
 // Azimuthal stage, fp32: every F is one chain of fp32 multiply-adds over k in
@@ -668,7 +670,7 @@ cudaError_t separable_prepare(yy_grid *g) {
   const int m1 = g->lmax + 1;
   A((void **)&g->sep_azf, (size_t)m1 * fold.cols * sizeof(double2));
   if (e != cudaSuccess) return e;
-  k_fold_az<<<(m1 * fold.cols + 255) / 256, 256>>>(m1, nt_pad, fold, g->sep_az, (double2 *)g->sep_azf);
+  k_fold_az<<<(m1 * fold.cols + 255) / 256, 256>>>(m1, fold, g->dph, fold_dph_low(g), (double2 *)g->sep_azf);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // float64: the polar stage's sums and the folded rows in shared memory.
   // fp32: grids whose table and 16 padded rows of a shell fit 227 KB; the others
